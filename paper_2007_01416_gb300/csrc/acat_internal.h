@@ -3,6 +3,8 @@
 
 #include <cstdint>
 
+#include <vector_types.h>
+
 #define ACAT_MAXP 4
 #define ACAT_MAXN 8
 
@@ -24,6 +26,18 @@ struct AcatTables {
   float ghf[ACAT_MAXP + 1][ACAT_MAXN];
   float taylorf[ACAT_MAXP + 1][ACAT_MAXN][ACAT_MAXN];
   float invfactf[ACAT_MAXN + 1];
+  // the weights as integers over one common denominator per p (exact in
+  // float), for the float-float recursion: g1 x LC, gamma^{k,0} / k! x LQ
+  // ([p][k][r]), gh x LH; r^l ([p][r][l]); 840 / k; 1 / (k LC) and 1 / LQ
+  float g1i[ACAT_MAXP + 1][ACAT_MAXN][ACAT_MAXN];
+  float lag[ACAT_MAXP + 1][ACAT_MAXN][ACAT_MAXN];
+  float ghi[ACAT_MAXP + 1][ACAT_MAXN];
+  float powr[ACAT_MAXP + 1][ACAT_MAXN][ACAT_MAXN];
+  float k840[ACAT_MAXN + 1];
+  double ilc[ACAT_MAXP + 1][ACAT_MAXN];
+  struct {
+    float x, y;
+  } ilq[ACAT_MAXP + 1];
 };
 
 void acat_build_tables(AcatTables *T);
@@ -49,6 +63,8 @@ struct Step1DArgs {
   float epsf, rf;             // float eps and thr / (1 - thr) of the filtered decision
   float factf[ACAT_MAXP + 1];
   float advf, gammaf, gm1f;   // adv, gamma, gamma - 1 rounded to float (FP32 path)
+  // gamma, kappa = (gamma - 1) / 2, 1 - kappa and gamma - 1 as float pairs
+  float2 sgam, skap, somk, sgm1;
   unsigned long long *smax;   // 3 slots: max wave speed as ordered double bits
   double *tslot;              // 3 slots: simulated time (nullable)
   int8_t *orders;             // N+1 order codes (nullable)
@@ -58,6 +74,22 @@ struct Step1DArgs {
   int *cnt;                   // one hand-off counter per CTA boundary (both nullable: the
                               // fused 8-warp step kernel runs instead of the small-CTA one)
 };
+
+// A double as a pair of floats, and the pairs of a step's arguments (host).
+inline float2 acat_pair(double x) {
+  float2 r;
+  r.x = (float)x;
+  r.y = (float)(x - (double)r.x);
+  return r;
+}
+template <class Args>
+inline void acat_set_pairs(Args &a) {
+  const double kappa = 0.5 * (a.gamma - 1.0);
+  a.sgam = acat_pair(a.gamma);
+  a.skap = acat_pair(kappa);
+  a.somk = acat_pair(1.0 - kappa);
+  a.sgm1 = acat_pair(a.gamma - 1.0);
+}
 
 // Work description of a batch of independent 1D instances (ragged sizes),
 // concatenated along the cell index: u[c][M] with instance b at cells

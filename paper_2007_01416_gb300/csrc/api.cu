@@ -134,6 +134,7 @@ Step1DArgs base_args(acat_ctx *c) {
   a.advf = (float)p.adv[0];
   a.gammaf = (float)p.gamma;
   a.gm1f = (float)(p.gamma - 1.0);
+  acat_set_pairs(a);
   a.smax = c->d_smax;
   a.status = c->d_status;
   // the small-CTA step: FP64 whenever its buffers exist, FP32 when chosen

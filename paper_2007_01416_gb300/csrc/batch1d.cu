@@ -58,9 +58,9 @@ __global__ void __launch_bounds__(NT) k_batch_dt(const Step1DArgs a, const Batch
 // rounds (two at 16 warps, within 48 KB of static shared memory) make tiles
 // of R NW GPW interfaces, so the tile's CTA barriers, order-decision pass and
 // update phase are shared by R times the flux work.
-template <int NW>
-struct RoundsB32 {
-  static constexpr int value = NW >= 16 ? 2 : 8;
+template <bool F32, int NW>
+struct Rounds {
+  static constexpr int value = F32 ? (NW >= 16 ? 2 : 8) : (NW >= 16 ? 1 : NW == 8 ? 2 : 4);
 };
 
 // Persistent batched step: CTAs of NW warps take the tiles of the (instance,
@@ -77,9 +77,9 @@ struct RoundsB32 {
 template <int P, int FLUX, bool F32, int NW, int LPN>
 __global__ void __launch_bounds__(NW * 32, MinCtas<P, F32>::value * 8 / NW)
     k_batch1d(const Step1DArgs a, const BatchArgs bt) {
-  constexpr int R = F32 ? RoundsB32<NW>::value : 1;
+  constexpr int R = Rounds<F32, NW>::value;
   using SM =
-      typename std::conditional<F32, Smem32<P, Phys<FLUX>::S, NW, LPN, R>, Smem64<P, Phys<FLUX>::S, NW>>::type;
+      typename std::conditional<F32, Smem32<P, Phys<FLUX>::S, NW, LPN, R>, Smem64<P, FLUX, NW, R>>::type;
   // FP32: two workspaces used alternately (tile_f32 ends without a barrier)
   __shared__ SM sm[F32 ? 2 : 1];
   // the next tile of this CTA, claimed by thread 0 before the current one and
@@ -98,7 +98,7 @@ __global__ void __launch_bounds__(NW * 32, MinCtas<P, F32>::value * 8 / NW)
       tile_f32<P, FLUX, NW, LPN, R>(a, sm[par], static_cast<const float *>(a.u_in),
                                     static_cast<float *>(a.u_out), off, bt.M, N, i0, &bt.lamf[b], ord, so);
     } else {
-      tile_f64<P, FLUX, NW>(a, sm[0], static_cast<const double *>(a.u_in), static_cast<double *>(a.u_out),
+      tile_f64<P, FLUX, NW, R>(a, sm[0], static_cast<const double *>(a.u_in), static_cast<double *>(a.u_out),
                             off, bt.M, N, i0, bt.lam[b], ord, so);
     }
     w = (long)s_next[par];
@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(NW * 32, MinCtas<P, F32>::value * 8 / NW)
 template <int FLUX, bool F32>
 __global__ void __launch_bounds__(NT) k_smax_batch(const Step1DArgs a, const BatchArgs bt) {
   constexpr int S = Phys<FLUX>::S;
-  __shared__ double red[NT / 32];
+  __shared__ unsigned long long red[NT / 32];
   for (long b = blockIdx.x; b < bt.B; b += gridDim.x) {
     const long off = bt.offs[b], N = bt.offs[b + 1] - off;
     double smax = 0.0;
@@ -241,7 +241,7 @@ int acat_batch_occupancy(int P, int flux, int prec, int nw, int lpn) {
 namespace {
 template <int NW, int LPN, bool F32>
 int cells_per_tile(int P) {
-  constexpr int R = F32 ? RoundsB32<NW>::value : 1;
+  constexpr int R = Rounds<F32, NW>::value;
   switch (P) {
   case 1: return Tiling<1, NW, LPN, R>::T;
   case 2: return Tiling<2, NW, LPN, R>::T;

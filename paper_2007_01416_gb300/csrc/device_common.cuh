@@ -413,6 +413,21 @@ __device__ __forceinline__ unsigned reject_set64(const double *q, int st, bool f
   return reject_set<PM>(d, e, [=](int j) { return q[j * st]; }, first, F, eps, thr, fact, psi2_mod);
 }
 
+// The same with the first differences of the component's cells already
+// rounded to float, d_j = u_{j+1} - u_j at du[j] (consecutive cells).
+template <int PM>
+__device__ __forceinline__ unsigned reject_set64d(const float *du, const double *q, bool first,
+                                                  const FiltConst &F, double eps, double thr, const double *fact,
+                                                  int psi2_mod) {
+  float d[2 * PM - 1], e[2 * PM - 1];
+#pragma unroll
+  for (int k = 0; k < 2 * PM - 1; k++) {
+    d[k] = du[k - PM + 1];
+    e[k] = 6.0e-8f * fabsf(d[k]) + 1e-44f;
+  }
+  return reject_set<PM>(d, e, [=](int j) { return q[j]; }, first, F, eps, thr, fact, psi2_mod);
+}
+
 // The same for a compensated float state hi + lo (the literal fallback reads
 // the exact value hi + lo).
 template <int PM>
@@ -602,6 +617,15 @@ __device__ __forceinline__ double psi1_pair(const float *hi, const float *lo, in
   return psi1_g<S>(
       [=](int c, int k) { return (double)hi[c * cs + k * st] + (double)lo[c * cs + k * st]; }, kind,
       limiter_form, adv);
+}
+
+// Maximum over the warp of non-negative doubles (NaN excluded), by the integer
+// order of their bits: two 32-bit reductions, off the FP64 pipe.
+__device__ __forceinline__ double warp_max_pos(double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  const unsigned hi = (unsigned)(b >> 32), m = __reduce_max_sync(0xffffffffu, hi);
+  const unsigned lo = __reduce_max_sync(0xffffffffu, hi == m ? (unsigned)b : 0u);
+  return __longlong_as_double((long long)(((unsigned long long)m << 32) | lo));
 }
 
 __device__ __forceinline__ void atomic_max_pos(unsigned long long *addr, double v) {

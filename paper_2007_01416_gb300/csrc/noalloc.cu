@@ -114,6 +114,7 @@ extern "C" int acat_run_noalloc(const acat_params *p, void *u_dev, int nsteps, d
   a.advf = (float)p->adv[0];
   a.gammaf = (float)p->gamma;
   a.gm1f = (float)(p->gamma - 1.0);
+  acat_set_pairs(a);
   a.smax = smax;
   a.tslot = tslot;
   a.status = status;

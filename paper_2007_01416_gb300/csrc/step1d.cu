@@ -45,7 +45,7 @@ namespace {
 template <int P, int FLUX>
 __global__ void __launch_bounds__(NT, MinCtas<P, false>::value) k_step1d_f64(const Step1DArgs a) {
   acat_pdl_wait();
-  __shared__ Smem64<P, Phys<FLUX>::S> sm;
+  __shared__ Smem64<P, FLUX> sm;
   __shared__ double s_lam;
   if (threadIdx.x == 0) s_lam = step_dt(a) / a.dx;
   __syncthreads();
@@ -86,52 +86,32 @@ __global__ void __launch_bounds__(NWF * 32, 16 / NWF) k_step1d_fine(const Step1D
   using TL = Tiling<P, NWF>;
   constexpr int S = Phys<FLUX>::S;
   constexpr int NTF = NWF * 32;
-  __shared__ double tile[S][TL::TW];
-  __shared__ double Fs[TL::NI][S];
-  __shared__ double red[NWF];
+  __shared__ Smem64<P, FLUX, NWF> sm;
   __shared__ double s_lam;
   __shared__ int s_own[2];
+  auto &Fs = sm.Fs;
   const long N = a.N, i0 = (long)blockIdx.x * TL::NI;
   const double *__restrict__ uin = static_cast<const double *>(a.u_in);
   double *__restrict__ uout = static_cast<double *>(a.u_out);
   if (threadIdx.x == 0) s_lam = step_dt(a) / a.dx;
-  for (int q = threadIdx.x; q < S * TL::TW; q += NTF) {
-    const int c = q / TL::TW, k = q - c * TL::TW;
-    tile[c][k] = uin[c * N + bc_index(i0 - TL::GH + k, N, a.bc)];
-  }
   __syncthreads();
-  const double lam = s_lam, gm1 = a.gamma - 1.0;
+  const double lam = s_lam;
+  stage_f64<P, FLUX, NWF, 1>(a, sm, uin, 0, N, N, i0, lam);
+  __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int grp = lane / TL::L, l = lane - grp * TL::L;
-  const bool valid = grp < TL::GPW;
   const int il = warp * TL::GPW + grp;
   const long m = i0 + il;
-  const bool active = valid && m <= N;
-  const int ic = il - 1 + TL::GH;
   const FiltConst FC = filt_const(a.epsf, a.rf, a.factf);
-  const int ps = select_order<P, S, false>(&tile[0][valid ? ic : 0], nullptr, nullptr, TL::TW, l, grp,
-                                           active, valid, FC, a.eps, a.thr, a.fact_tau, a.psi2_mod);
-  if (active && acat_in_bounds(ic - P + 1 >= 0 && ic + P < TL::TW && il < TL::NI, a.status)) {
-    double F[S];
-    const int base = grp * TL::L;
-    const double *q0 = &tile[0][ic];
-    if (ps == 4) {
-      if constexpr (P >= 4) cat_flux<4, FLUX, double>(q0, TL::TW, l, base, lam, a.adv, gm1, F);
-    } else if (ps == 3) {
-      if constexpr (P >= 3) if (l < 6) cat_flux<3, FLUX, double>(q0, TL::TW, l, base, lam, a.adv, gm1, F);
-    } else if (ps == 2) {
-      if constexpr (P >= 2) if (l < 4) cat_flux<2, FLUX, double>(q0, TL::TW, l, base, lam, a.adv, gm1, F);
-    } else {
-      flcat2_flux<FLUX, TL::L>(q0, TL::TW, l, ((1u << TL::L) - 1u) << base, lam, a.adv, a.gamma,
-                               a.limiter_form, a.lo_flux, F);
-    }
-    if (l == 0) {
-#pragma unroll
-      for (int c = 0; c < S; c++) Fs[il][c] = F[c];
-      if (a.orders) a.orders[m] = (int8_t)ps;
-    }
+  reject_pass_f64<P, FLUX, NWF, 1>(a, sm, i0, N, FC);
+  if (P >= 2) __syncthreads();
+  if (grp < TL::GPW && m <= N &&
+      acat_in_bounds(il - 1 + TL::GH - P + 1 >= 0 && il - 1 + TL::GH + P < TL::TW && il < TL::NI, a.status)) {
+    const int ps = iface_f64<P, FLUX, NWF, 1>(a, sm, il, grp, l, warp, lam);
+    if (l == 0 && a.orders) a.orders[m] = (int8_t)ps;
   }
   __syncthreads();
+  flux_finish_f64<P, FLUX, NWF, 1>(sm, i0, N);
   const long nI = (N + 1 - i0) < TL::NI ? (N + 1 - i0) : TL::NI;  // interfaces of this CTA
   const bool has_left = blockIdx.x > 0, has_right = i0 + TL::NI <= N;
   // the hand-off indices: this CTA's edge slots and counters
@@ -202,7 +182,7 @@ __global__ void __launch_bounds__(NWF * 32, 16 / NWF) k_step1d_fine(const Step1D
     double un[S];
 #pragma unroll
     for (int c = 0; c < S; c++) {
-      un[c] = tile[c][k] + lam * (Fl[c] - Fr[c]);
+      un[c] = sm.tile[c][k] + lam * (Fl[c] - Fr[c]);
       uout[c * N + i] = un[c];
     }
     bool ok;
@@ -210,16 +190,8 @@ __global__ void __launch_bounds__(NWF * 32, 16 / NWF) k_step1d_fine(const Step1D
     bad |= !ok;
   }
   if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(a.status, (unsigned)ACAT_STATUS_NONPHYSICAL);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) smax = fmax(smax, __shfl_xor_sync(0xffffffffu, smax, o));
-  if (lane == 0) red[warp] = smax;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double v = red[0];
-#pragma unroll
-    for (int w = 1; w < NWF; w++) v = fmax(v, red[w]);
-    atomic_max_pos(&a.smax[(a.slot + 1) % 3], v);
-  }
+  const double v = block_max<NWF>(smax, sm.red);
+  if (threadIdx.x == 0) atomic_max_pos(&a.smax[(a.slot + 1) % 3], v);
   acat_pdl_release();
 }
 

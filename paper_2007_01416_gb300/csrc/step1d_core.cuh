@@ -8,7 +8,7 @@
 #include <cstring>
 #include <type_traits>
 
-#include "phys1d.cuh"
+#include "split1d.cuh"
 
 namespace {
 
@@ -684,12 +684,22 @@ __device__ double step_dt(const Step1DArgs &a) {
   return dt;
 }
 
-// Shared-memory workspace of one 1D tile of NW warps.
-template <int P, int S, int NW = NT / 32>
+// Shared-memory workspace of one 1D tile of NW warps and R interface rounds.
+template <int P, int FLUX, int NW = NT / 32, int R = 1>
 struct Smem64 {
-  double tile[S][Tiling<P, NW>::TW];
-  double Fs[Tiling<P, NW>::NI][S];
-  double red[NW];
+  using TL = Tiling<P, NW, 1, R>;
+  static constexpr int S = Phys<FLUX>::S;
+  static constexpr bool kSplit = P >= 2 && FLUX != ACAT_FLUX_LINEAR;
+  double tile[S][TL::TW];
+  double Fs[TL::NI][S];  // fluxes; a float pair G until flux_finish_f64
+  typename std::conditional<kSplit, SplitRec<FLUX, TL::TW>, char>::type rec;
+  float4 xa[kSplit && S > 1 ? NW * 2 * XSET : 1];
+  float2 xb[kSplit && S > 1 ? NW * 2 * XSET : 1];
+  SplitLam lamk;
+  float du[S][TL::TW];               // u_{k+1} - u_k
+  unsigned char rej[S][TL::NI];      // rejected orders per (component, interface)
+  unsigned char code[TL::NI];        // p where Fs holds a pair, else 0
+  unsigned long long red[NW];
 };
 template <int P, int S, int NW = NT / 32, int LPN = 1, int R = 1>
 struct Smem32 {
@@ -699,73 +709,194 @@ struct Smem32 {
   float redf[NW];
 };
 
-// Block-wide maximum of `v` over NW warps (thread 0 returns it).
+// Block-wide maximum of `v` >= 0 over NW warps (thread 0 returns it).
 template <int NW = NT / 32>
-__device__ __forceinline__ double block_max(double v, double *red) {
+__device__ __forceinline__ double block_max(double v, unsigned long long *red) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-  if (lane == 0) red[warp] = v;
+  v = warp_max_pos(v);
+  if (lane == 0) red[warp] = (unsigned long long)__double_as_longlong(v);
   __syncthreads();
-  double r = red[0];
+  unsigned long long r = red[0];
   if (threadIdx.x == 0)
-    for (int w = 1; w < NW; w++) r = fmax(r, red[w]);
-  return r;
+    for (int w = 1; w < NW; w++) r = red[w] > r ? red[w] : r;
+  return __longlong_as_double((long long)r);
+}
+
+// Staging of an FP64 tile (cells i0 - GH + k of an instance of N cells whose
+// state starts at cell `off` of arrays with component stride M), one thread
+// per cell: the values, their first differences rounded to float (for the
+// order decisions) and the records of the float-float recursion, all of which
+// would otherwise be formed once per interface and node on the FP64 pipe.
+template <int P, int FLUX, int NW, int R>
+__device__ __forceinline__ void stage_f64(const Step1DArgs &a, Smem64<P, FLUX, NW, R> &sm,
+                                          const double *__restrict__ uin, long off, long M, long N, long i0,
+                                          double lam) {
+  using SM = Smem64<P, FLUX, NW, R>;
+  using TL = typename SM::TL;
+  constexpr int S = SM::S;
+  for (int k = threadIdx.x; k < TL::TW; k += NW * 32) {
+    const long g = bc_index(i0 - TL::GH + k, N, a.bc), g1 = bc_index(i0 - TL::GH + k + 1, N, a.bc);
+    if (!acat_in_bounds(g >= 0 && g < N && g1 >= 0 && g1 < N && off + N <= M, a.status)) continue;
+    double u[S];
+#pragma unroll
+    for (int c = 0; c < S; c++) {
+      u[c] = uin[c * M + off + g];
+      sm.tile[c][k] = u[c];
+      if constexpr (P >= 2) sm.du[c][k] = (float)__dsub_rn(uin[c * M + off + g1], u[c]);
+    }
+    if constexpr (SM::kSplit) split_record<FLUX, TL::TW>(sm.rec, k, u, a.gamma - 1.0);
+  }
+  if constexpr (SM::kSplit) split_lam(sm.lamk, lam, (int)threadIdx.x);
+}
+
+// The order decisions of a staged FP64 tile over all threads: rejected orders
+// of every (component, interface), as reject_pass_f32.
+template <int P, int FLUX, int NW, int R>
+__device__ __forceinline__ void reject_pass_f64(const Step1DArgs &a, Smem64<P, FLUX, NW, R> &sm, long i0, long N,
+                                                const FiltConst &FC) {
+  using TL = typename Smem64<P, FLUX, NW, R>::TL;
+  constexpr int S = Phys<FLUX>::S;
+  if constexpr (P >= 2) {
+    for (int q = threadIdx.x; q < S * TL::NI; q += NW * 32) {
+      const int c = q / TL::NI, il = q - c * TL::NI, ic = il - 1 + TL::GH;
+      unsigned r = 0;
+      if (i0 + il <= N && acat_in_bounds(ic - P + 1 >= 0 && ic + P < TL::TW, a.status))
+        r = reject_set64d<P>(&sm.du[c][ic], &sm.tile[c][ic], c == 0, FC, a.eps, a.thr, a.fact_tau, a.psi2_mod);
+      sm.rej[c][il] = (unsigned char)r;
+    }
+  }
+}
+
+// CAT2p flux of interface il by the first 2p lanes of its group: the
+// float-float recursion where it holds (Fs receives the pair G and code[il]
+// the order), else FP64.
+template <int p, int P, int FLUX, int NW, int R>
+__device__ __forceinline__ void cat_iface_f64(const Step1DArgs &a, Smem64<P, FLUX, NW, R> &sm, int il, int ic,
+                                              int l, int base, int warp, double lam) {
+  constexpr int S = Phys<FLUX>::S;
+  constexpr int TW = Smem64<P, FLUX, NW, R>::TL::TW;
+  if constexpr (FLUX == ACAT_FLUX_LINEAR) {
+    const double F = cat_linear<p>(&sm.tile[0][ic], l, base, lam, a.adv);
+    if (l == 0) sm.Fs[il][0] = F;
+  } else {
+    FF G[S];
+    bool ok;
+    if constexpr (FLUX == ACAT_FLUX_EULER1D) {
+      const int xo = warp * 2 * XSET + (P >= 3 ? xslot(base) : base);
+      ok = cat_split_euler<p, TW>(sm.rec, a, sm.lamk.v[p - 2], ic, l, base, &sm.xa[xo], &sm.xb[xo], G);
+    } else {
+      ok = cat_split_burgers<p, TW>(sm.rec, (float)a.cfl * __frcp_rn((float)lam), sm.lamk.v[p - 2], ic, l, base, G);
+    }
+    if (ok) {
+      if (l == 0) {
+#pragma unroll
+        for (int c = 0; c < S; c++) *reinterpret_cast<float2 *>(&sm.Fs[il][c]) = make_float2(G[c].h, G[c].l);
+        sm.code[il] = (unsigned char)p;
+      }
+    } else {
+      double F[S];
+      cat_flux<p, FLUX, double>(&sm.tile[0][ic], Smem64<P, FLUX, NW, R>::TL::TW, l, base, lam, a.adv,
+                                a.gamma - 1.0, F);
+      if (l == 0) {
+#pragma unroll
+        for (int c = 0; c < S; c++) sm.Fs[il][c] = F[c];
+      }
+    }
+  }
+}
+
+// Selected order and flux of interface il of an FP64 tile by the L lanes of
+// group grp.
+template <int P, int FLUX, int NW, int R>
+__device__ __forceinline__ int iface_f64(const Step1DArgs &a, Smem64<P, FLUX, NW, R> &sm, int il, int grp, int l,
+                                         int warp, double lam) {
+  using TL = typename Smem64<P, FLUX, NW, R>::TL;
+  constexpr int S = Phys<FLUX>::S;
+  const int ic = il - 1 + TL::GH, base = grp * TL::L;
+  int ps = 1;
+  if constexpr (P >= 2) {
+    unsigned r = 0;
+#pragma unroll
+    for (int c = 0; c < S; c++) r |= sm.rej[c][il];
+    const unsigned accept = ~r & ((1u << (P - 1)) - 1u);
+    ps = accept ? (32 - __clz(accept)) + 1 : 1;
+  }
+  if (l == 0) sm.code[il] = 0;
+  if (ps == 4) {
+    if constexpr (P >= 4) cat_iface_f64<4, P, FLUX, NW, R>(a, sm, il, ic, l, base, warp, lam);
+  } else if (ps == 3) {
+    if constexpr (P >= 3) if (l < 6) cat_iface_f64<3, P, FLUX, NW, R>(a, sm, il, ic, l, base, warp, lam);
+  } else if (ps == 2) {
+    if constexpr (P >= 2) if (l < 4) cat_iface_f64<2, P, FLUX, NW, R>(a, sm, il, ic, l, base, warp, lam);
+  } else {
+    double F[S];
+    flcat2_flux<FLUX, TL::L>(&sm.tile[0][ic], TL::TW, l, ((1u << TL::L) - 1u) << base, lam, a.adv, a.gamma,
+                             a.limiter_form, a.lo_flux, F);
+    if (l == 0) {
+#pragma unroll
+      for (int c = 0; c < S; c++) sm.Fs[il][c] = F[c];
+    }
+  }
+  return ps;
+}
+
+// The float pairs in Fs to fluxes F = f(u_i) + G, by all threads of the CTA
+// (one barrier before and one after).
+template <int P, int FLUX, int NW, int R>
+__device__ __forceinline__ void flux_finish_f64(Smem64<P, FLUX, NW, R> &sm, long i0, long N) {
+  using SM = Smem64<P, FLUX, NW, R>;
+  using TL = typename SM::TL;
+  if constexpr (SM::kSplit) {
+    for (int q = threadIdx.x; q < TL::NI * SM::S; q += NW * 32) {
+      const int il = q / SM::S, c = q - il * SM::S;
+      if (i0 + il > N) break;
+      const int p = sm.code[il];
+      if (p == 0) continue;
+      const float2 g = *reinterpret_cast<const float2 *>(&sm.Fs[il][c]);
+      const int ic = il - 1 + TL::GH;
+      double f;
+      if constexpr (FLUX == ACAT_FLUX_EULER1D) f = sm.rec.fd[c][ic];
+      else f = __dmul_rn(__dmul_rn(0.5, sm.tile[0][ic]), sm.tile[0][ic]);
+      sm.Fs[il][c] = fma(__dadd_rn((double)g.x, (double)g.y), split_ginv(p), f);
+    }
+    __syncthreads();
+  }
 }
 
 // One FP64 tile: cells [i0, i0 + T) of an instance of N cells whose state
 // starts at cell `off` of arrays with component stride M; orders (nullable)
 // points at the instance's interface 0; the tile's maximal wave speed goes to
-// *smax_out. The CTA has NW warps.
-template <int P, int FLUX, int NW = NT / 32>
-__device__ __forceinline__ void tile_f64(const Step1DArgs &a, Smem64<P, Phys<FLUX>::S, NW> &sm,
+// *smax_out. The CTA has NW warps; each lane group takes R interfaces in R
+// rounds.
+template <int P, int FLUX, int NW = NT / 32, int R = 1>
+__device__ __forceinline__ void tile_f64(const Step1DArgs &a, Smem64<P, FLUX, NW, R> &sm,
                                          const double *__restrict__ uin, double *__restrict__ uout,
                                          long off, long M, long N, long i0, double lam,
                                          int8_t *orders, unsigned long long *smax_out) {
-  using TL = Tiling<P, NW>;
+  using TL = typename Smem64<P, FLUX, NW, R>::TL;
   constexpr int NTB = NW * 32;
   constexpr int S = Phys<FLUX>::S;
-  for (int q = threadIdx.x; q < S * TL::TW; q += NTB) {
-    const int c = q / TL::TW, k = q - c * TL::TW;
-    const long g = bc_index(i0 - TL::GH + k, N, a.bc);
-    if (acat_in_bounds(g >= 0 && g < N && off + N <= M, a.status)) sm.tile[c][k] = uin[c * M + off + g];
-  }
+  stage_f64<P, FLUX, NW, R>(a, sm, uin, off, M, N, i0, lam);
   __syncthreads();
-  const double gm1 = a.gamma - 1.0;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int grp = lane / TL::L, l = lane - grp * TL::L;
-  const bool valid = grp < TL::GPW;
-  const int il = warp * TL::GPW + grp;  // local interface
-  const long m = i0 + il;               // interface between cells m-1 and m
-  const bool active = valid && m <= N;
-  const int ic = il - 1 + TL::GH;       // tile index of cell m-1
-
   const FiltConst FC = filt_const(a.epsf, a.rf, a.factf);
-  const int ps = select_order<P, S, false>(&sm.tile[0][valid ? ic : 0], nullptr, nullptr, TL::TW, l,
-                                           grp, active, valid, FC, a.eps, a.thr, a.fact_tau, a.psi2_mod);
-
-  double F[S];
-  const int base = grp * TL::L;
-  const double *q0 = &sm.tile[0][ic];
-  if (active && acat_in_bounds(ic - P + 1 >= 0 && ic + P < TL::TW && il < TL::NI && m <= N, a.status)) {
-    if (ps == 4) {
-      if constexpr (P >= 4) cat_flux<4, FLUX, double>(q0, TL::TW, l, base, lam, a.adv, gm1, F);
-    } else if (ps == 3) {
-      if constexpr (P >= 3) if (l < 6) cat_flux<3, FLUX, double>(q0, TL::TW, l, base, lam, a.adv, gm1, F);
-    } else if (ps == 2) {
-      if constexpr (P >= 2) if (l < 4) cat_flux<2, FLUX, double>(q0, TL::TW, l, base, lam, a.adv, gm1, F);
-    } else {
-      flcat2_flux<FLUX, TL::L>(q0, TL::TW, l, ((1u << TL::L) - 1u) << base, lam, a.adv, a.gamma,
-                               a.limiter_form, a.lo_flux, F);
-    }
-    if (l == 0) {
-#pragma unroll
-      for (int c = 0; c < S; c++) sm.Fs[il][c] = F[c];
-      if (orders && (il < TL::T || m == N)) orders[m] = (int8_t)ps;
+  reject_pass_f64<P, FLUX, NW, R>(a, sm, i0, N, FC);
+  if (P >= 2) __syncthreads();
+#pragma unroll 1
+  for (int rnd = 0; rnd < R; rnd++) {
+    if (rnd > 0) __syncwarp();  // the exchange slots of the last round are read
+    const int il = (rnd * NW + warp) * TL::GPW + grp;
+    const long m = i0 + il;  // interface between cells m-1 and m
+    if (grp < TL::GPW && m <= N &&
+        acat_in_bounds(il - 1 + TL::GH - P + 1 >= 0 && il - 1 + TL::GH + P < TL::TW && il < TL::NI, a.status)) {
+      const int ps = iface_f64<P, FLUX, NW, R>(a, sm, il, grp, l, warp, lam);
+      if (l == 0 && orders && (il < TL::T || m == N)) orders[m] = (int8_t)ps;
     }
   }
   __syncthreads();
+  flux_finish_f64<P, FLUX, NW, R>(sm, i0, N);
 
   double smax = 0.0;
   bool bad = false;

@@ -52,6 +52,14 @@ Q mul(Q a, Q b) {
 }
 Q neg(Q a) { return Q{-a.n, a.d}; }
 double to_d(Q a) { return (double)a.n / (double)a.d; }
+// a x m, an integer when m is a multiple of the denominator
+float times(Q a, int64_t m) { return (float)to_d(mul(a, mk(m, 1))); }
+
+// Common denominators per p of the node derivative weights (LC), of the time
+// weights gamma^{k,0} / k! (LQ, the coefficients of the Lagrange basis
+// polynomials) and of the flux weights (LH).
+constexpr int64_t kLC[ACAT_MAXP + 1] = {1, 1, 6, 60, 420}, kLQ[ACAT_MAXP + 1] = {1, 1, 6, 120, 5040},
+                  kLH[ACAT_MAXP + 1] = {1, 2, 12, 60, 840};
 
 // Weights of the k-th derivative at q (rational) over the integer nodes
 // x[0..n-1]; w[r] exact.
@@ -95,12 +103,26 @@ void acat_build_tables(AcatTables *T) {
     // gamma^{1,j}_{p,r}: first derivative at each node j
     for (int j = 0; j < n; j++) {
       lagrange_deriv(n, nodes, 1, mk(nodes[j], 1), w);
-      for (int r = 0; r < n; r++) T->g1[p][j][r] = to_d(w[r]);
+      for (int r = 0; r < n; r++) {
+        T->g1[p][j][r] = to_d(w[r]);
+        T->g1i[p][j][r] = times(w[r], kLC[p]);
+      }
     }
     // gamma^{k,0}_{p,r}: k-th derivative at 0 (time derivatives), k < 2p
+    int64_t kf = 1;
     for (int k = 0; k < n; k++) {
+      if (k > 1) kf *= k;
       lagrange_deriv(n, nodes, k, mk(0, 1), w);
-      for (int r = 0; r < n; r++) T->gk[p][k][r] = to_d(w[r]);
+      for (int r = 0; r < n; r++) {
+        T->gk[p][k][r] = to_d(w[r]);
+        T->lag[p][k][r] = times(mul(w[r], mk(1, kf)), kLQ[p]);
+      }
+      if (k > 0) T->ilc[p][k] = 1.0 / (double)(k * kLC[p]);
+    }
+    {
+      const double q = 1.0 / (double)kLQ[p];
+      T->ilq[p].x = (float)q;
+      T->ilq[p].y = (float)(q - (double)T->ilq[p].x);
     }
     // gamma^{2p-1,1/2}: the binomial (2p-1)-th difference (Eq. 3.12)
     lagrange_deriv(n, nodes, n - 1, mk(1, 2), w);
@@ -114,15 +136,20 @@ void acat_build_tables(AcatTables *T) {
     for (int m = 0; m < n; m++) {
       s = add(s, neg(d[m]));
       T->gh[p][m] = to_d(s);
+      T->ghi[p][m] = times(s, kLH[p]);
     }
     // Taylor coefficients r^l / l! at the 2p time levels
     for (int rr = 0; rr < n; rr++) {
       const int r = rr - p + 1;
       Q v{1, 1};
       T->taylor[p][rr][0] = 1.0;
+      int64_t pw = 1;
+      T->powr[p][rr][0] = 1.0f;
       for (int l = 1; l < n; l++) {
         v = mul(v, mk(r, l));
         T->taylor[p][rr][l] = to_d(v);
+        pw *= r;
+        T->powr[p][rr][l] = (float)pw;
       }
     }
     // (2p-1)! for tau_p
@@ -146,5 +173,6 @@ void acat_build_tables(AcatTables *T) {
       }
     }
   }
+  for (int k = 1; k <= ACAT_MAXN; k++) T->k840[k] = (float)(840 / k);
   for (int k = 0; k <= ACAT_MAXN; k++) T->invfactf[k] = (float)T->invfact[k];
 }
