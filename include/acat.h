@@ -163,16 +163,18 @@ int acat_create_batched(const acat_params *p, int n_inst, const int32_t *n_per_i
  *     bit for bit.
  *   - Batched contexts: the batch is cut into tiles of
  *     T = R nw floor(32 / (2P lpn)) - 1 consecutive cells of one instance,
- *     R = 8 interface rounds per lane group in FP32 (2 at nw = 16), 1 in
- *     FP64 (P = 3, nw = 8, lpn = 1: 319 in FP32, 39 in FP64); one CTA of nw
+ *     R = 8 interface rounds per lane group in FP32 (2 at nw = 16), 4, 2 and 1
+ *     in FP64 at nw = 4, 8 and 16 (P = 3, nw = 8, lpn = 1: 319 in FP32, 79 in
+ *     FP64); one CTA of nw
  *     warps per tile at a time,
  *     on a grid of (SM count) x cps CTAs that take the tiles from a queue
  *     (cps = 0: the kernel's occupancy). nw in {4, 8, 16}. At a fixed lpn,
  *     nw and cps only move work between CTAs: every interface flux, wave
  *     speed and update is computed from the same values, so the states are
  *     bit-identical.
- *   - Single-instance contexts: cps is 0. FP64: nw is fixed (8; 2 for the
- *     small-CTA step of large grids). FP32: nw = 8 (the fused step, lpn 1
+ *   - Single-instance contexts: cps is 0. FP64: nw is fixed, 8 or, for large
+ *     grids, 2: a label of the grid size, so that shapes a caller has stored
+ *     still apply; the step picks its tiles by a rule on P and N. FP32: nw = 8 (the fused step, lpn 1
  *     or 2), nw = 7 (the fused step in tiles of 7 floor(32 / 2P) - 1
  *     cells, lpn = 1: a grid of a few waves then fills every SM with the
  *     same number of CTAs) or nw = 2 (the small-CTA step with the boundary

@@ -53,7 +53,8 @@ struct Step1DArgs {
   int lo_flux;                // F^lo: ACAT_LO_*
   int slot;                   // step index mod 3 (dt-reduction slots)
   int lpn;                    // FP32 1D: lanes per stencil node (1, or 2 for P = 2, 4)
-  int nw;                     // FP32 1D fused step: warps per CTA (8, or 7; 0 reads as 8)
+  int nw;                     // warps per CTA: FP64 1D 4..8; FP32 1D fused step 8, or 7 (0 reads as 8)
+  int rounds;                 // FP64 1D: interface rounds per lane group
   double dx, cfl;
   double dt_fixed;            // > 0: imposed dt
   const double *dt_in;        // device: imposed dt (nullable; takes precedence)
@@ -70,9 +71,9 @@ struct Step1DArgs {
   int8_t *orders;             // N+1 order codes (nullable)
   double *dt_out;             // dt used (nullable)
   unsigned *status;           // sticky status bits
-  double *flux_buf;           // FP64 single instance: [S][N+1] CTA-edge fluxes, and
+  float *flux_buf;            // FP32 single instance: [S][N+1] CTA-edge increments, and
   int *cnt;                   // one hand-off counter per CTA boundary (both nullable: the
-                              // fused 8-warp step kernel runs instead of the small-CTA one)
+                              // fused step kernel runs instead of the small-CTA one)
 };
 
 // A double as a pair of floats, and the pairs of a step's arguments (host).
@@ -178,6 +179,8 @@ int acat_upload_tables_current_device();
 // returns an acat error code.
 int acat_ensure_tables(int dev);
 int acat_cells_per_cta_1d(int P, int prec);
-// CTAs of the small-CTA FP64 step (boundary counters it needs: that many).
+// Tile shape of the FP64 step of an N-cell instance on `sms` SMs.
+void acat_shape_f64(int P, long N, int sms, int *nw, int *rounds);
+// CTAs of the small-CTA FP32 step (boundary counters it needs: that many).
 int acat_fine_ctas_1d(int P, long N);
 double acat_fma_peak_run(int precision, void *stream);

@@ -51,9 +51,11 @@ struct acat_ctx {
   void *d_seg = nullptr;                  // adjoint run: recomputed states of a segment
   size_t seg_bytes = 0;
   void *d_bar = nullptr;                  // adjoint run: second cotangent buffer
-  double *d_flux = nullptr;               // 1D: CTA-edge fluxes (FP32: increments) of the small-CTA step
+  float *d_flux = nullptr;                // 1D FP32: CTA-edge increments of the small-CTA step
   int *d_cnt = nullptr;                   // 1D: its boundary hand-off counters
-  int snw = 8;                            // 1D FP32 single instance: warps per CTA (8 or 7 fused, 2 small-CTA)
+  int snw = 8;                            // 1D single instance: FP32 warps per CTA (8 or 7 fused, 2 small-CTA);
+                                          // FP64 the reported label (8, or 2 for large grids)
+  int fnw = 8, frounds = 1;               // 1D FP64: warps per CTA and interface rounds
 };
 
 namespace {
@@ -137,12 +139,13 @@ Step1DArgs base_args(acat_ctx *c) {
   acat_set_pairs(a);
   a.smax = c->d_smax;
   a.status = c->d_status;
-  // the small-CTA step: FP64 whenever its buffers exist, FP32 when chosen
-  const bool fine = c->d_flux && (p.precision != ACAT_PREC_F32 || c->snw == NWF_API);
+  // the small-CTA FP32 step when chosen
+  const bool fine = c->d_flux && c->snw == NWF_API;
   a.flux_buf = fine ? c->d_flux : nullptr;
   a.cnt = fine ? c->d_cnt : nullptr;
   a.lpn = c->lpn;
-  a.nw = p.precision == ACAT_PREC_F32 && c->snw == 7 ? 7 : 0;
+  a.nw = p.precision != ACAT_PREC_F32 ? c->fnw : (c->snw == 7 ? 7 : 0);
+  a.rounds = c->frounds;
   return a;
 }
 
@@ -386,21 +389,22 @@ int acat_create(const acat_params *p, acat_ctx **out) {
   if (e == cudaSuccess) e = cudaMalloc(&c->d_t, 3 * sizeof(double));
   if (e == cudaSuccess) e = cudaMalloc(&c->d_status, sizeof(unsigned));
   if (e == cudaSuccess) e = cudaMalloc(&c->d_work, sb);
-  // 1D FP64: the small-CTA step when the 8-warp fused step would not fit its
-  // CTAs in ~3/4 of one wave at 2 CTAs per SM (it then leaves SMs idle)
   int sms = 0;
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
-  const long fused_ctas = (p->nx + acat_cells_per_cta_1d(p->P, ACAT_PREC_F64) - 1) /
-                          acat_cells_per_cta_1d(p->P, ACAT_PREC_F64);
+  // 1D FP64: the tile shape, and the label acat_launch_shape reports (2 where
+  // 8-warp tiles of one round would exceed 3/4 of a wave at 2 CTAs per SM)
+  if (e == cudaSuccess && c->dim == 1 && p->precision == ACAT_PREC_F64) {
+    acat_shape_f64(p->P, p->nx, sms, &c->fnw, &c->frounds);
+    const long T = acat_cells_per_cta_1d(p->P, ACAT_PREC_F64), ctas = (p->nx + T - 1) / T;
+    c->snw = 4 * ctas > 3 * 2 * (long)sms ? NWF_API : 8;
+  }
   // 1D FP32: the small-CTA step is available to every context through
   // acat_set_launch_shape and the autotuner; the fused step (8 or 7 warps, set
   // below) stays the default (at FP32 step times the hand-off's fences and the
   // small CTAs' serial update phases cost more than their even load saves)
-  const bool f64_fine = p->precision == ACAT_PREC_F64 && 4 * fused_ctas > 3 * 2 * (long)sms;
-  const bool f32_fine = p->precision == ACAT_PREC_F32;
-  if (e == cudaSuccess && c->dim == 1 && (f64_fine || f32_fine)) {
+  if (e == cudaSuccess && c->dim == 1 && p->precision == ACAT_PREC_F32) {
     const size_t nc = (size_t)acat_fine_ctas_1d(p->P, p->nx);
-    e = cudaMalloc(&c->d_flux, (size_t)c->s * (size_t)(p->nx + 1) * sizeof(double));
+    e = cudaMalloc(&c->d_flux, (size_t)c->s * (size_t)(p->nx + 1) * sizeof(float));
     if (e == cudaSuccess) e = cudaMalloc(&c->d_cnt, nc * sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(c->d_cnt, 0, nc * sizeof(int));
   }
@@ -490,10 +494,8 @@ int acat_launch_shape(const acat_ctx *c, int *nw, int *lpn, int *cps) {
   if (c->batched) {
     w = c->bnw;
     k = c->bcps > 0 ? c->bcps : acat_batch_occupancy(c->p.P, c->p.flux, c->p.precision, c->bnw, c->lpn);
-  } else if (c->p.precision == ACAT_PREC_F32) {
+  } else {
     w = c->snw;
-  } else if (c->d_flux) {
-    w = NWF_API;  // the small-CTA FP64 step
   }
   if (nw) *nw = w;
   if (lpn) *lpn = c->lpn;

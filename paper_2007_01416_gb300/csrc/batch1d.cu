@@ -98,8 +98,9 @@ __global__ void __launch_bounds__(NW * 32, MinCtas<P, F32>::value * 8 / NW)
       tile_f32<P, FLUX, NW, LPN, R>(a, sm[par], static_cast<const float *>(a.u_in),
                                     static_cast<float *>(a.u_out), off, bt.M, N, i0, &bt.lamf[b], ord, so);
     } else {
-      tile_f64<P, FLUX, NW, R>(a, sm[0], static_cast<const double *>(a.u_in), static_cast<double *>(a.u_out),
-                            off, bt.M, N, i0, bt.lam[b], ord, so);
+      tile_f64<P, FLUX, NW, R>(a, sm[0], shape64<P>(NW * 32, R), static_cast<const double *>(a.u_in),
+                               static_cast<double *>(a.u_out), off, bt.M, N, i0, &bt.lam[b], ord, so);
+      __syncthreads();  // one workspace: the next tile's staging waits for this one's update
     }
     w = (long)s_next[par];
   }

@@ -262,7 +262,7 @@ __device__ __forceinline__ int psi2m_filter(const float *d, const float *e, floa
   const float sm = d[0] * d[0], s0 = d[1] * d[1], sp = d[2] * d[2];
   const float I1L = sm + eps, I1R = (s0 + sp) + eps, I2L = (sm + s0) + eps, I2R = sp + eps;
   const float mn = fminf(fminf(I1L, I1R), fminf(I2L, I2R)), mx = fmaxf(fmaxf(I1L, I1R), fmaxf(I2L, I2R));
-  if (!(mn > 1e-30f) || !(mx < 1e30f)) return -1;
+  if (!(mn > 1e-18f) || !(mx < 1e18f)) return -1;  // products of two stay normal floats
   const float I1 = I1L * I1R / (I1L + I1R), I2 = I2L * I2R / (I2L + I2R);
   float t[3], b[3];
 #pragma unroll
@@ -345,7 +345,8 @@ __device__ __forceinline__ void psi_filter_all(const float *d, const float *e, f
     el = fmaf(bl, 2.0f * fabsf(dl) + bl, el);
     er = fmaf(br, 2.0f * fabsf(dr) + br, er);
     const float IL = il + eps, IR = ir + eps;
-    if (!(IL > 1e-30f && IR > 1e-30f) || !(IL < 1e30f && IR < 1e30f)) {
+    // outside this range the product IL IR would leave the normal floats
+    if (!(IL > 1e-18f && IR > 1e-18f) || !(IL < 1e18f && IR < 1e18f)) {
       u |= bit;
       continue;
     }
@@ -413,8 +414,9 @@ __device__ __forceinline__ unsigned reject_set64(const double *q, int st, bool f
   return reject_set<PM>(d, e, [=](int j) { return q[j * st]; }, first, F, eps, thr, fact, psi2_mod);
 }
 
-// The same with the first differences of the component's cells already
-// rounded to float, d_j = u_{j+1} - u_j at du[j] (consecutive cells).
+// The same with the first differences of the component's cells already in
+// float, d_j = u_{j+1} - u_j truncated to 24 bits (0 below 2^-126) at du[j]
+// (consecutive cells).
 template <int PM>
 __device__ __forceinline__ unsigned reject_set64d(const float *du, const double *q, bool first,
                                                   const FiltConst &F, double eps, double thr, const double *fact,
@@ -423,7 +425,7 @@ __device__ __forceinline__ unsigned reject_set64d(const float *du, const double 
 #pragma unroll
   for (int k = 0; k < 2 * PM - 1; k++) {
     d[k] = du[k - PM + 1];
-    e[k] = 6.0e-8f * fabsf(d[k]) + 1e-44f;
+    e[k] = 1.2e-7f * fabsf(d[k]) + 1.2e-38f;
   }
   return reject_set<PM>(d, e, [=](int j) { return q[j]; }, first, F, eps, thr, fact, psi2_mod);
 }

@@ -115,6 +115,9 @@ extern "C" int acat_run_noalloc(const acat_params *p, void *u_dev, int nsteps, d
   a.gammaf = (float)p->gamma;
   a.gm1f = (float)(p->gamma - 1.0);
   acat_set_pairs(a);
+  int sms = 0;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return ACAT_ERR_CUDA;
+  acat_shape_f64(p->P, p->nx, sms, &a.nw, &a.rounds);
   a.smax = smax;
   a.tslot = tslot;
   a.status = status;

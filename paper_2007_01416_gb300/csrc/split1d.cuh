@@ -72,10 +72,37 @@ __device__ __forceinline__ void ff_acc(FF &s, FF x, float g) {
   s.h = t.h;
   s.l = __fadd_rn(__fadd_rn(s.l, t.l), e);
 }
-__device__ __forceinline__ FF ff_from(double x) {
-  const float h = (float)x;
-  return FF{h, (float)__dsub_rn(x, (double)h)};
+// The top 47 (pair, rounded) or all 53 bits (F3) of a double as floats, by
+// integer operations on its bits: conversions would occupy the FP64 pipe (64
+// cycles per warp each), and a record holds 21 of them. Parts carry the sign of
+// x; the parts after the first are 0 for |x| below 2^-75, all are below 2^-126,
+// and infinities, NaN and values beyond 2^127 give parts that are not finite.
+struct Bits64 {
+  unsigned hi, lo;  // the float bits of the top 24 bits; the low 29 bits of the mantissa
+  float ulp;        // +-2^(exponent - 52), the weight of the lowest mantissa bit
+};
+__device__ __forceinline__ Bits64 bits_of(double x) {
+  const unsigned h = (unsigned)__double2hiint(x), l = (unsigned)__double2loint(x);
+  const int e = (int)((h >> 20) & 0x7ffu) - 896;  // float exponent field
+  const unsigned s = h & 0x80000000u;
+  const unsigned mant = __funnelshift_l(l, h, 3) & 0x7fffffu;
+  Bits64 r;
+  const bool fin = e < 255, nz = e > 0;
+  r.hi = s | (nz ? (fin ? ((unsigned)e << 23) | mant : 0x7fffffffu) : 0u);
+  r.lo = nz ? l & 0x1fffffffu : 0u;
+  // 2^(e - 52 - 127), flushed to 0 below the normal range
+  r.ulp = __uint_as_float(s | (e > 52 ? (unsigned)(e - 52) << 23 : 0u));
+  return r;
 }
+// an integer up to 2^23 as a float
+__device__ __forceinline__ float small_float(unsigned n) {
+  return __fsub_rn(__uint_as_float(0x4b000000u + n), 8388608.0f);
+}
+__device__ __forceinline__ FF ff_bits(double x) {
+  const Bits64 b = bits_of(x);
+  return FF{__uint_as_float(b.hi), __fmul_rn(small_float((b.lo + 32u) >> 6), __fmul_rn(64.0f, b.ulp))};
+}
+__device__ __forceinline__ float f_bits(double x) { return __uint_as_float(bits_of(x).hi); }
 __device__ __forceinline__ FF ff_of(float2 a) { return FF{a.x, a.y}; }
 
 // An FP64 value as three floats h + m + l (exact for values in float's range),
@@ -84,12 +111,9 @@ struct F3 {
   float h, m, l;
 };
 __device__ __forceinline__ F3 f3_from(double x) {
-  F3 r;
-  r.h = (float)x;
-  const double y = __dsub_rn(x, (double)r.h);
-  r.m = (float)y;
-  r.l = (float)__dsub_rn(y, (double)r.m);
-  return r;
+  const Bits64 b = bits_of(x);
+  return F3{__uint_as_float(b.hi), __fmul_rn(small_float(b.lo >> 14), __fmul_rn(16384.0f, b.ulp)),
+            __fmul_rn(small_float(b.lo & 0x3fffu), b.ulp)};
 }
 __device__ __forceinline__ FF f3_diff(F3 a, F3 b) {
   const FF s = ff_two(a.h, -b.h), t = ff_two(a.m, -b.m), w = ff_two(s.h, t.h);
@@ -106,6 +130,10 @@ __device__ __forceinline__ double split_ginv(int p) {
 constexpr float SPLIT_TAU = 0x1p-5f;    // increments, of the local scales
 constexpr float SPLIT_QUAD = 0x1p-23f;  // quadratic terms that float carries
 constexpr float SPLIT_TAIL = 0x1p-28f;  // F^(k-2) from which on float suffices
+
+// A scale that the pairs carry: their low parts (2^-53 of it) stay normal floats
+// and so do products of two scales.
+__device__ __forceinline__ bool split_range(float x) { return x > 0x1p-42f && x < 0x1p60f; }
 
 // Per-cell records of a staged tile of TW cells (what a stencil node needs,
 // computed once per cell instead of once per interface and node).
@@ -128,7 +156,7 @@ struct SplitRec<ACAT_FLUX_EULER1D, TW> {
 template <int FLUX, int TW>
 __device__ __forceinline__ void split_record(SplitRec<FLUX, TW> &r, int k, const double *u, double gm1) {
   if constexpr (FLUX == ACAT_FLUX_BURGERS) {
-    const FF w = ff_from(u[0]);
+    const FF w = ff_bits(u[0]);
     const F3 f = f3_from(__dmul_rn(__dmul_rn(0.5, u[0]), u[0]));
     r.u[k] = make_float2(w.h, w.l);
     r.f[k] = make_float4(f.h, f.m, f.l, 0.0f);
@@ -141,10 +169,11 @@ __device__ __forceinline__ void split_record(SplitRec<FLUX, TW> &r, int k, const
     r.fd[0][k] = u[1];
     r.fd[1][k] = f1;
     r.fd[2][k] = f2;
-    const FF R = ff_from(u[0]), V = ff_from(v), Hh = ff_from(h);
+    const FF R = ff_bits(u[0]), V = ff_bits(v), Hh = ff_bits(h);
     const F3 a = f3_from(u[1]), b = f3_from(f1), c = f3_from(f2);
-    const bool fine = R.h > 0x1p-50f && R.h < 0x1p50f && Hh.h > 0x1p-50f && Hh.h < 0x1p50f;
-    const float s = fine ? __fsqrt_rn(Hh.h) : __int_as_float(0x7fffffff);
+    const float s0 = __fsqrt_rn(Hh.h), m0 = __fmul_rn(R.h, s0), m1 = __fmul_rn(R.h, Hh.h), m2 = __fmul_rn(m1, s0);
+    const bool fine = split_range(R.h) && split_range(Hh.h) && split_range(m0) && split_range(m1) && split_range(m2);
+    const float s = fine ? s0 : __int_as_float(0x7fffffff);
     r.q[0][k] = make_float4(R.h, R.l, V.h, V.l);
     r.q[1][k] = make_float4(Hh.h, Hh.l, s, a.l);
     r.q[2][k] = make_float4(a.h, b.h, c.h, b.l);
@@ -159,7 +188,7 @@ struct SplitLam {
 __device__ __forceinline__ void split_lam(SplitLam &s, double lam, int t) {
   if (t < 21) {
     const int p = 2 + t / 7, k1 = t - (p - 2) * 7 + 1;
-    const FF x = ff_from(__dmul_rn(-lam, c_tab.ilc[p][k1]));
+    const FF x = ff_bits(__dmul_rn(-lam, c_tab.ilc[p][k1]));
     s.v[p - 2][k1 - 1] = make_float2(x.h, x.l);
   }
 }
@@ -381,7 +410,7 @@ __device__ __forceinline__ bool cat_split_burgers(const SplitRec<ACAT_FLUX_BURGE
   const float4 fj = rec.f[jc], fi = rec.f[ic];
   const FF Y0 = f3_diff(F3{fj.x, fj.y, fj.z}, F3{fi.x, fi.y, fi.z});
   const float v2 = __fmul_rn(vs, vs);
-  if (!__all_sync(mask, vs > 0x1p-50f && vs < 0x1p50f && fabsf(Y0.h) <= SPLIT_TAU * v2)) return false;
+  if (!__all_sync(mask, split_range(vs) && split_range(v2) && fabsf(Y0.h) <= SPLIT_TAU * v2)) return false;
   FF S;
   bool allow = true;
 #pragma unroll 1

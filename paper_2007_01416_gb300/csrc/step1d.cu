@@ -42,16 +42,20 @@
 
 namespace {
 
+// Interface rounds per lane group an 8-warp FP64 tile has room for.
+constexpr int MAX_ROUNDS64 = 3;
+
 template <int P, int FLUX>
 __global__ void __launch_bounds__(NT, MinCtas<P, false>::value) k_step1d_f64(const Step1DArgs a) {
   acat_pdl_wait();
-  __shared__ Smem64<P, FLUX> sm;
+  __shared__ Smem64<P, FLUX, NT / 32, MAX_ROUNDS64> sm;
   __shared__ double s_lam;
-  if (threadIdx.x == 0) s_lam = step_dt(a) / a.dx;
-  __syncthreads();
-  tile_f64<P, FLUX>(a, sm, static_cast<const double *>(a.u_in), static_cast<double *>(a.u_out), 0,
-                    a.N, a.N, (long)blockIdx.x * Tiling<P>::T, s_lam, a.orders,
-                    &a.smax[(a.slot + 1) % 3]);
+  const Shape64 sh = shape64<P>((int)blockDim.x, a.rounds);
+  // dt by the last warp, which has the fewest cells to stage (none at R = 1)
+  if (threadIdx.x == blockDim.x - 32) s_lam = step_dt(a) / a.dx;
+  tile_f64<P, FLUX, NT / 32, MAX_ROUNDS64>(
+      a, sm, sh, static_cast<const double *>(a.u_in), static_cast<double *>(a.u_out), 0, a.N, a.N,
+      (long)blockIdx.x * (sh.NI - 1), &s_lam, a.orders, &a.smax[(a.slot + 1) % 3]);
   acat_pdl_release();
 }
 
@@ -68,130 +72,6 @@ __global__ void __launch_bounds__(NW * 32, MinCtas<P, true>::value) k_step1d_f32
   tile_f32<P, FLUX, NW, LPN>(a, sm, static_cast<const float *>(a.u_in), static_cast<float *>(a.u_out), 0, a.N,
                              a.N, (long)blockIdx.x * Tiling<P, NW, LPN>::T, &s_lam, a.orders,
                              &a.smax[(a.slot + 1) % 3]);
-  acat_pdl_release();
-}
-
-// FP64 step in small CTAs (NWF warps): CTA b computes the NI interfaces
-// [b NI, b NI + NI) and updates the cells between them; the cell between
-// two CTAs is updated by whichever of the two finishes second. Each CTA
-// publishes its edge fluxes, fences (release), and counts itself in at the
-// boundary counters of its left and right neighbours (atomicAdd; no CTA ever
-// waits): the one that reads 1 fences again (acquire), owns the boundary
-// cell, reads the other edge flux from L2 and resets the counter for the next
-// step. Small CTAs spread a step's interfaces evenly over the SMs, and no
-// interface is computed twice.
-template <int P, int FLUX>
-__global__ void __launch_bounds__(NWF * 32, 16 / NWF) k_step1d_fine(const Step1DArgs a) {
-  acat_pdl_wait();
-  using TL = Tiling<P, NWF>;
-  constexpr int S = Phys<FLUX>::S;
-  constexpr int NTF = NWF * 32;
-  __shared__ Smem64<P, FLUX, NWF> sm;
-  __shared__ double s_lam;
-  __shared__ int s_own[2];
-  auto &Fs = sm.Fs;
-  const long N = a.N, i0 = (long)blockIdx.x * TL::NI;
-  const double *__restrict__ uin = static_cast<const double *>(a.u_in);
-  double *__restrict__ uout = static_cast<double *>(a.u_out);
-  if (threadIdx.x == 0) s_lam = step_dt(a) / a.dx;
-  __syncthreads();
-  const double lam = s_lam;
-  stage_f64<P, FLUX, NWF, 1>(a, sm, uin, 0, N, N, i0, lam);
-  __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int grp = lane / TL::L, l = lane - grp * TL::L;
-  const int il = warp * TL::GPW + grp;
-  const long m = i0 + il;
-  const FiltConst FC = filt_const(a.epsf, a.rf, a.factf);
-  reject_pass_f64<P, FLUX, NWF, 1>(a, sm, i0, N, FC);
-  if (P >= 2) __syncthreads();
-  if (grp < TL::GPW && m <= N &&
-      acat_in_bounds(il - 1 + TL::GH - P + 1 >= 0 && il - 1 + TL::GH + P < TL::TW && il < TL::NI, a.status)) {
-    const int ps = iface_f64<P, FLUX, NWF, 1>(a, sm, il, grp, l, warp, lam);
-    if (l == 0 && a.orders) a.orders[m] = (int8_t)ps;
-  }
-  __syncthreads();
-  flux_finish_f64<P, FLUX, NWF, 1>(sm, i0, N);
-  const long nI = (N + 1 - i0) < TL::NI ? (N + 1 - i0) : TL::NI;  // interfaces of this CTA
-  const bool has_left = blockIdx.x > 0, has_right = i0 + TL::NI <= N;
-  // the hand-off indices: this CTA's edge slots and counters
-  const bool ho_ok = acat_in_bounds(i0 + TL::NI - 1 <= N || !has_right, a.status) &&
-                     acat_in_bounds(blockIdx.x < gridDim.x && (long)gridDim.x * TL::NI >= N + 1, a.status);
-  if (threadIdx.x == 0 && ho_ok) {
-    // publish the edge fluxes, then count in at both boundaries
-#pragma unroll
-    for (int c = 0; c < S; c++) {
-      if (has_left) a.flux_buf[c * (N + 1) + i0] = Fs[0][c];
-      if (has_right) a.flux_buf[c * (N + 1) + i0 + TL::NI - 1] = Fs[TL::NI - 1][c];
-    }
-    __threadfence();
-    int own0 = 0, own1 = 0;
-    if (has_left && atomicAdd(&a.cnt[blockIdx.x - 1], 1) == 1) {
-      own0 = 1;
-      a.cnt[blockIdx.x - 1] = 0;
-    }
-    if (has_right && atomicAdd(&a.cnt[blockIdx.x], 1) == 1) {
-      own1 = 1;
-      a.cnt[blockIdx.x] = 0;
-    }
-    // acquire: the neighbour's edge flux, published before its fence and
-    // atomic, is read (by any thread, after the barrier below) only after
-    // this fence, which follows the atomic that observed it
-    if (own0 | own1) __threadfence();
-    s_own[0] = own0;
-    s_own[1] = own1;
-  }
-  if (threadIdx.x == 0 && !ho_ok) s_own[0] = s_own[1] = 0;
-  __syncthreads();
-  double smax = 0.0;
-  bool bad = false;
-  // cells t = 0 .. nI - 2 lie between two interfaces of this CTA; task nI - 1
-  // is the left boundary cell i0 - 1, task nI the right one i0 + NI - 1
-  for (int t = threadIdx.x; t <= nI; t += NTF) {
-    long i;
-    int k;
-    double Fl[S], Fr[S];
-    if (t < nI - 1) {
-      i = i0 + t;
-      k = t + TL::GH;
-#pragma unroll
-      for (int c = 0; c < S; c++) {
-        Fl[c] = Fs[t][c];
-        Fr[c] = Fs[t + 1][c];
-      }
-    } else if (t == nI - 1) {
-      if (!s_own[0]) continue;
-      i = i0 - 1;
-      k = TL::GH - 1;
-#pragma unroll
-      for (int c = 0; c < S; c++) {
-        Fl[c] = __ldcg(&a.flux_buf[c * (N + 1) + i0 - 1]);
-        Fr[c] = Fs[0][c];
-      }
-    } else {
-      if (!s_own[1]) continue;
-      i = i0 + TL::NI - 1;
-      k = TL::NI - 1 + TL::GH;
-#pragma unroll
-      for (int c = 0; c < S; c++) {
-        Fl[c] = Fs[TL::NI - 1][c];
-        Fr[c] = __ldcg(&a.flux_buf[c * (N + 1) + i0 + TL::NI]);
-      }
-    }
-    if (!acat_in_bounds(k >= 0 && k < TL::TW && i >= 0 && i < N, a.status)) continue;
-    double un[S];
-#pragma unroll
-    for (int c = 0; c < S; c++) {
-      un[c] = sm.tile[c][k] + lam * (Fl[c] - Fr[c]);
-      uout[c * N + i] = un[c];
-    }
-    bool ok;
-    smax = fmax(smax, Phys<FLUX>::speed(un, a.adv, a.gamma, ok));
-    bad |= !ok;
-  }
-  if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(a.status, (unsigned)ACAT_STATUS_NONPHYSICAL);
-  const double v = block_max<NWF>(smax, sm.red);
-  if (threadIdx.x == 0) atomic_max_pos(&a.smax[(a.slot + 1) % 3], v);
   acat_pdl_release();
 }
 
@@ -222,7 +102,7 @@ __global__ void __launch_bounds__(NWF * 32, 16) k_step1d_fine_f32(const Step1DAr
   const long N = a.N, i0 = (long)blockIdx.x * TL::NI;
   const float *__restrict__ uin = static_cast<const float *>(a.u_in);
   float *__restrict__ uout = static_cast<float *>(a.u_out);
-  float *__restrict__ gbuf = reinterpret_cast<float *>(a.flux_buf);
+  float *__restrict__ gbuf = a.flux_buf;
   if (threadIdx.x == 0) s_lam = (float)(step_dt(a) / a.dx);
   for (int q = threadIdx.x; q < S * TL::TW; q += NTF) {
     const int c = q / TL::TW, k = q - c * TL::TW;
@@ -360,8 +240,9 @@ template <int P, int FLUX, bool F32>
 int launch_p(const Step1DArgs &a, cudaStream_t st) {
   using TL = Tiling<P>;
   if constexpr (!F32) {
-    if (a.flux_buf && a.cnt)  // small-CTA step with boundary hand-off
-      return acat_launch_dep(k_step1d_fine<P, FLUX>, (unsigned)acat_fine_ctas_1d(P, a.N), NWF * 32, st, a);
+    if (a.nw < 1 || a.nw > NT / 32 || a.rounds < 1 || a.rounds > MAX_ROUNDS64) return (int)cudaErrorInvalidValue;
+    const long T = (long)a.nw * Tiling<P>::GPW * a.rounds - 1;
+    return acat_launch_dep(k_step1d_f64<P, FLUX>, (unsigned)((a.N + T - 1) / T), a.nw * 32, st, a);
   }
   if constexpr (F32) {
     if (a.flux_buf && a.cnt && a.lpn == 1)  // small-CTA step with boundary hand-off
@@ -379,9 +260,10 @@ int launch_p(const Step1DArgs &a, cudaStream_t st) {
     }
     if (a.nw != 0 && a.nw != NT / 32) return (int)cudaErrorInvalidValue;
   }
-  const unsigned grid = (unsigned)((a.N + TL::T - 1) / TL::T);
-  if constexpr (F32) return acat_launch_dep(k_step1d_f32<P, FLUX, 1>, grid, NT, st, a);
-  else return acat_launch_dep(k_step1d_f64<P, FLUX>, grid, NT, st, a);
+  if constexpr (F32) {
+    const unsigned grid = (unsigned)((a.N + TL::T - 1) / TL::T);
+    return acat_launch_dep(k_step1d_f32<P, FLUX, 1>, grid, NT, st, a);
+  }
 }
 
 template <int FLUX, bool F32>
@@ -419,6 +301,31 @@ int launch_smax(int flux, const Step1DArgs &a, cudaStream_t st) {
 }
 
 }  // namespace
+
+// Warps per CTA and interface rounds of the FP64 step of an N-cell instance.
+// Measured over nw = 4..8, R = 1..3 and N = 400..262144, a step takes
+// waves x (F + R c) with F the latency outside the rounds (dt, staging, order
+// decisions, update) and c that of one round, F close to 2 c (P = 4, N = 450:
+// 17.7 us at R = 1, 23.3 at R = 2), and some 1.5 % more per warp resident on an SM
+// (16 warps fit at 128 registers). So: the shape with the least
+// waves (2 + R) (1 + 0.015 warps), waves whole up to 4 and averaged beyond.
+// N = 16384, us per step: P = 4 28.3 at (7, 2) against 36.9 at (8, 1); P = 3 23.5 at
+// (4, 2) against 29.5; P = 2 17.1-17.9 at (4..7, 1).
+void acat_shape_f64(int P, long N, int sms, int *nw_out, int *rounds_out) {
+  double best = 0.0;
+  for (int nw = 4; nw <= NT / 32; nw++)
+    for (int r = 1; r <= MAX_ROUNDS64; r++) {
+      const long T = (long)nw * (32 / (2 * P)) * r - 1;
+      const long cps = ((N + T - 1) / T + sms - 1) / sms, fit = 16 / nw;
+      const double waves = cps <= 4 * fit ? (double)((cps + fit - 1) / fit) : (double)cps / (double)fit;
+      const double cost = waves * (2 + r) * (1.0 + 0.015 * (double)(nw * (cps < fit ? cps : fit)));
+      if (best == 0.0 || cost < best) {
+        best = cost;
+        *nw_out = nw;
+        *rounds_out = r;
+      }
+    }
+}
 
 int acat_cells_per_cta_1d(int P, int /*prec*/) {
   switch (P) {

@@ -699,7 +699,6 @@ struct Smem64 {
   float du[S][TL::TW];               // u_{k+1} - u_k
   unsigned char rej[S][TL::NI];      // rejected orders per (component, interface)
   unsigned char code[TL::NI];        // p where Fs holds a pair, else 0
-  unsigned long long red[NW];
 };
 template <int P, int S, int NW = NT / 32, int LPN = 1, int R = 1>
 struct Smem32 {
@@ -722,6 +721,21 @@ __device__ __forceinline__ double block_max(double v, unsigned long long *red) {
   return __longlong_as_double((long long)r);
 }
 
+// Shape of an FP64 tile: NT threads, R interface rounds per lane group, NI
+// interfaces (NI - 1 updated cells) and TW staged cells.
+struct Shape64 {
+  int NT, R, NI, TW;
+};
+template <int P>
+__device__ __forceinline__ Shape64 shape64(int nt, int r) {
+  Shape64 s;
+  s.NT = nt;
+  s.R = r;
+  s.NI = (nt >> 5) * Tiling<P>::GPW * r;
+  s.TW = s.NI - 1 + 2 * Tiling<P>::GH;
+  return s;
+}
+
 // Staging of an FP64 tile (cells i0 - GH + k of an instance of N cells whose
 // state starts at cell `off` of arrays with component stride M), one thread
 // per cell: the values, their first differences rounded to float (for the
@@ -729,12 +743,12 @@ __device__ __forceinline__ double block_max(double v, unsigned long long *red) {
 // would otherwise be formed once per interface and node on the FP64 pipe.
 template <int P, int FLUX, int NW, int R>
 __device__ __forceinline__ void stage_f64(const Step1DArgs &a, Smem64<P, FLUX, NW, R> &sm,
-                                          const double *__restrict__ uin, long off, long M, long N, long i0,
-                                          double lam) {
+                                          const Shape64 &sh, const double *__restrict__ uin, long off, long M,
+                                          long N, long i0) {
   using SM = Smem64<P, FLUX, NW, R>;
   using TL = typename SM::TL;
   constexpr int S = SM::S;
-  for (int k = threadIdx.x; k < TL::TW; k += NW * 32) {
+  for (int k = threadIdx.x; k < sh.TW; k += sh.NT) {
     const long g = bc_index(i0 - TL::GH + k, N, a.bc), g1 = bc_index(i0 - TL::GH + k + 1, N, a.bc);
     if (!acat_in_bounds(g >= 0 && g < N && g1 >= 0 && g1 < N && off + N <= M, a.status)) continue;
     double u[S];
@@ -742,23 +756,25 @@ __device__ __forceinline__ void stage_f64(const Step1DArgs &a, Smem64<P, FLUX, N
     for (int c = 0; c < S; c++) {
       u[c] = uin[c * M + off + g];
       sm.tile[c][k] = u[c];
-      if constexpr (P >= 2) sm.du[c][k] = (float)__dsub_rn(uin[c * M + off + g1], u[c]);
+      if constexpr (P >= 2) sm.du[c][k] = f_bits(__dsub_rn(uin[c * M + off + g1], u[c]));
     }
     if constexpr (SM::kSplit) split_record<FLUX, TL::TW>(sm.rec, k, u, a.gamma - 1.0);
   }
-  if constexpr (SM::kSplit) split_lam(sm.lamk, lam, (int)threadIdx.x);
 }
 
 // The order decisions of a staged FP64 tile over all threads: rejected orders
-// of every (component, interface), as reject_pass_f32.
+// of every (component, interface), as reject_pass_f32; and the first threads'
+// share of the recursion's constants.
 template <int P, int FLUX, int NW, int R>
-__device__ __forceinline__ void reject_pass_f64(const Step1DArgs &a, Smem64<P, FLUX, NW, R> &sm, long i0, long N,
-                                                const FiltConst &FC) {
+__device__ __forceinline__ void reject_pass_f64(const Step1DArgs &a, Smem64<P, FLUX, NW, R> &sm, const Shape64 &sh,
+                                                long i0, long N, double lam) {
+  if constexpr (Smem64<P, FLUX, NW, R>::kSplit) split_lam(sm.lamk, lam, (int)threadIdx.x);
   using TL = typename Smem64<P, FLUX, NW, R>::TL;
   constexpr int S = Phys<FLUX>::S;
   if constexpr (P >= 2) {
-    for (int q = threadIdx.x; q < S * TL::NI; q += NW * 32) {
-      const int c = q / TL::NI, il = q - c * TL::NI, ic = il - 1 + TL::GH;
+    const FiltConst FC = filt_const(a.epsf, a.rf, a.factf);
+    for (int q = threadIdx.x; q < S * sh.NI; q += sh.NT) {
+      const int c = q / sh.NI, il = q - c * sh.NI, ic = il - 1 + TL::GH;
       unsigned r = 0;
       if (i0 + il <= N && acat_in_bounds(ic - P + 1 >= 0 && ic + P < TL::TW, a.status))
         r = reject_set64d<P>(&sm.du[c][ic], &sm.tile[c][ic], c == 0, FC, a.eps, a.thr, a.fact_tau, a.psi2_mod);
@@ -843,11 +859,11 @@ __device__ __forceinline__ int iface_f64(const Step1DArgs &a, Smem64<P, FLUX, NW
 // The float pairs in Fs to fluxes F = f(u_i) + G, by all threads of the CTA
 // (one barrier before and one after).
 template <int P, int FLUX, int NW, int R>
-__device__ __forceinline__ void flux_finish_f64(Smem64<P, FLUX, NW, R> &sm, long i0, long N) {
+__device__ __forceinline__ void flux_finish_f64(Smem64<P, FLUX, NW, R> &sm, const Shape64 &sh, long i0, long N) {
   using SM = Smem64<P, FLUX, NW, R>;
   using TL = typename SM::TL;
   if constexpr (SM::kSplit) {
-    for (int q = threadIdx.x; q < TL::NI * SM::S; q += NW * 32) {
+    for (int q = threadIdx.x; q < sh.NI * SM::S; q += sh.NT) {
       const int il = q / SM::S, c = q - il * SM::S;
       if (i0 + il > N) break;
       const int p = sm.code[il];
@@ -864,43 +880,42 @@ __device__ __forceinline__ void flux_finish_f64(Smem64<P, FLUX, NW, R> &sm, long
 }
 
 // One FP64 tile: cells [i0, i0 + T) of an instance of N cells whose state
-// starts at cell `off` of arrays with component stride M; orders (nullable)
-// points at the instance's interface 0; the tile's maximal wave speed goes to
-// *smax_out. The CTA has NW warps; each lane group takes R interfaces in R
-// rounds.
+// starts at cell `off` of arrays with component stride M, in the shape sh;
+// orders (nullable) points at the instance's interface 0; the tile's maximal
+// wave speed goes to *smax_out. lam_sm: dt / dx, published by the caller no
+// later than the staging barrier.
 template <int P, int FLUX, int NW = NT / 32, int R = 1>
-__device__ __forceinline__ void tile_f64(const Step1DArgs &a, Smem64<P, FLUX, NW, R> &sm,
+__device__ __forceinline__ void tile_f64(const Step1DArgs &a, Smem64<P, FLUX, NW, R> &sm, const Shape64 &sh,
                                          const double *__restrict__ uin, double *__restrict__ uout,
-                                         long off, long M, long N, long i0, double lam,
+                                         long off, long M, long N, long i0, const double *lam_sm,
                                          int8_t *orders, unsigned long long *smax_out) {
   using TL = typename Smem64<P, FLUX, NW, R>::TL;
-  constexpr int NTB = NW * 32;
   constexpr int S = Phys<FLUX>::S;
-  stage_f64<P, FLUX, NW, R>(a, sm, uin, off, M, N, i0, lam);
+  stage_f64<P, FLUX, NW, R>(a, sm, sh, uin, off, M, N, i0);
   __syncthreads();
+  const double lam = *lam_sm;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = sh.NT >> 5;
   const int grp = lane / TL::L, l = lane - grp * TL::L;
-  const FiltConst FC = filt_const(a.epsf, a.rf, a.factf);
-  reject_pass_f64<P, FLUX, NW, R>(a, sm, i0, N, FC);
+  reject_pass_f64<P, FLUX, NW, R>(a, sm, sh, i0, N, lam);
   if (P >= 2) __syncthreads();
 #pragma unroll 1
-  for (int rnd = 0; rnd < R; rnd++) {
+  for (int rnd = 0; rnd < sh.R; rnd++) {
     if (rnd > 0) __syncwarp();  // the exchange slots of the last round are read
-    const int il = (rnd * NW + warp) * TL::GPW + grp;
+    const int il = (rnd * nw + warp) * TL::GPW + grp;
     const long m = i0 + il;  // interface between cells m-1 and m
     if (grp < TL::GPW && m <= N &&
         acat_in_bounds(il - 1 + TL::GH - P + 1 >= 0 && il - 1 + TL::GH + P < TL::TW && il < TL::NI, a.status)) {
       const int ps = iface_f64<P, FLUX, NW, R>(a, sm, il, grp, l, warp, lam);
-      if (l == 0 && orders && (il < TL::T || m == N)) orders[m] = (int8_t)ps;
+      if (l == 0 && orders && (il < sh.NI - 1 || m == N)) orders[m] = (int8_t)ps;
     }
   }
   __syncthreads();
-  flux_finish_f64<P, FLUX, NW, R>(sm, i0, N);
+  flux_finish_f64<P, FLUX, NW, R>(sm, sh, i0, N);
 
   double smax = 0.0;
   bool bad = false;
-  for (int t = threadIdx.x; t < TL::T; t += NTB) {
+  for (int t = threadIdx.x; t < sh.NI - 1; t += sh.NT) {
     const long i = i0 + t;
     if (i >= N) break;
     if (!acat_in_bounds(t + 1 < TL::NI && t + TL::GH < TL::TW && off + i < M, a.status)) continue;
@@ -916,9 +931,8 @@ __device__ __forceinline__ void tile_f64(const Step1DArgs &a, Smem64<P, FLUX, NW
     smax = fmax(smax, sp);
   }
   if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(a.status, (unsigned)ACAT_STATUS_NONPHYSICAL);
-  const double v = block_max<NW>(smax, sm.red);
-  if (threadIdx.x == 0) atomic_max_pos(smax_out, v);
-  __syncthreads();
+  const double v = warp_max_pos(smax);
+  if (lane == 0 && warp * 32 < sh.NI - 1) atomic_max_pos(smax_out, v);
 }
 
 // Order selection and flux increment G of interface il of an FP32 tile, by
