@@ -150,6 +150,7 @@ struct Step2DArgs {
   float epsf, rf;
   float factf[ACAT_MAXP + 1];
   float advf[2], gammaf, gm1f;  // adv, gamma, gamma - 1 rounded to float (FP32 path)
+  float2 sgam, skap, somk, sgm1;  // as in Step1DArgs
   unsigned long long *smax;   // 3 slots x 2 directions: [slot][dir]
   double *tslot;              // 3 slots (nullable)
   int8_t *ord_x;              // NY x (NX+1) (nullable)

@@ -180,6 +180,7 @@ Step2DArgs base_args2(acat_ctx *c) {
   a.advf[1] = (float)p.adv[1];
   a.gammaf = (float)p.gamma;
   a.gm1f = (float)(p.gamma - 1.0);
+  acat_set_pairs(a);
   a.smax = c->d_smax;
   a.status = c->d_status;
   return a;

@@ -81,6 +81,34 @@ __device__ __forceinline__ double div_rn(double a, double b) { return __ddiv_rn(
 __device__ __forceinline__ float sqrt_rn(float a) { return __fsqrt_rn(a); }
 __device__ __forceinline__ double sqrt_rn(double a) { return __dsqrt_rn(a); }
 
+// The top 47 (pair, rounded) or all 53 bits (F3) of a double as floats, by
+// integer operations on its bits: conversions would occupy the FP64 pipe (64
+// cycles per warp each), and a record holds 21 of them. Parts carry the sign of
+// x; the parts after the first are 0 for |x| below 2^-75, all are below 2^-126,
+// and infinities, NaN and values beyond 2^127 give parts that are not finite.
+struct Bits64 {
+  unsigned hi, lo;  // the float bits of the top 24 bits; the low 29 bits of the mantissa
+  float ulp;        // +-2^(exponent - 52), the weight of the lowest mantissa bit
+};
+__device__ __forceinline__ Bits64 bits_of(double x) {
+  const unsigned h = (unsigned)__double2hiint(x), l = (unsigned)__double2loint(x);
+  const int e = (int)((h >> 20) & 0x7ffu) - 896;  // float exponent field
+  const unsigned s = h & 0x80000000u;
+  const unsigned mant = __funnelshift_l(l, h, 3) & 0x7fffffu;
+  Bits64 r;
+  const bool fin = e < 255, nz = e > 0;
+  r.hi = s | (nz ? (fin ? ((unsigned)e << 23) | mant : 0x7fffffffu) : 0u);
+  r.lo = nz ? l & 0x1fffffffu : 0u;
+  // 2^(e - 52 - 127), flushed to 0 below the normal range
+  r.ulp = __uint_as_float(s | (e > 52 ? (unsigned)(e - 52) << 23 : 0u));
+  return r;
+}
+// an integer up to 2^23 as a float
+__device__ __forceinline__ float small_float(unsigned n) {
+  return __fsub_rn(__uint_as_float(0x4b000000u + n), 8388608.0f);
+}
+__device__ __forceinline__ float f_bits(double x) { return __uint_as_float(bits_of(x).hi); }
+
 // fused multiply-add in the arithmetic type of its arguments
 __device__ __forceinline__ double fmar(double a, double b, double c) { return fma(a, b, c); }
 __device__ __forceinline__ float fmar(float a, float b, float c) { return fmaf(a, b, c); }
@@ -400,7 +428,9 @@ __device__ __forceinline__ unsigned reject_set(const float *d, const float *e, G
 }
 
 // reject_set of one component of an FP64 state, values at q[j*st],
-// j = -PM+1..PM.
+// j = -PM+1..PM. The differences are exact subtractions truncated to 24 bits by
+// integer operations (0 below 2^-126): conversions would cost the FP64 pipe as
+// much as the subtractions.
 template <int PM>
 __device__ __forceinline__ unsigned reject_set64(const double *q, int st, bool first, const FiltConst &F,
                                                  double eps, double thr, const double *fact, int psi2_mod) {
@@ -408,8 +438,8 @@ __device__ __forceinline__ unsigned reject_set64(const double *q, int st, bool f
 #pragma unroll
   for (int k = 0; k < 2 * PM - 1; k++) {
     const int j = k - PM + 1;
-    d[k] = (float)__dsub_rn(q[(j + 1) * st], q[j * st]);
-    e[k] = 6.0e-8f * fabsf(d[k]) + 1e-44f;
+    d[k] = f_bits(__dsub_rn(q[(j + 1) * st], q[j * st]));
+    e[k] = 1.2e-7f * fabsf(d[k]) + 1.2e-38f;
   }
   return reject_set<PM>(d, e, [=](int j) { return q[j * st]; }, first, F, eps, thr, fact, psi2_mod);
 }

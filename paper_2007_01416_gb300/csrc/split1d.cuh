@@ -72,37 +72,10 @@ __device__ __forceinline__ void ff_acc(FF &s, FF x, float g) {
   s.h = t.h;
   s.l = __fadd_rn(__fadd_rn(s.l, t.l), e);
 }
-// The top 47 (pair, rounded) or all 53 bits (F3) of a double as floats, by
-// integer operations on its bits: conversions would occupy the FP64 pipe (64
-// cycles per warp each), and a record holds 21 of them. Parts carry the sign of
-// x; the parts after the first are 0 for |x| below 2^-75, all are below 2^-126,
-// and infinities, NaN and values beyond 2^127 give parts that are not finite.
-struct Bits64 {
-  unsigned hi, lo;  // the float bits of the top 24 bits; the low 29 bits of the mantissa
-  float ulp;        // +-2^(exponent - 52), the weight of the lowest mantissa bit
-};
-__device__ __forceinline__ Bits64 bits_of(double x) {
-  const unsigned h = (unsigned)__double2hiint(x), l = (unsigned)__double2loint(x);
-  const int e = (int)((h >> 20) & 0x7ffu) - 896;  // float exponent field
-  const unsigned s = h & 0x80000000u;
-  const unsigned mant = __funnelshift_l(l, h, 3) & 0x7fffffu;
-  Bits64 r;
-  const bool fin = e < 255, nz = e > 0;
-  r.hi = s | (nz ? (fin ? ((unsigned)e << 23) | mant : 0x7fffffffu) : 0u);
-  r.lo = nz ? l & 0x1fffffffu : 0u;
-  // 2^(e - 52 - 127), flushed to 0 below the normal range
-  r.ulp = __uint_as_float(s | (e > 52 ? (unsigned)(e - 52) << 23 : 0u));
-  return r;
-}
-// an integer up to 2^23 as a float
-__device__ __forceinline__ float small_float(unsigned n) {
-  return __fsub_rn(__uint_as_float(0x4b000000u + n), 8388608.0f);
-}
 __device__ __forceinline__ FF ff_bits(double x) {
   const Bits64 b = bits_of(x);
   return FF{__uint_as_float(b.hi), __fmul_rn(small_float((b.lo + 32u) >> 6), __fmul_rn(64.0f, b.ulp))};
 }
-__device__ __forceinline__ float f_bits(double x) { return __uint_as_float(bits_of(x).hi); }
 __device__ __forceinline__ FF ff_of(float2 a) { return FF{a.x, a.y}; }
 
 // An FP64 value as three floats h + m + l (exact for values in float's range),

@@ -23,7 +23,7 @@
 // the 1D kernel: F = f(u_a) + G_F, G = g(u_a) + G_G about the anchor state.
 #include <type_traits>
 
-#include "device_common.cuh"
+#include "split2d.cuh"
 
 namespace {
 
@@ -70,10 +70,6 @@ struct Phys2<ACAT_FLUX_LINEAR> {
                                                      float *dg) {
     const float d[1] = {dh[0] + dl[0]};
     dflux2(B, d, df, dg);
-  }
-  __device__ static __forceinline__ void dflux2_x2(const Base &B, const float2 *d, float2 *df, float2 *dg) {
-    df[0] = f2mul(f2dup(B.ax), d[0]);
-    dg[0] = f2mul(f2dup(B.ay), d[0]);
   }
   __device__ static __forceinline__ float fspeed(const float *, float ax, float ay, float, int dir) {
     return dir == 0 ? fabsf(ax) : fabsf(ay);
@@ -193,26 +189,6 @@ struct Phys2<ACAT_FLUX_EULER2D> {
     dg[2] = dmw + dp;
     dg[3] = fmaf(dw, B.H, wn * dH);
   }
-  // the same for two increments packed in float2 lanes
-  __device__ static __forceinline__ void dflux2_x2(const Base &B, const float2 *d, float2 *df, float2 *dg) {
-    const float2 den = f2add(f2dup(B.rho), d[0]);
-    const float2 ri = make_float2(recip(den.x), recip(den.y));
-    const float2 dv = f2mul(f2fma(f2dup(-B.vl), d[0], f2fma(f2dup(-B.v), d[0], d[1])), ri);
-    const float2 dw = f2mul(f2fma(f2dup(-B.wl), d[0], f2fma(f2dup(-B.w), d[0], d[2])), ri);
-    const float2 vn = f2add(f2dup(B.v), dv), wn = f2add(f2dup(B.w), dw);
-    const float2 dmv = f2fma(f2dup(B.mx), dv, f2mul(d[1], vn)), dmw = f2fma(f2dup(B.my), dw, f2mul(d[2], wn));
-    const float2 dxy = f2fma(f2dup(B.mx), dw, f2mul(d[1], wn));
-    const float2 dp = f2mul(f2dup(B.gm1), f2fma(f2dup(-0.5f), f2add(dmv, dmw), d[3]));
-    const float2 dH = f2add(d[3], dp);
-    df[0] = d[1];
-    df[1] = f2add(dmv, dp);
-    df[2] = dxy;
-    df[3] = f2fma(dv, f2dup(B.H), f2mul(vn, dH));
-    dg[0] = d[2];
-    dg[1] = dxy;
-    dg[2] = f2add(dmw, dp);
-    dg[3] = f2fma(dw, f2dup(B.H), f2mul(wn, dH));
-  }
   __device__ static __forceinline__ float fspeed(const float *u, float, float, float gamma, int dir) {
     const float v = u[1] / u[0], w = u[2] / u[0];
     const float p = (gamma - 1.0f) * (u[3] - 0.5f * (u[1] * v + u[2] * w));
@@ -227,7 +203,115 @@ struct Phys2<ACAT_FLUX_EULER2D> {
 };
 
 // ---------------------------------------------------------------------------
-// FP64 block recursion (Eqs. 4.5-4.6) by 16 lanes; lane l <-> node
+// The increments f(u + d) - f(u), g(u + d) - g(u) split into Jacobian products
+// and remainders (closed forms, quadratic in d). The time weights are exact on
+// polynomials of degree <= 2p-1 in r and the Taylor sum of order k has degree
+// k-1, so one Jacobian product per order (lin) carries the linear part of all
+// time levels, and a level evaluates only the NR nonlinear terms (rem, from
+// the Taylor sums of the NX combinations X of U; rem2 two levels at once); add
+// puts their weighted sum over the levels into F and G. Euler:
+//   W = (bx - v a, by - w a), L = dH' - h a, (dv, dw) = W / (rho + a),
+//   Q11 = W1 dv, Q12 = W1 dw, Q22 = W2 dw, T = (dv, dw) (L - kappa (Q11 + Q22)):
+// 18 float instructions and one reciprocal per level, against 37 with the whole
+// increments of f and g.
+// ---------------------------------------------------------------------------
+template <int FLUX>
+struct RPhys2;
+
+template <>
+struct RPhys2<ACAT_FLUX_LINEAR> {
+  static constexpr int NX = 0, NR = 0;
+  struct Base {
+    float ax, ay;
+  };
+  __device__ static __forceinline__ Base base(const float *, const float *, float ax, float ay, float) {
+    return Base{ax, ay};
+  }
+  __device__ static __forceinline__ float init(const Base &, int) { return 0.0f; }
+  __device__ static __forceinline__ void lin(const Base &B, const float *U, float *, float *F, float *G) {
+    F[0] = B.ax * U[0];
+    G[0] = B.ay * U[0];
+  }
+  __device__ static __forceinline__ void rem(const Base &, const float *, float *) {}
+  __device__ static __forceinline__ void rem2(const Base &, const float2 *, float2 *) {}
+  __device__ static __forceinline__ void add(const Base &, const float *, const float *, float *, float *) {}
+};
+
+template <>
+struct RPhys2<ACAT_FLUX_EULER2D> {
+  static constexpr int NX = 4, NR = 5;
+  struct Base {
+    float rho, v, w, vl, wl, h, gm1, kap;  // v + vl, w + wl: float-float velocities (Phys2::base2)
+  };
+  __device__ static __forceinline__ Base base(const float *h, const float *l, float, float, float gm1) {
+    Base b;
+    b.rho = h[0];
+    const float ri = recip(h[0]);
+    b.v = h[1] * ri;
+    b.w = h[2] * ri;
+    b.vl = (fmaf(-b.v, h[0], h[1]) + fmaf(-b.v, l[0], l[1])) * ri;
+    b.wl = (fmaf(-b.w, h[0], h[2]) + fmaf(-b.w, l[0], l[2])) * ri;
+    const float p = gm1 * (h[3] - 0.5f * fmaf(h[1], b.v, h[2] * b.w));
+    b.h = (h[3] + p) * ri;
+    b.gm1 = gm1;
+    b.kap = 0.5f * gm1;
+    return b;
+  }
+  __device__ static __forceinline__ float init(const Base &B, int c) { return c == 0 ? B.rho : 0.0f; }
+  // F[1], G[2] hold the linear parts of d(mx v), d(my w) until add() forms the
+  // pressure increment
+  __device__ static __forceinline__ void lin(const Base &B, const float *U, float *X, float *F, float *G) {
+    const float W1 = fmaf(-B.vl, U[0], fmaf(-B.v, U[0], U[1])), W2 = fmaf(-B.wl, U[0], fmaf(-B.w, U[0], U[2]));
+    const float m1 = B.v * (U[1] + W1), m2 = B.w * (U[2] + W2);
+    const float Lp = fmaf(B.gm1, fmaf(-0.5f, m1 + m2, U[3]), U[3]);
+    X[0] = U[0];
+    X[1] = W1;
+    X[2] = W2;
+    X[3] = fmaf(-B.h, U[0], Lp);
+    F[0] = U[1];
+    F[1] = m1;
+    F[2] = fmaf(B.v, W2, B.w * U[1]);
+    F[3] = fmaf(B.v, Lp, B.h * W1);
+    G[0] = U[2];
+    G[2] = m2;
+    G[3] = fmaf(B.w, Lp, B.h * W2);
+  }
+  __device__ static __forceinline__ void rem(const Base &B, const float *X, float *R) {
+    const float ri = recip(X[0]);
+    const float dv = X[1] * ri, dw = X[2] * ri;
+    R[0] = X[1] * dv;
+    R[1] = X[1] * dw;
+    R[2] = X[2] * dw;
+    const float t = fmaf(-B.kap, R[0] + R[2], X[3]);
+    R[3] = dv * t;
+    R[4] = dw * t;
+  }
+  __device__ static __forceinline__ void rem2(const Base &B, const float2 *X, float2 *R) {
+    const float2 ri = make_float2(recip(X[0].x), recip(X[0].y));
+    const float2 dv = f2mul(X[1], ri), dw = f2mul(X[2], ri);
+    R[0] = f2mul(X[1], dv);
+    R[1] = f2mul(X[1], dw);
+    R[2] = f2mul(X[2], dw);
+    const float2 t = f2fma(f2dup(-B.kap), f2add(R[0], R[2]), X[3]);
+    R[3] = f2mul(dv, t);
+    R[4] = f2mul(dw, t);
+  }
+  __device__ static __forceinline__ void add(const Base &B, const float *U, const float *A, float *F, float *G) {
+    const float m1 = F[1] + A[0], m2 = G[2] + A[2];
+    const float dp = B.gm1 * fmaf(-0.5f, m1 + m2, U[3]);
+    const float kq = B.kap * (A[0] + A[2]);
+    F[1] = m1 + dp;
+    G[2] = m2 + dp;
+    F[2] += A[1];
+    G[1] = F[2];
+    F[3] += fmaf(-B.v, kq, A[3]);
+    G[3] += fmaf(-B.w, kq, A[4]);
+  }
+};
+
+// ---------------------------------------------------------------------------
+// FP64 block recursion (Eqs. 4.5-4.6) by 16 lanes (linear transport: F^(k-1) =
+// a U^(k-1) and no time levels); lane l <-> node
 // (a1, b1) = (l % n, l / n). q points at the anchor for component 0; `cs`
 // between components, `rs` between rows. Every lane returns F and G.
 // ---------------------------------------------------------------------------
@@ -283,9 +367,10 @@ __device__ __forceinline__ void cat2d_f64(const double *q, int cs, int rs, int l
       af[c] = TB::gk(p, k - 1, p - 1) * f0[c];
       ag[c] = TB::gk(p, k - 1, p - 1) * g0[c];
     }
+    if constexpr (FLUX == ACAT_FLUX_LINEAR) Phys2<FLUX>::flux2(U, af, ag, ax, ay, gm1);
 #pragma unroll
     for (int rr = 0; rr < n; rr++) {
-      if (rr == p - 1) continue;
+      if (FLUX == ACAT_FLUX_LINEAR || rr == p - 1) continue;
       const double cr = TB::taylor(p, rr, k - 1), wk = TB::gk(p, k - 1, rr);
       double fr[S], gr[S];
 #pragma unroll
@@ -354,21 +439,24 @@ __device__ __forceinline__ void cat2d_f32(const float *hi, const float *lo, int 
   }
   float Df[S], Dg[S];
   PH::dflux2_pair(PH::base2(ua, ual, ax, ay, gm1), dh, dl, Df, Dg);  // f(u_j) - f(u_a), g(u_j) - g(u_a)
-  const typename PH::Base bj = PH::base2(uj, ujl, ax, ay, gm1);
+  using RP = RPhys2<FLUX>;
+  const typename RP::Base bj = RP::base(uj, ujl, ax, ay, gm1);
   // the 2p - 1 levels r != 0 in pairs packed in float2 lanes, the last alone
-  constexpr int NL = n - 1, NP = NL / 2;
-  float Ff[S], Fg[S], Pf[S], Pg[S], dels[S];
-  float2 del2[NP][S];
+  constexpr int NL = n - 1, NP = NL / 2, NX = RP::NX, NR = RP::NR;
+  constexpr int NXA = NX > 0 ? NX : 1, NRA = NR > 0 ? NR : 1;
+  float Ff[S], Fg[S], Pf[S], Pg[S], xs1[NXA];
+  float2 xs2[NP][NXA];
 #pragma unroll
   for (int c = 0; c < S; c++) {
     Ff[c] = Pf[c] = Df[c];
     Fg[c] = Pg[c] = Dg[c];
-    dels[c] = 0.0f;
   }
 #pragma unroll
-  for (int q = 0; q < NP; q++)
+  for (int c = 0; c < NX; c++) {
+    xs1[c] = RP::init(bj, c);
 #pragma unroll
-    for (int c = 0; c < S; c++) del2[q][c] = make_float2(0.0f, 0.0f);
+    for (int q = 0; q < NP; q++) xs2[q][c] = f2dup(RP::init(bj, c));
+  }
 #pragma unroll
   for (int k = 2; k <= n; k++) {
     float Ux[S], Uy[S];
@@ -399,51 +487,40 @@ __device__ __forceinline__ void cat2d_f32(const float *hi, const float *lo, int 
         Uy[0] = fmaf(gy[r], __shfl_sync(mask, Pg[0], base + r * n + a1), Uy[0]);
       }
     }
-    float U[S], af[S], ag[S];
+    float U[S], X[NXA], A[NRA];
+    float2 A2[NRA];
 #pragma unroll
-    for (int c = 0; c < S; c++) {
-      U[c] = -(lx * Ux[c]) - ly * Uy[c];
-      af[c] = ag[c] = 0.0f;
-    }
-    float2 af2[S], ag2[S];
+    for (int c = 0; c < S; c++) U[c] = -(lx * Ux[c]) - ly * Uy[c];
+    RP::lin(bj, U, X, Pf, Pg);
 #pragma unroll
-    for (int c = 0; c < S; c++) af2[c] = ag2[c] = make_float2(0.0f, 0.0f);
+    for (int c = 0; c < NR; c++) A2[c] = make_float2(0.0f, 0.0f);
+    if constexpr (NX > 0) {
 #pragma unroll
-    for (int q = 0; q < NP; q++) {
-      const int ra = 2 * q < p - 1 ? 2 * q : 2 * q + 1, rb = 2 * q + 1 < p - 1 ? 2 * q + 1 : 2 * q + 2;
-      const float2 cr = make_float2(TB::taylor(p, ra, k - 1), TB::taylor(p, rb, k - 1));
-      const float2 wk = make_float2(TB::gk(p, k - 1, ra), TB::gk(p, k - 1, rb));
-      float2 ef[S], eg[S];
+      for (int q = 0; q < NP; q++) {
+        const int ra = 2 * q < p - 1 ? 2 * q : 2 * q + 1, rb = 2 * q + 1 < p - 1 ? 2 * q + 1 : 2 * q + 2;
+        const float2 cr = make_float2(TB::taylor(p, ra, k - 1), TB::taylor(p, rb, k - 1));
+        const float2 wk = make_float2(TB::gk(p, k - 1, ra), TB::gk(p, k - 1, rb));
+        float2 R2[NRA];
 #pragma unroll
-      for (int c = 0; c < S; c++) del2[q][c] = f2fma(cr, f2dup(U[c]), del2[q][c]);
-      PH::dflux2_x2(bj, del2[q], ef, eg);
+        for (int c = 0; c < NX; c++) xs2[q][c] = f2fma(cr, f2dup(X[c]), xs2[q][c]);
+        RP::rem2(bj, xs2[q], R2);
 #pragma unroll
-      for (int c = 0; c < S; c++) {
-        af2[c] = f2fma(wk, ef[c], af2[c]);
-        ag2[c] = f2fma(wk, eg[c], ag2[c]);
+        for (int c = 0; c < NR; c++) A2[c] = f2fma(wk, R2[c], A2[c]);
       }
-    }
-    {
       constexpr int rs = NL - 1 < p - 1 ? NL - 1 : NL;  // the last level
       const float cr = TB::taylor(p, rs, k - 1), wk = TB::gk(p, k - 1, rs);
-      float ef[S], eg[S];
+      float R1[NRA];
 #pragma unroll
-      for (int c = 0; c < S; c++) dels[c] = fmaf(cr, U[c], dels[c]);
-      PH::dflux2(bj, dels, ef, eg);
+      for (int c = 0; c < NX; c++) xs1[c] = fmaf(cr, X[c], xs1[c]);
+      RP::rem(bj, xs1, R1);
 #pragma unroll
-      for (int c = 0; c < S; c++) {
-        af[c] = fmaf(wk, ef[c], af[c]);
-        ag[c] = fmaf(wk, eg[c], ag[c]);
-      }
+      for (int c = 0; c < NR; c++) A[c] = fmaf(wk, R1[c], A2[c].x + A2[c].y);
     }
+    RP::add(bj, U, A, Pf, Pg);
 #pragma unroll
     for (int c = 0; c < S; c++) {
-      af[c] += af2[c].x + af2[c].y;
-      ag[c] += ag2[c].x + ag2[c].y;
-      Pf[c] = af[c];
-      Pg[c] = ag[c];
-      Ff[c] = fmaf(TB::invfact(k), af[c], Ff[c]);
-      Fg[c] = fmaf(TB::invfact(k), ag[c], Fg[c]);
+      Ff[c] = fmaf(TB::invfact(k), Pf[c], Ff[c]);
+      Fg[c] = fmaf(TB::invfact(k), Pg[c], Fg[c]);
     }
   }
 #pragma unroll
@@ -933,6 +1010,233 @@ __global__ void __launch_bounds__(NT, F32 ? 3 : (FLUX == ACAT_FLUX_LINEAR ? 3 : 
   }
 }
 
+// ---------------------------------------------------------------------------
+// 2D Euler FP64 step at P = 2: k_step2d's tiling with the block recursion in
+// float-float pairs (split2d.cuh). The cells' records are formed once per tile;
+// a block whose increments are too large for the pairs falls back to
+// cat2d_f64. 83 KB of dynamic shared memory, 2 CTAs per SM.
+// ---------------------------------------------------------------------------
+struct Smem2S {
+  double tile[4][TW2][TW2];
+  double Fx[TXY][TXY + 1][4];  // fluxes; a float pair G until the finish pass
+  double Gy[TXY + 1][TXY][4];
+  Split2Rec rec[TW2 * TW2];
+  float4 x[NT / 32][4][32];    // the warps' exchange slots
+  SplitLam lx, ly;
+  double dlx, dly;
+  unsigned char rej[8 * NA * NA];
+  unsigned char cF[TXY][TXY + 1], cG[TXY + 1][TXY];  // 2 where the flux is a pair
+};
+
+// The recursion of one anchor by 16 lanes. Lane l < 8 returns the flux sum of
+// direction l >> 2, component l & 3; the result is false (for all 16 lanes) when
+// the pairs do not hold.
+__device__ __forceinline__ bool cat2d_split(Smem2S &sm, const Step2DArgs &a, int cell, int l, int base, int warp,
+                                            FF &S) {
+  constexpr int p = 2, n = 4;
+  const unsigned mask = 0xffffu << base;
+  const int ia = l & 3, ib = l >> 2;
+  const Split2Const C = split2_const(a);
+  const Split2Slots xs{sm.x[warp][0], sm.x[warp][1], sm.x[warp][2], sm.x[warp][3]};
+  float gx[n], gy[n];
+#pragma unroll
+  for (int r = 0; r < n; r++) {
+    gx[r] = c_tab.g1i[p][ia][r];
+    gy[r] = c_tab.g1i[p][ib][r];
+  }
+  const int i0 = base + ib * n, j0 = base + ia;
+  const int dir = (l >> 2) & 1, fc = l & 3, f0 = dir ? base + p - 1 : base + (p - 1) * n, fs = dir ? n : 1;
+  bool allow = true;
+#pragma unroll 1
+  for (;;) {
+    Split2Node<p> N;
+    FF F[4], G[4];
+    const bool ok = split2_start(C, sm.rec[cell + (ib - p + 1) * TW2 + ia - p + 1], sm.rec[cell], N, F, G);
+    if (!__all_sync(mask, ok)) return false;
+    __syncwarp(mask);
+    split2_put(xs, base + l, F, G);
+    __syncwarp(mask);
+    S = FF{0.0f, 0.0f};
+    if (l < 8) split2_flux<p>(xs, dir, fc, f0, fs, 840.0f, S);
+    bool flt = allow, tail = false;
+#pragma unroll 1
+    for (int k = 2; k <= n; k++) {
+      const float2 lx = sm.lx.v[0][k - 2], ly = sm.ly.v[0][k - 2];
+      if (!tail && flt) tail = __all_sync(mask, split2_small(N, F, G));
+      if (tail) {
+        split2_tail(C, N, k, xs, i0, j0, n, gx, gy, lx.x, ly.x, F, G);
+      } else {
+        FF u[4];
+        split2_sums<p>(xs, i0, j0, n, gx, gy, ff_of(lx), ff_of(ly), u);
+        const Split2Lin o = split2_lin(C, N.v, N.w, N.h, u);
+        const float pk = c_tab.powr[p][n - 1][k - 1];
+        N.Ba = fmaf(pk, fabsf(u[0].h), N.Ba);
+        N.Bw = fmaf(pk, fmaxf(fabsf(o.W1.h), fabsf(o.W2.h)), N.Bw);
+        N.Bl = fmaf(pk, fabsf(o.L.h), N.Bl);
+        if (k == 2 && flt) flt = __all_sync(mask, split2_quad(N, 2.0f));
+        split2_order(C, N, k, flt, u, o, F, G);
+      }
+      __syncwarp(mask);
+      split2_put(xs, base + l, F, G);
+      __syncwarp(mask);
+      if (l < 8) split2_flux<p>(xs, dir, fc, f0, fs, c_tab.k840[k], S);
+    }
+    if (!__all_sync(mask, split2_held(N))) return false;
+    if (!flt || __all_sync(mask, split2_quad(N, 1.0f))) break;
+    allow = false;
+  }
+  return true;
+}
+
+__global__ void __launch_bounds__(NT, 2) k_step2d_split(const Step2DArgs a) {
+  constexpr int FLUX = ACAT_FLUX_EULER2D, P = 2, S = 4, CELLS = TW2 * TW2, RS = TW2;
+  using PH = Phys2<FLUX>;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  Smem2S &sm = *reinterpret_cast<Smem2S *>(smem_raw);
+  const long NXl = a.NX, NYl = a.NY;
+  const long x0 = (long)blockIdx.x * TXY, y0 = (long)blockIdx.y * TXY;
+  if (threadIdx.x == NT - 32) {
+    const double dt = step_dt2(a);
+    sm.dlx = dt / a.dx;
+    sm.dly = dt / a.dy;
+  }
+  const double gm1 = a.gamma - 1.0;
+  for (int q = threadIdx.x; q < CELLS; q += NT) {
+    const int yy = q / TW2, xx = q - yy * TW2;
+    const long gx = bc2(x0 - GH2 + xx, NXl, a.bc), gy = bc2(y0 - GH2 + yy, NYl, a.bc);
+    if (!acat_in_bounds(gx >= 0 && gx < NXl && gy >= 0 && gy < NYl, a.status)) continue;
+    double u[S];
+#pragma unroll
+    for (int c = 0; c < S; c++) {
+      u[c] = static_cast<const double *>(a.u_in)[((long)c * NYl + gy) * NXl + gx];
+      sm.tile[c][yy][xx] = u[c];
+    }
+    split2_record(sm.rec[q], u, gm1);
+  }
+  for (int q = threadIdx.x; q < 2 * TXY * (TXY + 1); q += NT) (&sm.cF[0][0])[q] = 0;  // cF and cG
+  __syncthreads();
+  const double lxd = sm.dlx, lyd = sm.dly;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int grp = lane >> 4, l = lane & 15, base = grp * 16;
+  if (warp == 0) {
+    split_lam(sm.lx, lxd, lane);
+    split_lam(sm.ly, lyd, lane);
+  }
+  const FiltConst FC = filt_const(a.epsf, a.rf, a.factf);
+  for (int q = threadIdx.x; q < 2 * S * NA * NA; q += NT) {
+    const int dc = q / (NA * NA), an = q - dc * NA * NA, dir = dc / S, c = dc - dir * S;
+    const int ax = an % NA - 1, ay = an / NA - 1;
+    const bool inside = x0 + ax < NXl && y0 + ay < NYl;
+    unsigned r = 0;
+    if (inside && (dir == 0 ? ay >= 0 : ax >= 0))
+      r = reject_set64<P>(&sm.tile[c][ay + GH2][ax + GH2], dir == 0 ? 1 : RS, c == 0, FC, a.eps, a.thr, a.fact_tau,
+                          a.psi2_mod);
+    sm.rej[q] = (unsigned char)r;
+  }
+  __syncthreads();
+#pragma unroll 1
+  for (int round = 0; round < NA * NA / 16; round++) {
+    const int an = round * 16 + warp * 2 + grp;
+    const int ax = an % NA - 1, ay = an / NA - 1;  // anchor relative to (x0, y0)
+    const long gxa = x0 + ax, gya = y0 + ay;
+    const bool inside = gxa < NXl && gya < NYl;
+    const bool needF = inside && ay >= 0, needG = inside && ax >= 0;
+    const int cell = (ay + GH2) * TW2 + ax + GH2;
+    const double *q64 = &sm.tile[0][ay + GH2][ax + GH2];
+    unsigned rx = 0, ry = 0;
+#pragma unroll
+    for (int c = 0; c < S; c++) {
+      rx |= sm.rej[c * NA * NA + an];
+      ry |= sm.rej[(S + c) * NA * NA + an];
+    }
+    const int px = rx & 1u ? 1 : 2, py = ry & 1u ? 1 : 2;
+    const bool blkF = needF && px == 2, blkG = needG && py == 2;
+    if (blkF || blkG) {
+      FF s;
+      if (cat2d_split(sm, a, cell, l, base, warp, s)) {
+        const int c = l & 3;
+        if (l < 4 && blkF) *reinterpret_cast<float2 *>(&sm.Fx[ay][ax + 1][c]) = make_float2(s.h, s.l);
+        if (l >= 4 && l < 8 && blkG) *reinterpret_cast<float2 *>(&sm.Gy[ay + 1][ax][c]) = make_float2(s.h, s.l);
+        if (l == 0 && blkF) sm.cF[ay][ax + 1] = 2;
+        if (l == 0 && blkG) sm.cG[ay + 1][ax] = 2;
+      } else {
+        double F[S], G[S];
+        cat2d_f64<2, FLUX>(q64, CELLS, RS, l, base, lxd, lyd, a.adv[0], a.adv[1], gm1, F, G);
+        if (l == 0) {
+#pragma unroll
+          for (int c = 0; c < S; c++) {
+            if (blkF) sm.Fx[ay][ax + 1][c] = F[c];
+            if (blkG) sm.Gy[ay + 1][ax][c] = G[c];
+          }
+        }
+      }
+    }
+    const bool flF = needF && !blkF, flG = needG && !blkG;
+    if (l == 0) {
+      if (flF || flG) {
+        double F1[S], G1[S];
+        flcat2_2d_f64<FLUX>(q64, CELLS, RS, flF, flG, lxd, lyd, a.adv[0], a.adv[1], a.gamma, a.limiter_form,
+                            a.lo_flux, F1, G1);
+#pragma unroll
+        for (int c = 0; c < S; c++) {
+          if (flF) sm.Fx[ay][ax + 1][c] = F1[c];
+          if (flG) sm.Gy[ay + 1][ax][c] = G1[c];
+        }
+      }
+      if (needF && a.ord_x && (ax >= 0 || gxa == -1)) a.ord_x[gya * (NXl + 1) + (gxa + 1)] = (int8_t)px;
+      if (needG && a.ord_y && (ay >= 0 || gya == -1)) a.ord_y[(gya + 1) * NXl + gxa] = (int8_t)py;
+    }
+  }
+  __syncthreads();
+  // pairs to fluxes: F = f(u_a) + G
+  for (int q = threadIdx.x; q < 2 * TXY * (TXY + 1); q += NT) {
+    if ((&sm.cF[0][0])[q] == 0) continue;
+    const int d = q / (TXY * (TXY + 1)), e = q - d * TXY * (TXY + 1);
+    const int yy = d ? e / TXY - 1 : e / (TXY + 1), xx = d ? e % TXY : e % (TXY + 1) - 1;
+    double u[S], f[S], g[S];
+#pragma unroll
+    for (int c = 0; c < S; c++) u[c] = sm.tile[c][yy + GH2][xx + GH2];
+    PH::flux2(u, f, g, 0.0, 0.0, gm1);
+    double *o = d ? sm.Gy[yy + 1][xx] : sm.Fx[yy][xx + 1];
+#pragma unroll
+    for (int c = 0; c < S; c++) {
+      const float2 t = *reinterpret_cast<const float2 *>(&o[c]);
+      o[c] = fma(__dadd_rn((double)t.x, (double)t.y), split_ginv(2), d ? g[c] : f[c]);
+    }
+  }
+  __syncthreads();
+  // update and wave-speed epilogue
+  double mx = 0.0, my = 0.0;
+  bool bad = false;
+  for (int t = threadIdx.x; t < TXY * TXY; t += NT) {
+    const int cy = t / TXY, cx = t - cy * TXY;
+    const long gx = x0 + cx, gy = y0 + cy;
+    if (gx >= NXl || gy >= NYl) continue;
+    double un[S];
+    double *uo = static_cast<double *>(a.u_out);
+#pragma unroll
+    for (int c = 0; c < S; c++) {
+      un[c] = sm.tile[c][cy + GH2][cx + GH2] + lxd * (sm.Fx[cy][cx][c] - sm.Fx[cy][cx + 1][c]) +
+              lyd * (sm.Gy[cy][cx][c] - sm.Gy[cy + 1][cx][c]);
+      uo[((long)c * NYl + gy) * NXl + gx] = un[c];
+    }
+    double sx, sy;
+    bool ok;
+    PH::speed2(un, a.adv[0], a.adv[1], a.gamma, sx, sy, ok);
+    bad |= !ok;
+    mx = fmax(mx, sx);
+    my = fmax(my, sy);
+  }
+  if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(a.status, (unsigned)ACAT_STATUS_NONPHYSICAL);
+  mx = warp_max_pos(mx);
+  my = warp_max_pos(my);
+  if (lane == 0) {
+    const int z = (a.slot + 1) % 3;
+    atomic_max_pos(&a.smax[z * 2 + 0], mx);
+    atomic_max_pos(&a.smax[z * 2 + 1], my);
+  }
+}
+
 template <int FLUX, bool F32>
 __global__ void __launch_bounds__(NT) k_smax2d(const Step2DArgs a) {
   constexpr int S = Phys2<FLUX>::S;
@@ -1005,10 +1309,21 @@ template <int P, int FLUX>
 struct Smem2H {
   static constexpr int S = Phys2<FLUX>::S;
   static constexpr int TW = TXH + 2 * P;
+  static constexpr bool kSplit = FLUX == ACAT_FLUX_EULER2D;
   double tile[S][TW][TW];
-  double Fx[TXH][TXH + 1][S];
+  double Fx[TXH][TXH + 1][S];  // fluxes; a float pair G until the finish pass
   double Gy[TXH + 1][TXH][S];
-  double X[NT][S], Y[NT][S];  // F^(k), G^(k) of the nodes of a round
+  // F^(k), G^(k) of the nodes of a round (FP64, or float pairs)
+  union {
+    struct {
+      double X[NT][S], Y[NT][S];
+    };
+    float4 x4[kSplit ? 4 : 1][kSplit ? NT : 1];
+  };
+  Split2Rec rec[kSplit ? TW * TW : 1];
+  SplitLam slx, sly;
+  unsigned char cF[TXH][TXH + 1], cG[TXH + 1][TXH];  // p where the flux is a pair, else 0
+  int bad[NT / 16], nfail;
   unsigned rej[NAH * NAH];    // rejected orders: bit dir * (P - 1) + (p - 2)
   unsigned short task[P + 1][2 * NAH * NAH];
   int ntask[P + 1];
@@ -1088,9 +1403,10 @@ __device__ __forceinline__ void block_tasks(Smem2H<P, FLUX> &sm, const Step2DArg
           af[c] = TB::gk(p, k - 1, z) * f0[c];
           ag[c] = TB::gk(p, k - 1, z) * g0[c];
         }
+        if constexpr (FLUX == ACAT_FLUX_LINEAR) PH::flux2(U, af, ag, axv, ayv, gm1);
 #pragma unroll
         for (int rr = 0; rr < n; rr++) {
-          if (rr == z) continue;
+          if (FLUX == ACAT_FLUX_LINEAR || rr == z) continue;
           const double cr = TB::taylor(p, rr, k - 1), wk = TB::gk(p, k - 1, rr);
           double fr[S], gr[S];
 #pragma unroll
@@ -1222,9 +1538,10 @@ __device__ __forceinline__ void rect_tasks(Smem2H<P, FLUX> &sm, const Step2DArgs
           af[c] = TB::gk(pm, k - 1, zt) * f0[c];
           ag[c] = TB::gk(pm, k - 1, zt) * g0[c];
         }
+        if constexpr (FLUX == ACAT_FLUX_LINEAR) PH::flux2(U, af, ag, axv, ayv, gm1);
 #pragma unroll
         for (int rr = 0; rr < NM; rr++) {
-          if (rr >= n || rr == zt) continue;
+          if (FLUX == ACAT_FLUX_LINEAR || rr >= n || rr == zt) continue;
           const double cr = TB::taylor(pm, rr, k - 1), wk = TB::gk(pm, k - 1, rr);
           double fr[S], gr[S];
 #pragma unroll
@@ -1274,17 +1591,120 @@ __device__ __forceinline__ void rect_tasks(Smem2H<P, FLUX> &sm, const Step2DArgs
   }
 }
 
+// The block tasks of order p in float-float pairs (split2d.cuh), one thread per
+// node, NT / (2p)^2 tasks per round. The choices of precision are those of the
+// round (one vote of the CTA with the barriers that the exchange needs anyway);
+// the tasks whose increments are too large for the pairs are left in
+// sm.task[p][0 .. ntask) for block_tasks, the FP64 recursion.
+template <int p, int P, int FLUX>
+__device__ __forceinline__ void split_tasks(Smem2H<P, FLUX> &sm, const Step2DArgs &a) {
+  constexpr int n = 2 * p, nn = n * n, per = NT / nn, z = p - 1, TW = Smem2H<P, FLUX>::TW;
+  const int nt = sm.ntask[p];
+  const int tid = threadIdx.x, ti = tid / nn, node = tid - ti * nn;
+  const int ia = node % n, ib = node / n;
+  const Split2Const C = split2_const(a);
+  const Split2Slots xs{sm.x4[0], sm.x4[1], sm.x4[2], sm.x4[3]};
+  float gx[n], gy[n];
+#pragma unroll
+  for (int r = 0; r < n; r++) {
+    gx[r] = c_tab.g1i[p][ia][r];
+    gy[r] = c_tab.g1i[p][ib][r];
+  }
+  const int i0 = ti * nn + ib * n, j0 = ti * nn + ia;
+  const int dir = (node >> 2) & 1, fc = node & 3, f0 = ti * nn + (dir ? z : z * n), fs = dir ? n : 1;
+  if (tid == 0) sm.nfail = 0;
+#pragma unroll 1
+  for (int base = 0; base < nt; base += per) {
+    const bool act = ti < per && base + ti < nt;
+    const unsigned tk = act ? sm.task[p][base + ti] : 0u;
+    const int an = (int)(tk & 0xffu);
+    const int ax = an % NAH - 1, ay = an / NAH - 1;
+    bool allow = true;
+    FF S;
+#pragma unroll 1
+    for (;;) {
+      if (tid < per) sm.bad[tid] = 0;
+      __syncthreads();
+      Split2Node<p> N;
+      FF F[4], G[4];
+      if (act) {
+        const int tx = acat_tile_index(ax + P - p + 1 + ia, TW, a.status);
+        const int ty = acat_tile_index(ay + P - p + 1 + ib, TW, a.status);
+        if (!split2_start(C, sm.rec[ty * TW + tx], sm.rec[(ay + P) * TW + ax + P], N, F, G)) sm.bad[ti] = 1;
+        split2_put(xs, tid, F, G);
+      }
+      __syncthreads();
+      const bool off = !act || sm.bad[ti] != 0;  // no say in the round's votes
+      S = FF{0.0f, 0.0f};
+      if (act && node < 8) split2_flux<p>(xs, dir, fc, f0, fs, 840.0f, S);
+      bool flt = allow, tail = false;
+#pragma unroll 1
+      for (int k = 2; k <= n; k++) {
+        const float2 lx = sm.slx.v[p - 2][k - 2], ly = sm.sly.v[p - 2][k - 2];
+        if (!tail && flt) tail = __syncthreads_and(off || split2_small(N, F, G)) != 0;
+        if (tail) {
+          if (act) split2_tail(C, N, k, xs, i0, j0, n, gx, gy, lx.x, ly.x, F, G);
+        } else {
+          FF u[4];
+          Split2Lin o;
+          if (act) {
+            split2_sums<p>(xs, i0, j0, n, gx, gy, ff_of(lx), ff_of(ly), u);
+            o = split2_lin(C, N.v, N.w, N.h, u);
+            const float pk = c_tab.powr[p][n - 1][k - 1];
+            N.Ba = fmaf(pk, fabsf(u[0].h), N.Ba);
+            N.Bw = fmaf(pk, fmaxf(fabsf(o.W1.h), fabsf(o.W2.h)), N.Bw);
+            N.Bl = fmaf(pk, fabsf(o.L.h), N.Bl);
+          }
+          if (k == 2 && flt) flt = __syncthreads_and(off || split2_quad(N, 2.0f)) != 0;
+          if (act) split2_order(C, N, k, flt, u, o, F, G);
+        }
+        __syncthreads();
+        if (act) split2_put(xs, tid, F, G);
+        __syncthreads();
+        if (act && node < 8) split2_flux<p>(xs, dir, fc, f0, fs, c_tab.k840[k], S);
+      }
+      if (!off && !split2_held(N)) sm.bad[ti] = 1;
+      // (off is the state before this order's verdict: a block that fails here
+      // has no say in whether the round repeats)
+      if (!flt || __syncthreads_and(off || !split2_held(N) || split2_quad(N, 1.0f))) break;
+      allow = false;
+    }
+    __syncthreads();
+    if (act) {
+      if (sm.bad[ti]) {
+        if (node == 0) sm.task[p][atomicAdd(&sm.nfail, 1)] = (unsigned short)tk;  // below base + per: read already
+      } else if (node < 8) {
+        const float2 v = make_float2(S.h, S.l);
+        if (dir == 0 && (tk & WANT_F)) {
+          *reinterpret_cast<float2 *>(&sm.Fx[ay][ax + 1][fc]) = v;
+          if (fc == 0) sm.cF[ay][ax + 1] = (unsigned char)p;
+        }
+        if (dir == 1 && (tk & WANT_G)) {
+          *reinterpret_cast<float2 *>(&sm.Gy[ay + 1][ax][fc]) = v;
+          if (fc == 0) sm.cG[ay + 1][ax] = (unsigned char)p;
+        }
+      }
+    }
+    __syncthreads();
+  }
+  __syncthreads();
+  if (tid == 0) sm.ntask[p] = sm.nfail;
+  __syncthreads();
+}
+
 template <int P, int FLUX>
 __global__ void __launch_bounds__(NT, 1) k_step2d_hi(const Step2DArgs a) {
   using PH = Phys2<FLUX>;
   constexpr int S = PH::S;
   constexpr int TW = Smem2H<P, FLUX>::TW;
   constexpr int CELLS = TW * TW;
-  __shared__ Smem2H<P, FLUX> sm;
+  using SM = Smem2H<P, FLUX>;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  SM &sm = *reinterpret_cast<SM *>(smem_raw);
   const int tid = threadIdx.x;
   const long NXl = a.NX, NYl = a.NY;
   const long x0 = (long)blockIdx.x * TXH, y0 = (long)blockIdx.y * TXH;
-  if (tid == 0) {
+  if (tid == NT - 32) {
     const double dt = step_dt2(a);
     sm.lx = dt / a.dx;
     sm.ly = dt / a.dy;
@@ -1293,14 +1713,28 @@ __global__ void __launch_bounds__(NT, 1) k_step2d_hi(const Step2DArgs a) {
   if (tid == 0) sm.nrtask = 0;
   for (int q = tid; q < NAH * NAH; q += NT) sm.rej[q] = 0u;
   const double *uin = static_cast<const double *>(a.u_in);
-  for (int q = tid; q < S * CELLS; q += NT) {
-    const int c = q / CELLS, rem = q - c * CELLS, yy = rem / TW, xx = rem - yy * TW;
+  for (int q = tid; q < CELLS; q += NT) {
+    const int yy = q / TW, xx = q - yy * TW;
     const long gx = bc2(x0 - P + xx, NXl, a.bc), gy = bc2(y0 - P + yy, NYl, a.bc);
     if (!acat_in_bounds(gx >= 0 && gx < NXl && gy >= 0 && gy < NYl, a.status)) continue;
-    sm.tile[c][yy][xx] = uin[((long)c * NYl + gy) * NXl + gx];
+    double u[S];
+#pragma unroll
+    for (int c = 0; c < S; c++) {
+      u[c] = uin[((long)c * NYl + gy) * NXl + gx];
+      sm.tile[c][yy][xx] = u[c];
+    }
+    if constexpr (SM::kSplit) split2_record(sm.rec[q], u, a.gamma - 1.0);
   }
+  if constexpr (SM::kSplit)
+    for (int q = tid; q < 2 * TXH * (TXH + 1); q += NT) (&sm.cF[0][0])[q] = 0;  // cF and cG
   __syncthreads();
   const double lx = sm.lx, ly = sm.ly;
+  if constexpr (SM::kSplit) {
+    if (tid < 32) {
+      split_lam(sm.slx, lx, tid);
+      split_lam(sm.sly, ly, tid);
+    }
+  }
   // --- order decisions of every (anchor, direction, p, component) ----------
   constexpr int NPAIR = 2 * S;  // (direction, component): every order p = 2..P at once
   const FiltConst FC = filt_const(a.epsf, a.rf, a.factf);
@@ -1354,10 +1788,34 @@ __global__ void __launch_bounds__(NT, 1) k_step2d_hi(const Step2DArgs a) {
   }
   __syncthreads();
   // --- block recursions, one order at a time ------------------------------
+  if constexpr (SM::kSplit) {
+    split_tasks<2, P, FLUX>(sm, a);
+    if constexpr (P >= 3) split_tasks<3, P, FLUX>(sm, a);
+    if constexpr (P >= 4) split_tasks<4, P, FLUX>(sm, a);
+  }
   block_tasks<2, P, FLUX>(sm, a, lx, ly);
   if constexpr (P >= 3) block_tasks<3, P, FLUX>(sm, a, lx, ly);
   if constexpr (P >= 4) block_tasks<4, P, FLUX>(sm, a, lx, ly);
   if (a.rect_2d) rect_tasks<P, FLUX>(sm, a, lx, ly);
+  if constexpr (SM::kSplit) {  // pairs to fluxes: F = f(u_a) + G
+    for (int q = tid; q < 2 * TXH * (TXH + 1); q += NT) {
+      const int p = (&sm.cF[0][0])[q];
+      if (p == 0) continue;
+      const int d = q / (TXH * (TXH + 1)), e = q - d * TXH * (TXH + 1);
+      const int yy = d ? e / TXH - 1 : e / (TXH + 1), xx = d ? e % TXH : e % (TXH + 1) - 1;
+      double u[S], f[S], g[S];
+#pragma unroll
+      for (int c = 0; c < S; c++) u[c] = sm.tile[c][yy + P][xx + P];
+      PH::flux2(u, f, g, 0.0, 0.0, a.gamma - 1.0);
+      double *o = d ? sm.Gy[yy + 1][xx] : sm.Fx[yy][xx + 1];
+#pragma unroll
+      for (int c = 0; c < S; c++) {
+        const float2 t = *reinterpret_cast<const float2 *>(&o[c]);
+        o[c] = fma(__dadd_rn((double)t.x, (double)t.y), split_ginv(p), d ? g[c] : f[c]);
+      }
+    }
+    __syncthreads();
+  }
   // --- update and wave-speed epilogue (Eq. 4.9) ---------------------------
   double mx = 0.0, my = 0.0;
   bool bad = false;
@@ -1382,11 +1840,8 @@ __global__ void __launch_bounds__(NT, 1) k_step2d_hi(const Step2DArgs a) {
   }
   const int lane = tid & 31;
   if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(a.status, (unsigned)ACAT_STATUS_NONPHYSICAL);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    my = fmax(my, __shfl_xor_sync(0xffffffffu, my, o));
-  }
+  mx = warp_max_pos(mx);
+  my = warp_max_pos(my);
   if (lane == 0) {
     const int zs = (a.slot + 1) % 3;
     atomic_max_pos(&a.smax[zs * 2 + 0], mx);
@@ -1394,10 +1849,22 @@ __global__ void __launch_bounds__(NT, 1) k_step2d_hi(const Step2DArgs a) {
   }
 }
 
+// Launches a kernel with more than 48 KB of dynamic shared memory.
+template <typename K>
+int launch_big(K kernel, dim3 grid, size_t smem, const Step2DArgs &a, cudaStream_t st) {
+  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return (int)e;
+  kernel<<<grid, NT, smem, st>>>(a);
+  return (int)cudaGetLastError();
+}
+
 template <int P, int FLUX, bool F32>
 int launch2(const Step2DArgs &a, cudaStream_t st) {
   dim3 grid((unsigned)((a.NX + TXY - 1) / TXY), (unsigned)((a.NY + TXY - 1) / TXY));
-  k_step2d<P, FLUX, F32><<<grid, NT, 0, st>>>(a);
+  if constexpr (P == 2 && FLUX == ACAT_FLUX_EULER2D && !F32)
+    return launch_big(k_step2d_split, grid, sizeof(Smem2S), a, st);
+  else
+    k_step2d<P, FLUX, F32><<<grid, NT, 0, st>>>(a);
   return (int)cudaGetLastError();
 }
 
@@ -1466,7 +1933,8 @@ template <int P, int FLUX>
 __device__ __forceinline__ void block_tasks_f32(Smem2HF<P, FLUX> &sm, const Step2DArgs &a, float lx, float ly) {
   const TabSF &TB = sm.tab;
   using PH = Phys2<FLUX>;
-  constexpr int S = PH::S;
+  using RP = RPhys2<FLUX>;
+  constexpr int S = PH::S, NX = RP::NX, NR = RP::NR, NXA = NX > 0 ? NX : 1, NRA = NR > 0 ? NR : 1;
   constexpr int NM = 2 * P, NN = NM * NM, per = NT / NN;
   const float gm1 = a.gm1f, axv = a.advf[0], ayv = a.advf[1];
   const int nt = sm.ntask;
@@ -1483,8 +1951,8 @@ __device__ __forceinline__ void block_tasks_f32(Smem2HF<P, FLUX> &sm, const Step
     const int n1 = 2 * p1, n2 = 2 * p2, pm = p1 > p2 ? p1 : p2, n = 2 * pm, zt = pm - 1;
     const bool act = slot_ok && ia < n1 && ib < n2;
     const int ax = an % NAF<P> - 1, ay = an / NAF<P> - 1;
-    float Ff[S], Fg[S], dels[NM][S];
-    typename PH::Base bj;
+    float Ff[S], Fg[S], xs[NM][NXA];
+    typename RP::Base bj;
     if (act) {
       const int tx = acat_tile_index(ax + P - p1 + 1 + ia, Smem2HF<P, FLUX>::TW, a.status);
       const int ty = acat_tile_index(ay + P - p2 + 1 + ib, Smem2HF<P, FLUX>::TW, a.status);
@@ -1499,12 +1967,12 @@ __device__ __forceinline__ void block_tasks_f32(Smem2HF<P, FLUX> &sm, const Step
         dl[c] = ujl[c] - ual[c];
       }
       PH::dflux2_pair(PH::base2(ua, ual, axv, ayv, gm1), dh, dl, Ff, Fg);  // f(u_j) - f(u_a), g(u_j) - g(u_a)
-      bj = PH::base2(uj, ujl, axv, ayv, gm1);
+      bj = RP::base(uj, ujl, axv, ayv, gm1);
     } else {
       float z[S];
 #pragma unroll
       for (int c = 0; c < S; c++) z[c] = Ff[c] = Fg[c] = 0.0f;
-      bj = PH::base(z, axv, ayv, gm1);
+      bj = RP::base(z, z, axv, ayv, gm1);
     }
 #pragma unroll
     for (int c = 0; c < S; c++) {
@@ -1514,7 +1982,7 @@ __device__ __forceinline__ void block_tasks_f32(Smem2HF<P, FLUX> &sm, const Step
 #pragma unroll
     for (int rr = 0; rr < NM; rr++)
 #pragma unroll
-      for (int c = 0; c < S; c++) dels[rr][c] = 0.0f;
+      for (int c = 0; c < NX; c++) xs[rr][c] = RP::init(bj, c);
     // the derivative weights of the node's row and column, read once per task
     // at P <= 3 (at P = 4 they would cost the registers of the second CTA per
     // SM, and the loop reads them from the shared table)
@@ -1570,23 +2038,22 @@ __device__ __forceinline__ void block_tasks_f32(Smem2HF<P, FLUX> &sm, const Step
       }
       __syncthreads();
       if (go) {
-        float af[S], ag[S];
+        float X[NXA], A[NRA], af[S], ag[S];
+        RP::lin(bj, U, X, af, ag);
 #pragma unroll
-        for (int c = 0; c < S; c++) af[c] = ag[c] = 0.0f;
+        for (int c = 0; c < NR; c++) A[c] = 0.0f;
 #pragma unroll
-        for (int rr = 0; rr < NM; rr++) {
+        for (int rr = 0; rr < (NX > 0 ? NM : 0); rr++) {
           if (rr >= n || rr == zt) continue;
           const float cr = TB.taylor[pm][rr][k - 1], wk = TB.gk[pm][k - 1][rr];
-          float ef[S], eg[S];
+          float R[NRA];
 #pragma unroll
-          for (int c = 0; c < S; c++) dels[rr][c] = fmaf(cr, U[c], dels[rr][c]);
-          PH::dflux2(bj, dels[rr], ef, eg);  // f(u_j + del) - f(u_j): the level's weights sum to 0
+          for (int c = 0; c < NX; c++) xs[rr][c] = fmaf(cr, X[c], xs[rr][c]);
+          RP::rem(bj, xs[rr], R);
 #pragma unroll
-          for (int c = 0; c < S; c++) {
-            af[c] = fmaf(wk, ef[c], af[c]);
-            ag[c] = fmaf(wk, eg[c], ag[c]);
-          }
+          for (int c = 0; c < NR; c++) A[c] = fmaf(wk, R[c], A[c]);
         }
+        RP::add(bj, U, A, af, ag);
 #pragma unroll
         for (int c = 0; c < S; c++) {
           sm.X[xw][c] = af[c];
@@ -1804,8 +2271,7 @@ int launch2_hi_f32(const Step2DArgs &a, cudaStream_t st) {
 template <int P, int FLUX>
 int launch2_hi(const Step2DArgs &a, cudaStream_t st) {
   dim3 grid((unsigned)((a.NX + TXH - 1) / TXH), (unsigned)((a.NY + TXH - 1) / TXH));
-  k_step2d_hi<P, FLUX><<<grid, NT, 0, st>>>(a);
-  return (int)cudaGetLastError();
+  return launch_big(k_step2d_hi<P, FLUX>, grid, sizeof(Smem2H<P, FLUX>), a, st);
 }
 
 template <int FLUX, bool F32>
