@@ -56,21 +56,29 @@ __device__ __forceinline__ FF ff_addf(FF a, float b) {
   const FF s = ff_two(a.h, b);
   return ff_fast(s.h, __fadd_rn(s.l, a.l));
 }
+// Products and running sums leave their low part unnormalised (a few units of the
+// high part's last place), which the operations below allow for; ff_add
+// normalises, as its operands may cancel.
 __device__ __forceinline__ FF ff_mul(FF a, FF b) {
   const float p = __fmul_rn(a.h, b.h);
-  return ff_fast(p, fmaf(a.l, b.h, fmaf(a.h, b.l, fmaf(a.h, b.h, -p))));
+  return FF{p, fmaf(a.l, b.h, fmaf(a.h, b.l, fmaf(a.h, b.h, -p)))};
 }
 __device__ __forceinline__ FF ff_mulf(FF a, float g) {
   const float p = __fmul_rn(a.h, g);
-  return ff_fast(p, fmaf(a.l, g, fmaf(a.h, g, -p)));
+  return FF{p, fmaf(a.l, g, fmaf(a.h, g, -p))};
 }
-// s += x g, the low part left unnormalised (ff_norm after the sum)
+// s += x g
 __device__ __forceinline__ void ff_acc(FF &s, FF x, float g) {
   const float p = __fmul_rn(x.h, g);
-  const float e = fmaf(x.l, g, fmaf(x.h, g, -p));
+  const float e = fmaf(x.h, g, -p);
   const FF t = ff_two(s.h, p);
   s.h = t.h;
-  s.l = __fadd_rn(__fadd_rn(s.l, t.l), e);
+  s.l = __fadd_rn(fmaf(x.l, g, __fadd_rn(s.l, t.l)), e);
+}
+// w / d with d's approximate reciprocal r
+__device__ __forceinline__ FF ff_quot(FF w, FF d, float r) {
+  const float q = __fmul_rn(w.h, r);
+  return FF{q, __fmul_rn(__fadd_rn(fmaf(-q, d.h, w.h), fmaf(-q, d.l, w.l)), r)};
 }
 __device__ __forceinline__ FF ff_bits(double x) {
   const Bits64 b = bits_of(x);
@@ -334,12 +342,7 @@ __device__ __forceinline__ bool cat_split_euler(const SplitRec<ACAT_FLUX_EULER1D
           ff_acc(A[q], u[0], c);
           ff_acc(W[q], w, c);
           ff_acc(L[q], L1, c);
-          A[q] = ff_norm(A[q]);
-          W[q] = ff_norm(W[q]);
-          L[q] = ff_norm(L[q]);
-          const float r0 = recip(A[q].h), d0 = __fmul_rn(W[q].h, r0);
-          const float rem = __fadd_rn(fmaf(-d0, A[q].h, W[q].h), fmaf(-d0, A[q].l, W[q].l));
-          const FF dv = ff_fast(d0, __fmul_rn(rem, r0));
+          const FF dv = ff_quot(W[q], A[q], recip(A[q].h));
           const FF Q = ff_mul(W[q], dv);
           const FF T = ff_mul(dv, ff_add(L[q], ff_neg(ff_mul(kap, Q))));
           ff_acc(sq, Q, wt);
@@ -421,7 +424,6 @@ __device__ __forceinline__ bool cat_split_burgers(const SplitRec<ACAT_FLUX_BURGE
         for (int q = 0; q < NL; q++) {
           const int rr = q < p - 1 ? q : q + 1;
           ff_acc(D[q], u, c_tab.powr[p][rr][k - 1]);
-          D[q] = ff_norm(D[q]);
           ff_acc(sq, ff_mul(D[q], D[q]), c_tab.lag[p][k - 1][rr]);
         }
         sq = ff_mul(ff_norm(sq), FF{c_tab.ilq[p].x, c_tab.ilq[p].y});

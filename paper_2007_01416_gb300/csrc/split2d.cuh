@@ -93,11 +93,7 @@ __device__ __forceinline__ void split2_remf(const Split2Const &C, FF v, FF w, co
 // The nonlinear terms at Taylor sums (D, W1, W2, L), D = rho + a.
 __device__ __forceinline__ void split2_terms(FF kap, FF D, FF W1, FF W2, FF L, FF *q) {
   const float r0 = recip(D.h);
-  const float d1 = __fmul_rn(W1.h, r0), d2 = __fmul_rn(W2.h, r0);
-  const FF dv = ff_fast(
-      d1, __fmul_rn(__fadd_rn(fmaf(-d1, D.h, W1.h), fmaf(-d1, D.l, W1.l)), r0));
-  const FF dw = ff_fast(
-      d2, __fmul_rn(__fadd_rn(fmaf(-d2, D.h, W2.h), fmaf(-d2, D.l, W2.l)), r0));
+  const FF dv = ff_quot(W1, D, r0), dw = ff_quot(W2, D, r0);
   q[0] = ff_mul(W1, dv);
   q[1] = ff_mul(W1, dw);
   q[2] = ff_mul(W2, dw);
@@ -256,10 +252,6 @@ __device__ __forceinline__ void split2_order(const Split2Const &C, Split2Node<p>
       ff_acc(N.W1[i], o.W1, c);
       ff_acc(N.W2[i], o.W2, c);
       ff_acc(N.L[i], o.L, c);
-      N.A[i] = ff_norm(N.A[i]);
-      N.W1[i] = ff_norm(N.W1[i]);
-      N.W2[i] = ff_norm(N.W2[i]);
-      N.L[i] = ff_norm(N.L[i]);
       FF t[5];
       split2_terms(C.kap, N.A[i], N.W1[i], N.W2[i], N.L[i], t);
 #pragma unroll

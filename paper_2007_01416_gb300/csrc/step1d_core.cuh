@@ -383,13 +383,28 @@ struct RPhys<ACAT_FLUX_EULER1D> {
   }
 };
 
+// Sum over the n lanes of a group (lane l, first lane base) by a tree of
+// shuffles; every lane returns it at n = 2, 4, 8, lane `base` at n = 6.
+template <int n>
+__device__ __forceinline__ float group_sum(unsigned mask, int base, int l, float t) {
+  if constexpr (n == 6) {
+    t = __fadd_rn(t, __shfl_sync(mask, t, base + (l < 3 ? l + 3 : l - 3)));
+    const float a = __shfl_sync(mask, t, base + (l + 1) % 6), b = __shfl_sync(mask, t, base + (l + 2) % 6);
+    return __fadd_rn(__fadd_rn(t, a), b);
+  } else {
+#pragma unroll
+    for (int w = 1; w < n; w <<= 1) t = __fadd_rn(t, __shfl_sync(mask, t, base + (l ^ w)));
+    return t;
+  }
+}
+
 // CAT2p increment G of one interface by a group of 2p lanes (lane l <-> node
 // j = l - p + 1). hi/lo point at cell i of component 0 of the compensated
 // tile, components `cs` apart. xg: the group's exchange slots in shared
 // memory (node r at xg[r], two sets XSET apart used alternately by k),
 // through which the lanes of the group read the F^(k-2) of all nodes of a
 // system: one 16-byte store and 2p 16-byte broadcast loads per lane and order
-// instead of 2p s shuffles (scalar laws shuffle). Every lane returns G.
+// instead of 2p s shuffles (scalar laws shuffle). Lane 0 of the group returns G.
 template <int p, int FLUX>
 __device__ __forceinline__ void cat_delta(const float *hi, const float *lo, int cs, int l, int base,
                                           float lam, float adv, float gm1, float4 *xg, float *Gout) {
@@ -514,13 +529,7 @@ __device__ __forceinline__ void cat_delta(const float *hi, const float *lo, int 
   }
   const float w = TB::gh(p, l);
 #pragma unroll
-  for (int c = 0; c < S; c++) {
-    const float v = w * Fsum[c];
-    float t = 0.0f;
-#pragma unroll
-    for (int r = 0; r < n; r++) t += __shfl_sync(mask, v, base + r);
-    Gout[c] = t;
-  }
+  for (int c = 0; c < S; c++) Gout[c] = group_sum<n>(mask, base, l, __fmul_rn(w, Fsum[c]));
 }
 
 // cat_delta by a group of 4p lanes, two per node: lane l <-> node
@@ -1009,8 +1018,8 @@ __device__ __forceinline__ void tile_f64(const Step1DArgs &a, Smem64<P, FLUX, NW
 // the L lanes of group grp (all 32 lanes of the warp call it; lane l of the
 // group). thi, tlo: component 0 of the staged tile (components tw apart),
 // cell k of the tile at index k; interface il lies between tile cells
-// il - 1 + GH and il + GH. xw: the warp's exchange slots. Every lane of an
-// active group returns the code p_s and G (lanes beyond the selected order's
+// il - 1 + GH and il + GH. xw: the warp's exchange slots. The lanes of an
+// active group returns the code p_s and lane 0 G (lanes beyond the selected order's
 // 2p return G unset).
 // rej (nullable): the tile's rejected orders per (component, interface), from
 // reject_pass_f32; the group then ORs its interface's bits instead of

@@ -405,15 +405,18 @@ __device__ __forceinline__ void cat2d_f64(const double *q, int cs, int rs, int l
 }
 
 // FP32 block recursion in the delta formulation about the anchor state u_a:
-// returns G_F = F - f(u_a) and G_G = G - g(u_a). xw: the warp's 128 exchange
+// G_F = F - f(u_a) and G_G = G - g(u_a). xw: the warp's 128 exchange
 // slots in shared memory (two sets of 2 x 32 used alternately by k), through
 // which a system's nodes read the F^(k-2) of their row and the G^(k-2) of
 // their column: two 16-byte stores and 2 x 2p 16-byte loads per lane and
-// order instead of 2 x 2p s shuffles (scalar laws shuffle).
+// order instead of 2 x 2p s shuffles (scalar laws shuffle). Lane l < 2S returns
+// component l % S of G_F (l < S) or G_G: systems sum it from the slots order by
+// order (four loads and FMAs against sums of every node's F and G over the
+// orders and a final sum over the nodes by shuffles).
 template <int p, int FLUX>
 __device__ __forceinline__ void cat2d_f32(const float *hi, const float *lo, int cs, int rs, int l,
                                           int base, float lx, float ly, float ax, float ay, float gm1,
-                                          float4 *xw, float *GFo, float *GGo) {
+                                          float4 *xw, float *Go) {
   using TB = Tab<float>;
   using PH = Phys2<FLUX>;
   constexpr int S = PH::S;
@@ -444,12 +447,15 @@ __device__ __forceinline__ void cat2d_f32(const float *hi, const float *lo, int 
   // the 2p - 1 levels r != 0 in pairs packed in float2 lanes, the last alone
   constexpr int NL = n - 1, NP = NL / 2, NX = RP::NX, NR = RP::NR;
   constexpr int NXA = NX > 0 ? NX : 1, NRA = NR > 0 ? NR : 1;
-  float Ff[S], Fg[S], Pf[S], Pg[S], xs1[NXA];
+  float Pf[S], Pg[S], xs1[NXA], sum = 0.0f, Ff = 0.0f, Fg = 0.0f;
   float2 xs2[NP][NXA];
+  // the slots (as floats) and weights of this lane's flux sum
+  const int dir = (l / S) & 1, fs = 4 * (dir ? n : 1);
+  const int f0 = (dir ? 32 : 0) * 4 + 4 * (base + (dir ? p - 1 : (p - 1) * n)) + l % S;
 #pragma unroll
   for (int c = 0; c < S; c++) {
-    Ff[c] = Pf[c] = Df[c];
-    Fg[c] = Pg[c] = Dg[c];
+    Pf[c] = Df[c];
+    Pg[c] = Dg[c];
   }
 #pragma unroll
   for (int c = 0; c < NX; c++) {
@@ -470,6 +476,13 @@ __device__ __forceinline__ void cat2d_f32(const float *hi, const float *lo, int 
       xb[32 + base + l] =
           make_float4(Pg[0], Pg[1], S > 2 ? Pg[S > 2 ? 2 : 0] : 0.0f, S > 3 ? Pg[S > 3 ? 3 : 0] : 0.0f);
       __syncwarp(mask);
+      if (l < 2 * S) {
+        const float *q = reinterpret_cast<const float *>(xb) + f0;
+        float t = 0.0f;
+#pragma unroll
+        for (int r = 0; r < n; r++) t = fmaf(TB::gh(p, r), q[r * fs], t);
+        sum = fmaf(TB::invfact(k - 1), t, sum);
+      }
 #pragma unroll
       for (int r = 0; r < n; r++) {
         const float4 f = xb[base + b1 * n + r], g = xb[32 + base + r * n + a1];
@@ -481,6 +494,8 @@ __device__ __forceinline__ void cat2d_f32(const float *hi, const float *lo, int 
         }
       }
     } else {
+      Ff = fmaf(TB::invfact(k - 1), Pf[0], Ff);
+      Fg = fmaf(TB::invfact(k - 1), Pg[0], Fg);
 #pragma unroll
       for (int r = 0; r < n; r++) {
         Ux[0] = fmaf(gx[r], __shfl_sync(mask, Pf[0], base + b1 * n + r), Ux[0]);
@@ -517,23 +532,30 @@ __device__ __forceinline__ void cat2d_f32(const float *hi, const float *lo, int 
       for (int c = 0; c < NR; c++) A[c] = fmaf(wk, R1[c], A2[c].x + A2[c].y);
     }
     RP::add(bj, U, A, Pf, Pg);
-#pragma unroll
-    for (int c = 0; c < S; c++) {
-      Ff[c] = fmaf(TB::invfact(k), Pf[c], Ff[c]);
-      Fg[c] = fmaf(TB::invfact(k), Pg[c], Fg[c]);
-    }
   }
+  if constexpr (S > 1) {
+    float4 *xb = xw + ((n + 1) & 1) * 64;
+    xb[base + l] = make_float4(Pf[0], Pf[1], Pf[S > 2 ? 2 : 0], Pf[S > 3 ? 3 : 0]);
+    xb[32 + base + l] = make_float4(Pg[0], Pg[1], Pg[S > 2 ? 2 : 0], Pg[S > 3 ? 3 : 0]);
+    __syncwarp(mask);
+    if (l < 2 * S) {
+      const float *q = reinterpret_cast<const float *>(xb) + f0;
+      float t = 0.0f;
 #pragma unroll
-  for (int c = 0; c < S; c++) {
-    const float vF = TB::gh(p, a1) * Ff[c], vG = TB::gh(p, b1) * Fg[c];
+      for (int r = 0; r < n; r++) t = fmaf(TB::gh(p, r), q[r * fs], t);
+      *Go = fmaf(TB::invfact(n), t, sum);
+    }
+  } else {
+    Ff = fmaf(TB::invfact(n), Pf[0], Ff);
+    Fg = fmaf(TB::invfact(n), Pg[0], Fg);
+    const float vF = TB::gh(p, a1) * Ff, vG = TB::gh(p, b1) * Fg;
     float tF = 0.0f, tG = 0.0f;
 #pragma unroll
     for (int r = 0; r < n; r++) {
       tF += __shfl_sync(mask, vF, base + (p - 1) * n + r);
       tG += __shfl_sync(mask, vG, base + r * n + (p - 1));
     }
-    GFo[c] = tF;
-    GGo[c] = tG;
+    *Go = l == 0 ? tF : tG;
   }
 }
 
@@ -784,6 +806,8 @@ __global__ void __launch_bounds__(NT, F32 ? 3 : (FLUX == ACAT_FLUX_LINEAR ? 3 : 
   __shared__ R Fx[TXY][TXY + 1][S];
   __shared__ R Gy[TXY + 1][TXY][S];
   __shared__ double s_dt;
+  __shared__ unsigned short task[P >= 2 ? NA * NA : 1];  // blocks: anchor, wants F (bit 8), G (bit 9)
+  __shared__ int s_ntask;
   __shared__ double s_red[2][NT / 32];
   const long NXl = a.NX, NYl = a.NY;
   const long x0 = (long)blockIdx.x * TXY, y0 = (long)blockIdx.y * TXY;
@@ -791,6 +815,7 @@ __global__ void __launch_bounds__(NT, F32 ? 3 : (FLUX == ACAT_FLUX_LINEAR ? 3 : 
   __shared__ double s_lx, s_ly;
   __shared__ float s_lxf, s_lyf;
   if (threadIdx.x == 0) {
+    s_ntask = 0;
     s_dt = step_dt2(a);
     s_lx = s_dt / a.dx;
     s_ly = s_dt / a.dy;
@@ -843,68 +868,69 @@ __global__ void __launch_bounds__(NT, F32 ? 3 : (FLUX == ACAT_FLUX_LINEAR ? 3 : 
     __syncthreads();
   }
 
-  for (int round = 0; round < NA * NA / 16; round++) {
-    const int an = round * 16 + warp * 2 + grp;
-    const int ax = an % NA - 1, ay = an / NA - 1;  // anchor relative to (x0, y0)
+  // --- per anchor (one thread each): orders, FL-CAT2 directions, block list ---
+  static_assert(NA * NA == NT, "one anchor per thread");
+  {
+    const int an = threadIdx.x, ax = an % NA - 1, ay = an / NA - 1;  // anchor relative to (x0, y0)
     const long gxa = x0 + ax, gya = y0 + ay;
     const bool inside = gxa < NXl && gya < NYl;
-    const bool needF = inside && ay >= 0;
-    const bool needG = inside && ax >= 0;
+    const bool needF = inside && ay >= 0, needG = inside && ax >= 0;
     const int tx = ax + GH2, ty = ay + GH2;
-    const double *q64 = F32 ? nullptr : &tile[0][F32 ? 0 : ty][F32 ? 0 : tx];
-    unsigned rej = 0;
+    int px = 1, py = 1;
     if constexpr (P >= 2) {
+      unsigned rx = 0, ry = 0;
 #pragma unroll
       for (int c = 0; c < S; c++) {
-        rej |= rej2[c * NA * NA + an];
-        rej |= (unsigned)rej2[(S + c) * NA * NA + an] << (P - 1);
+        rx |= rej2[c * NA * NA + an];
+        ry |= rej2[(S + c) * NA * NA + an];
       }
+      px = rx & 1u ? 1 : 2;
+      py = ry & 1u ? 1 : 2;
+      const bool blkF = needF && px == 2, blkG = needG && py == 2;
+      if (blkF || blkG)
+        task[atomicAdd(&s_ntask, 1)] = (unsigned short)(an | (blkF ? 1 << 8 : 0) | (blkG ? 1 << 9 : 0));
     }
-    int px = 1, py = 1;
-    if (P >= 2) {
-      const unsigned all = (1u << (P - 1)) - 1u;
-      const unsigned accx = ~rej & all, accy = ~(rej >> (P - 1)) & all;
-      px = accx ? (32 - __clz(accx)) + 1 : 1;
-      py = accy ? (32 - __clz(accy)) + 1 : 1;
-    }
-    const bool blkF = needF && px >= 2, blkG = needG && py >= 2;
-    R F[S], G[S];
-    if (P >= 2 && (blkF || blkG)) {
-      if constexpr (P >= 2) {
-        if constexpr (F32) {
-          cat2d_f32<2, FLUX>(&thi[0][ty][tx], &tlo[0][ty][tx], CS, RS, l, base, s_lxf, s_lyf, a.advf[0],
-                             a.advf[1], a.gm1f, &xs2[warp * 128], F, G);
-        } else {
-          cat2d_f64<2, FLUX>(q64, CS, RS, l, base, lxd, lyd, a.adv[0], a.adv[1], a.gamma - 1.0, F, G);
-        }
-      }
-    }
-    const bool flF = needF && !blkF, flG = needG && !blkG;
-    if (l == 0 && (flF || flG)) {
+    if (needF && a.ord_x && (ax >= 0 || gxa == -1)) a.ord_x[gya * (NXl + 1) + (gxa + 1)] = (int8_t)px;
+    if (needG && a.ord_y && (ay >= 0 || gya == -1)) a.ord_y[(gya + 1) * NXl + gxa] = (int8_t)py;
+    const bool flF = needF && px < 2, flG = needG && py < 2;
+    if (flF || flG) {
       R F1[S], G1[S];
-      if constexpr (F32) {
+      if constexpr (F32)
         flcat2_2d_f32<FLUX>(&thi[0][ty][tx], &tlo[0][ty][tx], CS, RS, flF, flG, s_lxf, s_lyf, a.advf[0],
                             a.advf[1], a.gammaf, a.gm1f, a.limiter_form, a.lo_flux, F1, G1);
-      } else {
-        flcat2_2d_f64<FLUX>(q64, CS, RS, flF, flG, lxd, lyd, a.adv[0], a.adv[1], a.gamma,
+      else
+        flcat2_2d_f64<FLUX>(&tile[0][ty][tx], CS, RS, flF, flG, lxd, lyd, a.adv[0], a.adv[1], a.gamma,
                             a.limiter_form, a.lo_flux, F1, G1);
-      }
 #pragma unroll
       for (int c = 0; c < S; c++) {
-        if (flF) F[c] = F1[c];
-        if (flG) G[c] = G1[c];
+        if (flF) Fx[ay][ax + 1][c] = F1[c];
+        if (flG) Gy[ay + 1][ax][c] = G1[c];
       }
     }
-    if (l == 0) {
-      if (needF) {
+  }
+  // --- the block recursions, 16 lanes each, from the list --------------------
+  if constexpr (P >= 2) {
+    __syncthreads();
+#pragma unroll 1
+    for (int t = warp * 2 + grp; t < s_ntask; t += 2 * (NT / 32)) {
+      const int tk = task[t], an = tk & 0xff, ax = an % NA - 1, ay = an / NA - 1;
+      const int tx = ax + GH2, ty = ay + GH2;
+      if constexpr (F32) {
+        float v;
+        cat2d_f32<2, FLUX>(&thi[0][ty][tx], &tlo[0][ty][tx], CS, RS, l, base, s_lxf, s_lyf, a.advf[0],
+                           a.advf[1], a.gm1f, &xs2[warp * 128], &v);
+        if (l < S && (tk & 0x100)) Fx[ay][ax + 1][l % S] = v;
+        if (l >= S && l < 2 * S && (tk & 0x200)) Gy[ay + 1][ax][l % S] = v;
+      } else {
+        R F[S], G[S];
+        cat2d_f64<2, FLUX>(&tile[0][ty][tx], CS, RS, l, base, lxd, lyd, a.adv[0], a.adv[1], a.gamma - 1.0, F, G);
+        if (l == 0) {
 #pragma unroll
-        for (int c = 0; c < S; c++) Fx[ay][ax + 1][c] = F[c];
-        if (a.ord_x && (ax >= 0 || gxa == -1)) a.ord_x[gya * (NXl + 1) + (gxa + 1)] = (int8_t)px;
-      }
-      if (needG) {
-#pragma unroll
-        for (int c = 0; c < S; c++) Gy[ay + 1][ax][c] = G[c];
-        if (a.ord_y && (ay >= 0 || gya == -1)) a.ord_y[(gya + 1) * NXl + gxa] = (int8_t)py;
+          for (int c = 0; c < S; c++) {
+            if (tk & 0x100) Fx[ay][ax + 1][c] = F[c];
+            if (tk & 0x200) Gy[ay + 1][ax][c] = G[c];
+          }
+        }
       }
     }
   }
@@ -1026,6 +1052,8 @@ struct Smem2S {
   double dlx, dly;
   unsigned char rej[8 * NA * NA];
   unsigned char cF[TXY][TXY + 1], cG[TXY + 1][TXY];  // 2 where the flux is a pair
+  unsigned short task[NA * NA];                      // blocks: anchor, wants F (bit 8), G (bit 9)
+  int ntask;
 };
 
 // The recursion of one anchor by 16 lanes. Lane l < 8 returns the flux sum of
@@ -1099,6 +1127,7 @@ __global__ void __launch_bounds__(NT, 2) k_step2d_split(const Step2DArgs a) {
     const double dt = step_dt2(a);
     sm.dlx = dt / a.dx;
     sm.dly = dt / a.dy;
+    sm.ntask = 0;
   }
   const double gm1 = a.gamma - 1.0;
   for (int q = threadIdx.x; q < CELLS; q += NT) {
@@ -1134,15 +1163,11 @@ __global__ void __launch_bounds__(NT, 2) k_step2d_split(const Step2DArgs a) {
     sm.rej[q] = (unsigned char)r;
   }
   __syncthreads();
-#pragma unroll 1
-  for (int round = 0; round < NA * NA / 16; round++) {
-    const int an = round * 16 + warp * 2 + grp;
-    const int ax = an % NA - 1, ay = an / NA - 1;  // anchor relative to (x0, y0)
+  {
+    const int an = threadIdx.x, ax = an % NA - 1, ay = an / NA - 1;  // anchor relative to (x0, y0)
     const long gxa = x0 + ax, gya = y0 + ay;
     const bool inside = gxa < NXl && gya < NYl;
     const bool needF = inside && ay >= 0, needG = inside && ax >= 0;
-    const int cell = (ay + GH2) * TW2 + ax + GH2;
-    const double *q64 = &sm.tile[0][ay + GH2][ax + GH2];
     unsigned rx = 0, ry = 0;
 #pragma unroll
     for (int c = 0; c < S; c++) {
@@ -1151,40 +1176,45 @@ __global__ void __launch_bounds__(NT, 2) k_step2d_split(const Step2DArgs a) {
     }
     const int px = rx & 1u ? 1 : 2, py = ry & 1u ? 1 : 2;
     const bool blkF = needF && px == 2, blkG = needG && py == 2;
-    if (blkF || blkG) {
-      FF s;
-      if (cat2d_split(sm, a, cell, l, base, warp, s)) {
-        const int c = l & 3;
-        if (l < 4 && blkF) *reinterpret_cast<float2 *>(&sm.Fx[ay][ax + 1][c]) = make_float2(s.h, s.l);
-        if (l >= 4 && l < 8 && blkG) *reinterpret_cast<float2 *>(&sm.Gy[ay + 1][ax][c]) = make_float2(s.h, s.l);
-        if (l == 0 && blkF) sm.cF[ay][ax + 1] = 2;
-        if (l == 0 && blkG) sm.cG[ay + 1][ax] = 2;
-      } else {
-        double F[S], G[S];
-        cat2d_f64<2, FLUX>(q64, CELLS, RS, l, base, lxd, lyd, a.adv[0], a.adv[1], gm1, F, G);
-        if (l == 0) {
+    if (blkF || blkG)
+      sm.task[atomicAdd(&sm.ntask, 1)] = (unsigned short)(an | (blkF ? 1 << 8 : 0) | (blkG ? 1 << 9 : 0));
+    if (needF && a.ord_x && (ax >= 0 || gxa == -1)) a.ord_x[gya * (NXl + 1) + (gxa + 1)] = (int8_t)px;
+    if (needG && a.ord_y && (ay >= 0 || gya == -1)) a.ord_y[(gya + 1) * NXl + gxa] = (int8_t)py;
+    const bool flF = needF && px < 2, flG = needG && py < 2;
+    if (flF || flG) {
+      double F1[S], G1[S];
+      flcat2_2d_f64<FLUX>(&sm.tile[0][ay + GH2][ax + GH2], CELLS, RS, flF, flG, lxd, lyd, a.adv[0], a.adv[1],
+                          a.gamma, a.limiter_form, a.lo_flux, F1, G1);
 #pragma unroll
-          for (int c = 0; c < S; c++) {
-            if (blkF) sm.Fx[ay][ax + 1][c] = F[c];
-            if (blkG) sm.Gy[ay + 1][ax][c] = G[c];
-          }
-        }
+      for (int c = 0; c < S; c++) {
+        if (flF) sm.Fx[ay][ax + 1][c] = F1[c];
+        if (flG) sm.Gy[ay + 1][ax][c] = G1[c];
       }
     }
-    const bool flF = needF && !blkF, flG = needG && !blkG;
-    if (l == 0) {
-      if (flF || flG) {
-        double F1[S], G1[S];
-        flcat2_2d_f64<FLUX>(q64, CELLS, RS, flF, flG, lxd, lyd, a.adv[0], a.adv[1], a.gamma, a.limiter_form,
-                            a.lo_flux, F1, G1);
+  }
+  __syncthreads();
+#pragma unroll 1
+  for (int t = warp * 2 + grp; t < sm.ntask; t += 2 * (NT / 32)) {
+    const int tk = sm.task[t], an = tk & 0xff, ax = an % NA - 1, ay = an / NA - 1;
+    const bool blkF = (tk & 0x100) != 0, blkG = (tk & 0x200) != 0;
+    FF s;
+    if (cat2d_split(sm, a, (ay + GH2) * TW2 + ax + GH2, l, base, warp, s)) {
+      const int c = l & 3;
+      if (l < 4 && blkF) *reinterpret_cast<float2 *>(&sm.Fx[ay][ax + 1][c]) = make_float2(s.h, s.l);
+      if (l >= 4 && l < 8 && blkG) *reinterpret_cast<float2 *>(&sm.Gy[ay + 1][ax][c]) = make_float2(s.h, s.l);
+      if (l == 0 && blkF) sm.cF[ay][ax + 1] = 2;
+      if (l == 0 && blkG) sm.cG[ay + 1][ax] = 2;
+    } else {
+      double F[S], G[S];
+      cat2d_f64<2, FLUX>(&sm.tile[0][ay + GH2][ax + GH2], CELLS, RS, l, base, lxd, lyd, a.adv[0], a.adv[1], gm1, F,
+                         G);
+      if (l == 0) {
 #pragma unroll
         for (int c = 0; c < S; c++) {
-          if (flF) sm.Fx[ay][ax + 1][c] = F1[c];
-          if (flG) sm.Gy[ay + 1][ax][c] = G1[c];
+          if (blkF) sm.Fx[ay][ax + 1][c] = F[c];
+          if (blkG) sm.Gy[ay + 1][ax][c] = G[c];
         }
       }
-      if (needF && a.ord_x && (ax >= 0 || gxa == -1)) a.ord_x[gya * (NXl + 1) + (gxa + 1)] = (int8_t)px;
-      if (needG && a.ord_y && (ay >= 0 || gya == -1)) a.ord_y[(gya + 1) * NXl + gxa] = (int8_t)py;
     }
   }
   __syncthreads();
