@@ -26,21 +26,24 @@ struct AcatTables {
   float ghf[ACAT_MAXP + 1][ACAT_MAXN];
   float taylorf[ACAT_MAXP + 1][ACAT_MAXN][ACAT_MAXN];
   float invfactf[ACAT_MAXN + 1];
-  // the weights as integers over one common denominator per p (exact in
-  // float), for the float-float recursion: g1 x LC, gamma^{k,0} / k! x LQ
-  // ([p][k][r]), gh x LH; r^l ([p][r][l]); 840 / k; 1 / (k LC) and 1 / LQ
-  float g1i[ACAT_MAXP + 1][ACAT_MAXN][ACAT_MAXN];
-  float lag[ACAT_MAXP + 1][ACAT_MAXN][ACAT_MAXN];
-  float ghi[ACAT_MAXP + 1][ACAT_MAXN];
-  float powr[ACAT_MAXP + 1][ACAT_MAXN][ACAT_MAXN];
-  float k840[ACAT_MAXN + 1];
-  double ilc[ACAT_MAXP + 1][ACAT_MAXN];
-  struct {
-    float x, y;
-  } ilq[ACAT_MAXP + 1];
+  double ilc[ACAT_MAXP + 1][ACAT_MAXN];  // 1 / (k LC), see SplitTab
 };
 
+// The weights of the float-float recursion: integers over one common
+// denominator per p, exact in float (g1 x LC, gamma^{k,0} / k! x LQ, gh x LH), for
+// p = 2..4 at index p - 2. Kept in global memory and copied to shared memory by
+// each CTA: a step of one wave touches every entry once, and constant memory
+// would serve each line with a miss of its own.
+struct alignas(16) SplitTab {
+  float2 lv[3][7][7];  // [p-2][k-2][level q]: r^(k-1) and gamma^{k-1,0}_r / (k-1)! x LQ of the level's r != 0
+  float g1[3][8][8];   // [p-2][j][r]
+  float gh[3][8];
+  float k840[8];       // 840 / k at k - 1
+};
+static_assert(sizeof(SplitTab) % 16 == 0, "copied in 16-byte pieces");
+
 void acat_build_tables(AcatTables *T);
+void acat_build_split(SplitTab *T);
 
 // Arguments of one 1D step launch (passed by value).
 struct Step1DArgs {
@@ -161,15 +164,15 @@ struct Step2DArgs {
 
 int acat_launch_step2d(int P, int flux, int prec, const Step2DArgs &a, void *stream);
 int acat_launch_smax2d(int flux, int prec, const Step2DArgs &a, void *stream);
-int acat_upload_tables_1d(const AcatTables *T);
+int acat_upload_tables_1d(const AcatTables *T, const SplitTab *G);
 int acat_upload_tables_adj(const AcatTables *T);
-int acat_upload_tables_batch(const AcatTables *T);
+int acat_upload_tables_batch(const AcatTables *T, const SplitTab *G);
 int acat_adjoint_slots(int P);
 // Adjoint of one 1D step (a.u_in = u^n, dt from a.dt_in or a.dt_fixed): ubar0 from ubar1.
 // FP64: double states and cotangents, double contrib; FP32: compensated float pairs, float contrib.
 int acat_launch_adjoint1d(int P, int flux, int prec, const Step1DArgs &a, const void *ubar1, void *contrib,
                           void *ubar0, void *stream);
-int acat_upload_tables_2d(const AcatTables *T);
+int acat_upload_tables_2d(const AcatTables *T, const SplitTab *G);
 
 // Initial wave-speed reduction into smax[slot] (and t = 0 into tslot[slot]).
 int acat_launch_smax1d(int flux, int prec, const Step1DArgs &a, void *stream);

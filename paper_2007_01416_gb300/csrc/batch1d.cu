@@ -86,6 +86,9 @@ __global__ void __launch_bounds__(NW * 32, MinCtas<P, F32>::value * 8 / NW)
   // read after it: the tile's staging barrier publishes it, and the two slots
   // alternate, so a claim never overwrites a slot another thread still reads
   __shared__ long long s_next[2];
+  if constexpr (!F32) {  // published by the first tile's staging barrier
+    if constexpr (SM::kSplit) split_tab(sm[0].tab, (int)threadIdx.x, NW * 32);
+  }
   int par = 0;
   for (long w = blockIdx.x; w < bt.ntiles; par ^= 1) {
     if (threadIdx.x == 0) s_next[par] = (long long)gridDim.x + atomicAdd(bt.next, 1);
@@ -275,4 +278,7 @@ int acat_launch_smax_batch(int flux, int prec, const Step1DArgs &a, const BatchA
                                : launch_smax_batch<false>(flux, a, bt, st);
 }
 
-int acat_upload_tables_batch(const AcatTables *T) { return (int)cudaMemcpyToSymbol(c_tab, T, sizeof *T); }
+int acat_upload_tables_batch(const AcatTables *T, const SplitTab *G) {
+  const int e = (int)cudaMemcpyToSymbol(c_tab, T, sizeof *T);
+  return e ? e : (int)cudaMemcpyToSymbol(g_split, G, sizeof *G);
+}

@@ -35,7 +35,16 @@
 
 #include "phys1d.cuh"
 
+static __device__ SplitTab g_split;  // uploaded beside c_tab
+
 namespace {
+
+// The table to shared memory by the first threads of a CTA (at least 64).
+__device__ __forceinline__ void split_tab(SplitTab &t, int tid, int nthreads) {
+  const float4 *src = reinterpret_cast<const float4 *>(&g_split);
+  float4 *dst = reinterpret_cast<float4 *>(&t);
+  for (int q = tid; q < (int)(sizeof(SplitTab) / 16); q += nthreads) dst[q] = __ldg(&src[q]);
+}
 
 // ---- float-float arithmetic (Knuth's TwoSum, Dekker's Fast2Sum, TwoProd by FMA) ----
 __device__ __forceinline__ FF ff_two(float a, float b) {
@@ -103,6 +112,10 @@ __device__ __forceinline__ FF f3_diff(F3 a, F3 b) {
 
 // Common denominators of the integer weights (index p).
 __device__ __forceinline__ constexpr float split_lq(int p) { return p == 4 ? 5040.0f : p == 3 ? 120.0f : 6.0f; }
+__device__ __forceinline__ constexpr FF split_ilq(int p) {  // 1 / LQ
+  return FF{(float)(1.0 / (double)split_lq(p)),
+            (float)(1.0 / (double)split_lq(p) - (double)(float)(1.0 / (double)split_lq(p)))};
+}
 // 1 / (840 LH): the flux sums carry 840 / k and gh x LH
 __device__ __forceinline__ double split_ginv(int p) {
   return p == 4 ? 1.0 / (840.0 * 840.0) : p == 3 ? 1.0 / (840.0 * 60.0) : 1.0 / (840.0 * 12.0);
@@ -199,14 +212,14 @@ __device__ __forceinline__ FF split_sum(unsigned mask, int base, int l, FF t) {
 // the group); G is in lane `base`.
 template <int p, int TW>
 __device__ __forceinline__ bool cat_split_euler(const SplitRec<ACAT_FLUX_EULER1D, TW> &rec, const Step1DArgs &a,
-                                                const float2 *lamk, int ic, int l, int base, float4 *xa,
-                                                float2 *xb, FF *G) {
+                                                const SplitTab &tab, const float2 *lamk, int ic, int l, int base,
+                                                float4 *xa, float2 *xb, FF *G) {
   constexpr int n = 2 * p, NL = n - 1;
   const unsigned mask = ((1u << n) - 1u) << base;
   const FF gam = ff_of(a.sgam), kap = ff_of(a.skap), omk = ff_of(a.somk), gm = ff_of(a.sgm1);
   float g1r[n];
 #pragma unroll
-  for (int r = 0; r < n; r++) g1r[r] = c_tab.g1i[p][l][r];
+  for (int r = 0; r < n; r++) g1r[r] = tab.g1[p - 2][l][r];
   const int jc = ic + l - p + 1;
   const float4 q0 = rec.q[0][jc], q1 = rec.q[1][jc];
   const FF rho{q0.x, q0.y}, v{q0.z, q0.w}, h{q1.x, q1.y};
@@ -244,7 +257,8 @@ __device__ __forceinline__ bool cat_split_euler(const SplitRec<ACAT_FLUX_EULER1D
 #pragma unroll 1
     for (int k = 2; k <= n; k++) {
       const float2 lk = lamk[k - 2];
-      const float pk = c_tab.powr[p][n - 1][k - 1], ck = c_tab.k840[k];  // p^(k-1), 840 / k
+      const float2 *lv = tab.lv[p - 2][k - 2];
+      const float pk = lv[NL - 1].x, ck = tab.k840[k - 1];  // p^(k-1), 840 / k
       float4 *xs = xa + (k & 1) * XSET;
       if (!tail && flt)
         tail = __all_sync(mask, fabsf(Y[0].h) <= SPLIT_TAIL * rs && fabsf(Y[1].h) <= SPLIT_TAIL * rh &&
@@ -271,8 +285,7 @@ __device__ __forceinline__ bool cat_split_euler(const SplitRec<ACAT_FLUX_EULER1D
         float sq = 0.0f, st = 0.0f;
 #pragma unroll
         for (int q = 0; q < NL; q++) {
-          const int rr = q < p - 1 ? q : q + 1;
-          const float c = c_tab.powr[p][rr][k - 1], wt = c_tab.lag[p][k - 1][rr];
+          const float c = lv[q].x, wt = lv[q].y;
           A[q].h = fmaf(c, u0, A[q].h);
           W[q].h = fmaf(c, w, W[q].h);
           L[q].h = fmaf(c, L1, L[q].h);
@@ -320,8 +333,7 @@ __device__ __forceinline__ bool cat_split_euler(const SplitRec<ACAT_FLUX_EULER1D
         float sq = 0.0f, st = 0.0f;
 #pragma unroll
         for (int q = 0; q < NL; q++) {
-          const int rr = q < p - 1 ? q : q + 1;
-          const float c = c_tab.powr[p][rr][k - 1], wt = c_tab.lag[p][k - 1][rr];
+          const float c = lv[q].x, wt = lv[q].y;
           A[q].h = fmaf(c, u[0].h, A[q].h);
           W[q].h = fmaf(c, w.h, W[q].h);
           L[q].h = fmaf(c, L1.h, L[q].h);
@@ -337,8 +349,7 @@ __device__ __forceinline__ bool cat_split_euler(const SplitRec<ACAT_FLUX_EULER1D
         FF sq{0.0f, 0.0f}, st{0.0f, 0.0f};
 #pragma unroll
         for (int q = 0; q < NL; q++) {
-          const int rr = q < p - 1 ? q : q + 1;
-          const float c = c_tab.powr[p][rr][k - 1], wt = c_tab.lag[p][k - 1][rr];
+          const float c = lv[q].x, wt = lv[q].y;
           ff_acc(A[q], u[0], c);
           ff_acc(W[q], w, c);
           ff_acc(L[q], L1, c);
@@ -348,7 +359,7 @@ __device__ __forceinline__ bool cat_split_euler(const SplitRec<ACAT_FLUX_EULER1D
           ff_acc(sq, Q, wt);
           ff_acc(st, T, wt);
         }
-        const FF iq{c_tab.ilq[p].x, c_tab.ilq[p].y};
+        constexpr FF iq = split_ilq(p);
         sq = ff_mul(ff_norm(sq), iq);
         st = ff_mul(ff_norm(st), iq);
         y1 = ff_add(y1, ff_mul(omk, sq));
@@ -365,7 +376,7 @@ __device__ __forceinline__ bool cat_split_euler(const SplitRec<ACAT_FLUX_EULER1D
     if (!flt || __all_sync(mask, Bw * Bw <= SPLIT_QUAD * rs * rs && Bw * Bl <= SPLIT_QUAD * rs * rh)) break;
     allow = false;  // the remainders grew past float: once more with pairs
   }
-  const float gw = c_tab.ghi[p][l];
+  const float gw = tab.gh[p - 2][l];
 #pragma unroll
   for (int c = 0; c < 3; c++) G[c] = split_sum<n>(mask, base, l, ff_mulf(ff_norm(S[c]), gw));
   return true;
@@ -375,12 +386,13 @@ __device__ __forceinline__ bool cat_split_euler(const SplitRec<ACAT_FLUX_EULER1D
 // cfl / lambda (the largest |u| when the CFL rule set dt).
 template <int p, int TW>
 __device__ __forceinline__ bool cat_split_burgers(const SplitRec<ACAT_FLUX_BURGERS, TW> &rec, float vs,
-                                                  const float2 *lamk, int ic, int l, int base, FF *G) {
+                                                  const SplitTab &tab, const float2 *lamk, int ic, int l, int base,
+                                                  FF *G) {
   constexpr int n = 2 * p, NL = n - 1;
   const unsigned mask = ((1u << n) - 1u) << base;
   float g1r[n];
 #pragma unroll
-  for (int r = 0; r < n; r++) g1r[r] = c_tab.g1i[p][l][r];
+  for (int r = 0; r < n; r++) g1r[r] = tab.g1[p - 2][l][r];
   const int jc = ic + l - p + 1;
   const FF uj = ff_of(rec.u[jc]);
   const float4 fj = rec.f[jc], fi = rec.f[ic];
@@ -400,42 +412,41 @@ __device__ __forceinline__ bool cat_split_burgers(const SplitRec<ACAT_FLUX_BURGE
     float B = 0.0f;
 #pragma unroll 1
     for (int k = 2; k <= n; k++) {
-      const float2 lk = lamk[k - 2];
+      const float2 lk = lamk[k - 2], *lv = tab.lv[p - 2][k - 2];
       FF u{0.0f, 0.0f};
 #pragma unroll
       for (int r = 0; r < n; r++)
         ff_acc(u, FF{__shfl_sync(mask, Y.h, base + r), __shfl_sync(mask, Y.l, base + r)}, g1r[r]);
       u = ff_mul(ff_norm(u), FF{lk.x, lk.y});
-      B = fmaf(c_tab.powr[p][n - 1][k - 1], fabsf(u.h), B);
+      B = fmaf(lv[NL - 1].x, fabsf(u.h), B);
       if (k == 2 && flt) flt = __all_sync(mask, 4.0f * B * B <= SPLIT_QUAD * v2);
       Y = ff_mul(uj, u);
       if (flt) {
         float sq = 0.0f;
 #pragma unroll
         for (int q = 0; q < NL; q++) {
-          const int rr = q < p - 1 ? q : q + 1;
-          D[q].h = fmaf(c_tab.powr[p][rr][k - 1], u.h, D[q].h);
-          sq = fmaf(c_tab.lag[p][k - 1][rr], __fmul_rn(D[q].h, D[q].h), sq);
+          D[q].h = fmaf(lv[q].x, u.h, D[q].h);
+          sq = fmaf(lv[q].y, __fmul_rn(D[q].h, D[q].h), sq);
         }
         Y = ff_addf(Y, __fmul_rn(sq, 0.5f / split_lq(p)));
       } else {
         FF sq{0.0f, 0.0f};
 #pragma unroll
         for (int q = 0; q < NL; q++) {
-          const int rr = q < p - 1 ? q : q + 1;
-          ff_acc(D[q], u, c_tab.powr[p][rr][k - 1]);
-          ff_acc(sq, ff_mul(D[q], D[q]), c_tab.lag[p][k - 1][rr]);
+          ff_acc(D[q], u, lv[q].x);
+          ff_acc(sq, ff_mul(D[q], D[q]), lv[q].y);
         }
-        sq = ff_mul(ff_norm(sq), FF{c_tab.ilq[p].x, c_tab.ilq[p].y});
+        constexpr FF iq = split_ilq(p);
+        sq = ff_mul(ff_norm(sq), iq);
         Y = ff_add(Y, FF{0.5f * sq.h, 0.5f * sq.l});
       }
-      ff_acc(S, Y, c_tab.k840[k]);
+      ff_acc(S, Y, tab.k840[k - 1]);
     }
     if (!__all_sync(mask, B <= SPLIT_TAU * vs)) return false;
     if (!flt || __all_sync(mask, B * B <= SPLIT_QUAD * v2)) break;
     allow = false;
   }
-  G[0] = split_sum<n>(mask, base, l, ff_mulf(ff_norm(S), c_tab.ghi[p][l]));
+  G[0] = split_sum<n>(mask, base, l, ff_mulf(ff_norm(S), tab.gh[p - 2][l]));
   return true;
 }
 

@@ -217,17 +217,17 @@ __device__ __forceinline__ void split2_sums(const Split2Slots &x, int i0, int j0
   for (int c = 0; c < 4; c++) u[c] = ff_add(ff_mul(ff_norm(a[c]), lx), ff_mul(ff_norm(b[c]), ly));
 }
 
-// Order k of a node in pairs; flt: remainders in float. u: from split2_sums.
+// An order of a node in pairs (lv: the order's level weights); flt: remainders in
+// float. u: from split2_sums.
 template <int p>
-__device__ __forceinline__ void split2_order(const Split2Const &C, Split2Node<p> &N, int k, bool flt,
+__device__ __forceinline__ void split2_order(const Split2Const &C, Split2Node<p> &N, const float2 *lv, bool flt,
                                              const FF *u, const Split2Lin &o, FF *F, FF *G) {
   constexpr int NL = 2 * p - 1;
   if (flt) {
     float q[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
     for (int i = 0; i < NL; i++) {
-      const int rr = i < p - 1 ? i : i + 1;
-      const float c = c_tab.powr[p][rr][k - 1], wt = c_tab.lag[p][k - 1][rr];
+      const float c = lv[i].x, wt = lv[i].y;
       N.A[i].h = fmaf(c, u[0].h, N.A[i].h);
       N.W1[i].h = fmaf(c, o.W1.h, N.W1[i].h);
       N.W2[i].h = fmaf(c, o.W2.h, N.W2[i].h);
@@ -246,8 +246,7 @@ __device__ __forceinline__ void split2_order(const Split2Const &C, Split2Node<p>
     for (int e = 0; e < 5; e++) q[e] = FF{0.0f, 0.0f};
 #pragma unroll
     for (int i = 0; i < NL; i++) {
-      const int rr = i < p - 1 ? i : i + 1;
-      const float c = c_tab.powr[p][rr][k - 1], wt = c_tab.lag[p][k - 1][rr];
+      const float c = lv[i].x, wt = lv[i].y;
       ff_acc(N.A[i], u[0], c);
       ff_acc(N.W1[i], o.W1, c);
       ff_acc(N.W2[i], o.W2, c);
@@ -257,16 +256,16 @@ __device__ __forceinline__ void split2_order(const Split2Const &C, Split2Node<p>
 #pragma unroll
       for (int e = 0; e < 5; e++) ff_acc(q[e], t[e], wt);
     }
-    const FF iq{c_tab.ilq[p].x, c_tab.ilq[p].y};
+    constexpr FF iq = split_ilq(p);
 #pragma unroll
     for (int e = 0; e < 5; e++) q[e] = ff_mul(ff_norm(q[e]), iq);
     split2_rem(C, N.v, N.w, u, o, q, F, G);
   }
 }
 
-// Order k of a node in float (F, G high parts only).
+// An order of a node in float (F, G high parts only).
 template <int p>
-__device__ __forceinline__ void split2_tail(const Split2Const &C, Split2Node<p> &N, int k, const Split2Slots &x,
+__device__ __forceinline__ void split2_tail(const Split2Const &C, Split2Node<p> &N, const float2 *lv, const Split2Slots &x,
                                             int i0, int j0, int js, const float *gx, const float *gy, float lx,
                                             float ly, FF *F, FF *G) {
   constexpr int n = 2 * p, NL = n - 1;
@@ -290,15 +289,14 @@ __device__ __forceinline__ void split2_tail(const Split2Const &C, Split2Node<p> 
   const float m1 = __fmul_rn(v, __fadd_rn(u[1], W1)), m2 = __fmul_rn(w, __fadd_rn(u[2], W2));
   const float dp = fmaf(gm1, u[3], __fmul_rn(-kap, __fadd_rn(m1, m2)));
   const float Lp = __fadd_rn(u[3], dp), L1 = fmaf(-h, u[0], Lp);
-  const float pk = c_tab.powr[p][n - 1][k - 1];
+  const float pk = lv[NL - 1].x;
   N.Ba = fmaf(pk, fabsf(u[0]), N.Ba);
   N.Bw = fmaf(pk, fmaxf(fabsf(W1), fabsf(W2)), N.Bw);
   N.Bl = fmaf(pk, fabsf(L1), N.Bl);
   float q[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
   for (int i = 0; i < NL; i++) {
-    const int rr = i < p - 1 ? i : i + 1;
-    const float c = c_tab.powr[p][rr][k - 1], wt = c_tab.lag[p][k - 1][rr];
+    const float c = lv[i].x, wt = lv[i].y;
     N.A[i].h = fmaf(c, u[0], N.A[i].h);
     N.W1[i].h = fmaf(c, W1, N.W1[i].h);
     N.W2[i].h = fmaf(c, W2, N.W2[i].h);
@@ -327,22 +325,17 @@ __device__ __forceinline__ void split2_tail(const Split2Const &C, Split2Node<p> 
 // (840 / k) sum_r gh_r F^(k-1)_r/(k-1)! over the row j2 = 0 (direction 0) or the
 // column j1 = 0 from the slots; i0, st: first slot and stride.
 template <int p>
-__device__ __forceinline__ void split2_flux(const Split2Slots &x, int dir, int c, int i0, int st, float ck,
-                                            FF &S) {
+__device__ __forceinline__ void split2_flux(const Split2Slots &x, const SplitTab &tab, int dir, int c, int i0,
+                                            int st, float ck, FF &S) {
   const float *H = reinterpret_cast<const float *>(dir ? x.Gh : x.Fh);
   const float *Lo = reinterpret_cast<const float *>(dir ? x.Gl : x.Fl);
   FF t{0.0f, 0.0f};
 #pragma unroll
   for (int r = 0; r < 2 * p; r++) {
     const int i = (i0 + r * st) * 4 + c;
-    ff_acc(t, FF{H[i], Lo[i]}, c_tab.ghi[p][r]);
+    ff_acc(t, FF{H[i], Lo[i]}, tab.gh[p - 2][r]);
   }
   ff_acc(S, ff_norm(t), ck);
 }
-
-// -lambda / ((k-1) LC) of both directions, k = 2..2p, for p = 2..P
-struct Split2Lam {
-  SplitLam x, y;
-};
 
 }  // namespace

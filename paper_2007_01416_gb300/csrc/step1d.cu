@@ -53,6 +53,7 @@ __global__ void __launch_bounds__(NT, MinCtas<P, false>::value) k_step1d_f64(con
   const Shape64 sh = shape64<P>((int)blockDim.x, a.rounds);
   // dt by the last warp, which has the fewest cells to stage (none at R = 1)
   if (threadIdx.x == blockDim.x - 32) s_lam = step_dt(a) / a.dx;
+  if constexpr (decltype(sm)::kSplit) split_tab(sm.tab, (int)threadIdx.x, (int)blockDim.x);
   tile_f64<P, FLUX, NT / 32, MAX_ROUNDS64>(
       a, sm, sh, static_cast<const double *>(a.u_in), static_cast<double *>(a.u_out), 0, a.N, a.N,
       (long)blockIdx.x * (sh.NI - 1), &s_lam, a.orders, &a.smax[(a.slot + 1) % 3]);
@@ -363,14 +364,19 @@ int acat_launch_smax1d(int flux, int prec, const Step1DArgs &a, void *stream) {
   return (int)cudaErrorInvalidValue;
 }
 
-int acat_upload_tables_1d(const AcatTables *T) { return (int)cudaMemcpyToSymbol(c_tab, T, sizeof *T); }
+int acat_upload_tables_1d(const AcatTables *T, const SplitTab *G) {
+  const int e = (int)cudaMemcpyToSymbol(c_tab, T, sizeof *T);
+  return e ? e : (int)cudaMemcpyToSymbol(g_split, G, sizeof *G);
+}
 
 int acat_upload_tables_current_device() {
   AcatTables T;
   acat_build_tables(&T);
-  int e = acat_upload_tables_1d(&T);
-  if (e == 0) e = acat_upload_tables_2d(&T);
+  SplitTab G;
+  acat_build_split(&G);
+  int e = acat_upload_tables_1d(&T, &G);
+  if (e == 0) e = acat_upload_tables_2d(&T, &G);
   if (e == 0) e = acat_upload_tables_adj(&T);
-  if (e == 0) e = acat_upload_tables_batch(&T);
+  if (e == 0) e = acat_upload_tables_batch(&T, &G);
   return e;
 }

@@ -775,6 +775,7 @@ struct Smem64 {
   float4 xa[kSplit && S > 1 ? NW * 2 * XSET : 1];
   float2 xb[kSplit && S > 1 ? NW * 2 * XSET : 1];
   SplitLam lamk;
+  typename std::conditional<kSplit, SplitTab, char>::type tab;  // filled once per CTA by the kernel
   float du[S][TL::TW];               // u_{k+1} - u_k
   unsigned char rej[S][TL::NI];      // rejected orders per (component, interface)
   unsigned char code[TL::NI];        // p where Fs holds a pair, else 0
@@ -878,9 +879,10 @@ __device__ __forceinline__ void cat_iface_f64(const Step1DArgs &a, Smem64<P, FLU
     bool ok;
     if constexpr (FLUX == ACAT_FLUX_EULER1D) {
       const int xo = warp * 2 * XSET + (P >= 3 ? xslot(base) : base);
-      ok = cat_split_euler<p, TW>(sm.rec, a, sm.lamk.v[p - 2], ic, l, base, &sm.xa[xo], &sm.xb[xo], G);
+      ok = cat_split_euler<p, TW>(sm.rec, a, sm.tab, sm.lamk.v[p - 2], ic, l, base, &sm.xa[xo], &sm.xb[xo], G);
     } else {
-      ok = cat_split_burgers<p, TW>(sm.rec, (float)a.cfl * __frcp_rn((float)lam), sm.lamk.v[p - 2], ic, l, base, G);
+      ok = cat_split_burgers<p, TW>(sm.rec, (float)a.cfl * __frcp_rn((float)lam), sm.tab, sm.lamk.v[p - 2], ic, l,
+                                    base, G);
     }
     if (ok) {
       if (l == 0) {

@@ -1049,6 +1049,7 @@ struct Smem2S {
   Split2Rec rec[TW2 * TW2];
   float4 x[NT / 32][4][32];    // the warps' exchange slots
   SplitLam lx, ly;
+  SplitTab tab;
   double dlx, dly;
   unsigned char rej[8 * NA * NA];
   unsigned char cF[TXY][TXY + 1], cG[TXY + 1][TXY];  // 2 where the flux is a pair
@@ -1069,8 +1070,8 @@ __device__ __forceinline__ bool cat2d_split(Smem2S &sm, const Step2DArgs &a, int
   float gx[n], gy[n];
 #pragma unroll
   for (int r = 0; r < n; r++) {
-    gx[r] = c_tab.g1i[p][ia][r];
-    gy[r] = c_tab.g1i[p][ib][r];
+    gx[r] = sm.tab.g1[p - 2][ia][r];
+    gy[r] = sm.tab.g1[p - 2][ib][r];
   }
   const int i0 = base + ib * n, j0 = base + ia;
   const int dir = (l >> 2) & 1, fc = l & 3, f0 = dir ? base + p - 1 : base + (p - 1) * n, fs = dir ? n : 1;
@@ -1085,29 +1086,29 @@ __device__ __forceinline__ bool cat2d_split(Smem2S &sm, const Step2DArgs &a, int
     split2_put(xs, base + l, F, G);
     __syncwarp(mask);
     S = FF{0.0f, 0.0f};
-    if (l < 8) split2_flux<p>(xs, dir, fc, f0, fs, 840.0f, S);
+    if (l < 8) split2_flux<p>(xs, sm.tab, dir, fc, f0, fs, 840.0f, S);
     bool flt = allow, tail = false;
 #pragma unroll 1
     for (int k = 2; k <= n; k++) {
-      const float2 lx = sm.lx.v[0][k - 2], ly = sm.ly.v[0][k - 2];
+      const float2 lx = sm.lx.v[0][k - 2], ly = sm.ly.v[0][k - 2], *lv = sm.tab.lv[p - 2][k - 2];
       if (!tail && flt) tail = __all_sync(mask, split2_small(N, F, G));
       if (tail) {
-        split2_tail(C, N, k, xs, i0, j0, n, gx, gy, lx.x, ly.x, F, G);
+        split2_tail(C, N, lv, xs, i0, j0, n, gx, gy, lx.x, ly.x, F, G);
       } else {
         FF u[4];
         split2_sums<p>(xs, i0, j0, n, gx, gy, ff_of(lx), ff_of(ly), u);
         const Split2Lin o = split2_lin(C, N.v, N.w, N.h, u);
-        const float pk = c_tab.powr[p][n - 1][k - 1];
+        const float pk = lv[n - 2].x;
         N.Ba = fmaf(pk, fabsf(u[0].h), N.Ba);
         N.Bw = fmaf(pk, fmaxf(fabsf(o.W1.h), fabsf(o.W2.h)), N.Bw);
         N.Bl = fmaf(pk, fabsf(o.L.h), N.Bl);
         if (k == 2 && flt) flt = __all_sync(mask, split2_quad(N, 2.0f));
-        split2_order(C, N, k, flt, u, o, F, G);
+        split2_order(C, N, lv, flt, u, o, F, G);
       }
       __syncwarp(mask);
       split2_put(xs, base + l, F, G);
       __syncwarp(mask);
-      if (l < 8) split2_flux<p>(xs, dir, fc, f0, fs, c_tab.k840[k], S);
+      if (l < 8) split2_flux<p>(xs, sm.tab, dir, fc, f0, fs, sm.tab.k840[k - 1], S);
     }
     if (!__all_sync(mask, split2_held(N))) return false;
     if (!flt || __all_sync(mask, split2_quad(N, 1.0f))) break;
@@ -1143,6 +1144,7 @@ __global__ void __launch_bounds__(NT, 2) k_step2d_split(const Step2DArgs a) {
     split2_record(sm.rec[q], u, gm1);
   }
   for (int q = threadIdx.x; q < 2 * TXY * (TXY + 1); q += NT) (&sm.cF[0][0])[q] = 0;  // cF and cG
+  split_tab(sm.tab, threadIdx.x, NT);
   __syncthreads();
   const double lxd = sm.dlx, lyd = sm.dly;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1352,6 +1354,7 @@ struct Smem2H {
   };
   Split2Rec rec[kSplit ? TW * TW : 1];
   SplitLam slx, sly;
+  SplitTab tab;
   unsigned char cF[TXH][TXH + 1], cG[TXH + 1][TXH];  // p where the flux is a pair, else 0
   int bad[NT / 16], nfail;
   unsigned rej[NAH * NAH];    // rejected orders: bit dir * (P - 1) + (p - 2)
@@ -1637,8 +1640,8 @@ __device__ __forceinline__ void split_tasks(Smem2H<P, FLUX> &sm, const Step2DArg
   float gx[n], gy[n];
 #pragma unroll
   for (int r = 0; r < n; r++) {
-    gx[r] = c_tab.g1i[p][ia][r];
-    gy[r] = c_tab.g1i[p][ib][r];
+    gx[r] = sm.tab.g1[p - 2][ia][r];
+    gy[r] = sm.tab.g1[p - 2][ib][r];
   }
   const int i0 = ti * nn + ib * n, j0 = ti * nn + ia;
   const int dir = (node >> 2) & 1, fc = node & 3, f0 = ti * nn + (dir ? z : z * n), fs = dir ? n : 1;
@@ -1666,32 +1669,32 @@ __device__ __forceinline__ void split_tasks(Smem2H<P, FLUX> &sm, const Step2DArg
       __syncthreads();
       const bool off = !act || sm.bad[ti] != 0;  // no say in the round's votes
       S = FF{0.0f, 0.0f};
-      if (act && node < 8) split2_flux<p>(xs, dir, fc, f0, fs, 840.0f, S);
+      if (act && node < 8) split2_flux<p>(xs, sm.tab, dir, fc, f0, fs, 840.0f, S);
       bool flt = allow, tail = false;
 #pragma unroll 1
       for (int k = 2; k <= n; k++) {
-        const float2 lx = sm.slx.v[p - 2][k - 2], ly = sm.sly.v[p - 2][k - 2];
+        const float2 lx = sm.slx.v[p - 2][k - 2], ly = sm.sly.v[p - 2][k - 2], *lv = sm.tab.lv[p - 2][k - 2];
         if (!tail && flt) tail = __syncthreads_and(off || split2_small(N, F, G)) != 0;
         if (tail) {
-          if (act) split2_tail(C, N, k, xs, i0, j0, n, gx, gy, lx.x, ly.x, F, G);
+          if (act) split2_tail(C, N, lv, xs, i0, j0, n, gx, gy, lx.x, ly.x, F, G);
         } else {
           FF u[4];
           Split2Lin o;
           if (act) {
             split2_sums<p>(xs, i0, j0, n, gx, gy, ff_of(lx), ff_of(ly), u);
             o = split2_lin(C, N.v, N.w, N.h, u);
-            const float pk = c_tab.powr[p][n - 1][k - 1];
+            const float pk = lv[n - 2].x;
             N.Ba = fmaf(pk, fabsf(u[0].h), N.Ba);
             N.Bw = fmaf(pk, fmaxf(fabsf(o.W1.h), fabsf(o.W2.h)), N.Bw);
             N.Bl = fmaf(pk, fabsf(o.L.h), N.Bl);
           }
           if (k == 2 && flt) flt = __syncthreads_and(off || split2_quad(N, 2.0f)) != 0;
-          if (act) split2_order(C, N, k, flt, u, o, F, G);
+          if (act) split2_order(C, N, lv, flt, u, o, F, G);
         }
         __syncthreads();
         if (act) split2_put(xs, tid, F, G);
         __syncthreads();
-        if (act && node < 8) split2_flux<p>(xs, dir, fc, f0, fs, c_tab.k840[k], S);
+        if (act && node < 8) split2_flux<p>(xs, sm.tab, dir, fc, f0, fs, sm.tab.k840[k - 1], S);
       }
       if (!off && !split2_held(N)) sm.bad[ti] = 1;
       // (off is the state before this order's verdict: a block that fails here
@@ -1757,6 +1760,7 @@ __global__ void __launch_bounds__(NT, 1) k_step2d_hi(const Step2DArgs a) {
   }
   if constexpr (SM::kSplit)
     for (int q = tid; q < 2 * TXH * (TXH + 1); q += NT) (&sm.cF[0][0])[q] = 0;  // cF and cG
+  if constexpr (SM::kSplit) split_tab(sm.tab, tid, NT);
   __syncthreads();
   const double lx = sm.lx, ly = sm.ly;
   if constexpr (SM::kSplit) {
@@ -2351,4 +2355,7 @@ int acat_launch_smax2d(int flux, int prec, const Step2DArgs &a, void *stream) {
   return (int)cudaGetLastError();
 }
 
-int acat_upload_tables_2d(const AcatTables *T) { return (int)cudaMemcpyToSymbol(c_tab, T, sizeof *T); }
+int acat_upload_tables_2d(const AcatTables *T, const SplitTab *G) {
+  const int e = (int)cudaMemcpyToSymbol(c_tab, T, sizeof *T);
+  return e ? e : (int)cudaMemcpyToSymbol(g_split, G, sizeof *G);
+}

@@ -103,26 +103,13 @@ void acat_build_tables(AcatTables *T) {
     // gamma^{1,j}_{p,r}: first derivative at each node j
     for (int j = 0; j < n; j++) {
       lagrange_deriv(n, nodes, 1, mk(nodes[j], 1), w);
-      for (int r = 0; r < n; r++) {
-        T->g1[p][j][r] = to_d(w[r]);
-        T->g1i[p][j][r] = times(w[r], kLC[p]);
-      }
+      for (int r = 0; r < n; r++) T->g1[p][j][r] = to_d(w[r]);
     }
     // gamma^{k,0}_{p,r}: k-th derivative at 0 (time derivatives), k < 2p
-    int64_t kf = 1;
     for (int k = 0; k < n; k++) {
-      if (k > 1) kf *= k;
       lagrange_deriv(n, nodes, k, mk(0, 1), w);
-      for (int r = 0; r < n; r++) {
-        T->gk[p][k][r] = to_d(w[r]);
-        T->lag[p][k][r] = times(mul(w[r], mk(1, kf)), kLQ[p]);
-      }
+      for (int r = 0; r < n; r++) T->gk[p][k][r] = to_d(w[r]);
       if (k > 0) T->ilc[p][k] = 1.0 / (double)(k * kLC[p]);
-    }
-    {
-      const double q = 1.0 / (double)kLQ[p];
-      T->ilq[p].x = (float)q;
-      T->ilq[p].y = (float)(q - (double)T->ilq[p].x);
     }
     // gamma^{2p-1,1/2}: the binomial (2p-1)-th difference (Eq. 3.12)
     lagrange_deriv(n, nodes, n - 1, mk(1, 2), w);
@@ -136,20 +123,15 @@ void acat_build_tables(AcatTables *T) {
     for (int m = 0; m < n; m++) {
       s = add(s, neg(d[m]));
       T->gh[p][m] = to_d(s);
-      T->ghi[p][m] = times(s, kLH[p]);
     }
     // Taylor coefficients r^l / l! at the 2p time levels
     for (int rr = 0; rr < n; rr++) {
       const int r = rr - p + 1;
       Q v{1, 1};
       T->taylor[p][rr][0] = 1.0;
-      int64_t pw = 1;
-      T->powr[p][rr][0] = 1.0f;
       for (int l = 1; l < n; l++) {
         v = mul(v, mk(r, l));
         T->taylor[p][rr][l] = to_d(v);
-        pw *= r;
-        T->powr[p][rr][l] = (float)pw;
       }
     }
     // (2p-1)! for tau_p
@@ -173,6 +155,41 @@ void acat_build_tables(AcatTables *T) {
       }
     }
   }
-  for (int k = 1; k <= ACAT_MAXN; k++) T->k840[k] = (float)(840 / k);
   for (int k = 0; k <= ACAT_MAXN; k++) T->invfactf[k] = (float)T->invfact[k];
+}
+
+void acat_build_split(SplitTab *T) {
+  std::memset(T, 0, sizeof *T);
+  for (int p = 2; p <= ACAT_MAXP; p++) {
+    const int n = 2 * p;
+    int nodes[ACAT_MAXN];
+    for (int r = 0; r < n; r++) nodes[r] = r - p + 1;
+    Q w[ACAT_MAXN + 1];
+    for (int j = 0; j < n; j++) {
+      lagrange_deriv(n, nodes, 1, mk(nodes[j], 1), w);
+      for (int r = 0; r < n; r++) T->g1[p - 2][j][r] = times(w[r], kLC[p]);
+    }
+    int64_t kf = 1;
+    for (int k = 1; k < n; k++) {  // the order k + 1 takes the k-th time derivative
+      kf *= k;
+      lagrange_deriv(n, nodes, k, mk(0, 1), w);
+      for (int q = 0; q < n - 1; q++) {
+        const int rr = q < p - 1 ? q : q + 1;
+        int64_t pw = 1;
+        for (int l = 0; l < k; l++) pw *= nodes[rr];
+        T->lv[p - 2][k - 1][q].x = (float)pw;
+        T->lv[p - 2][k - 1][q].y = times(mul(w[rr], mk(1, kf)), kLQ[p]);
+      }
+    }
+    int cen[ACAT_MAXN + 1];
+    for (int r = 0; r <= n; r++) cen[r] = r - p;
+    Q d[ACAT_MAXN + 1];
+    lagrange_deriv(n + 1, cen, 1, mk(0, 1), d);
+    Q s{0, 1};
+    for (int m = 0; m < n; m++) {
+      s = add(s, neg(d[m]));
+      T->gh[p - 2][m] = times(s, kLH[p]);
+    }
+  }
+  for (int k = 1; k <= ACAT_MAXN; k++) T->k840[k - 1] = (float)(840 / k);
 }
