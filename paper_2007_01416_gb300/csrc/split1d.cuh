@@ -24,13 +24,21 @@
 //  4. Precision by magnitude. With all increments below TAU = 2^-5 of the local
 //     flux scales the float-float error is below the FP64 kernel's own rounding
 //     (CPU experiments against 64-bit-mantissa arithmetic, rms error in units of
-//     2^-53 of the flux scale at increments of 2^-5: 0.24 against 0.40 of the FP64
+//     2^-53 of the flux scale at increments of 2^-5: 0.25 against 0.40 of the FP64
 //     recursion at p = 4, 0.19 against 0.32 at p = 2; equal at 2^-3.5). Above TAU
-//     the caller evaluates the recursion in FP64. Where the quadratic terms are
-//     below 2^-23 of the scales (increments near 2^-12) q needs no more than
-//     float; and from the order on at which F^(k-2) is below 2^-28 of the scales
-//     the rest of the recursion is float. Both leave the measured error unchanged
-//     (0.19-0.21). Each decision is taken per interface, by a vote of its lanes.
+//     the caller evaluates the recursion in FP64. The remainders take one of
+//     three forms, by the size of the Taylor sums (time increments):
+//       0  in float, where the quadratic terms are below 2^-23 of the scales;
+//       1  their leading term exactly, the rest in float: with d_r = r d_1 + d'_r,
+//          the products r^2 d_1 d_1 / rho are polynomials of degree 2 in r, so
+//          their weighted sum is d_1 d_1 / rho at k = 3 and 0 otherwise (one pair);
+//          what is left is cubic, or carries the small d', and is formed without
+//          cancellation. For cubic terms below 2^-25 and d' d_1 below 2^-23;
+//       2  in pairs.
+//     From the order on at which F^(k-2) is below 2^-28 of the scales the sums
+//     are float too (forms 0 and 1). All leave the measured error unchanged
+//     (0.19-0.22). Each decision is taken per interface, by a vote of its lanes,
+//     and checked against bounds of all Taylor sums at the end.
 #pragma once
 
 #include "phys1d.cuh"
@@ -123,7 +131,16 @@ __device__ __forceinline__ double split_ginv(int p) {
 
 constexpr float SPLIT_TAU = 0x1p-5f;    // increments, of the local scales
 constexpr float SPLIT_QUAD = 0x1p-23f;  // quadratic terms that float carries
+constexpr float SPLIT_CUB = 0x1p-27f;   // form 1: cubic terms that float carries,
+constexpr float SPLIT_MIX = 0x1p-25f;   // and products of the first-order and the further terms
 constexpr float SPLIT_TAIL = 0x1p-28f;  // F^(k-2) from which on float suffices
+
+// Whether the cubic terms W W max(a, W) and W L max(a, W) are below SPLIT_CUB of
+// the scales (a of rho, w of rs, l of rh).
+__device__ __forceinline__ bool split_cubic(float a, float w, float l, float rho, float rs, float rh) {
+  const float x = __fmul_rn(a, recip(rho)), y = __fmul_rn(w, recip(rs)), z = __fmul_rn(l, recip(rh));
+  return __fmul_rn(__fmul_rn(y, fmaxf(y, z)), fmaxf(x, y)) <= SPLIT_CUB;
+}
 
 // A scale that the pairs carry: their low parts (2^-53 of it) stay normal floats
 // and so do products of two scales.

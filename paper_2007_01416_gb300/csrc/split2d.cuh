@@ -130,6 +130,10 @@ struct Split2Node {
   float rs, rh, rhs;  // scales of rho v, of pressure and of energy flux
   FF A[NL], W1[NL], W2[NL], L[NL];
   float Ba, Bw, Bl;   // bounds of the Taylor sums
+  int form;           // of the remainders (split1d.cuh): 0, 1 or 2, the same for all nodes of a vote
+  FF w1, w2, l1;      // form 1: the first-order terms,
+  float q1[5];        // their products over rho (float),
+  float Pw, Pl;       // and their bounds p |W1|, p |L1|
 };
 
 // Loads node `r` of the block anchored at record `ra`; returns
@@ -157,7 +161,10 @@ __device__ __forceinline__ bool split2_start(const Split2Const &C, const Split2R
   N.rs = __fmul_rn(uh.x, r.hs.z);
   N.rh = __fmul_rn(uh.x, r.hs.x);
   N.rhs = __fmul_rn(N.rh, r.hs.z);
-  N.Ba = N.Bw = N.Bl = 0.0f;
+  N.Ba = N.Bw = N.Bl = N.Pw = N.Pl = 0.0f;
+  N.w1 = N.w2 = N.l1 = FF{0.0f, 0.0f};
+#pragma unroll
+  for (int q = 0; q < 5; q++) N.q1[q] = 0.0f;
 #pragma unroll
   for (int q = 0; q < Split2Node<p>::NL; q++) {
     N.A[q] = N.rho;
@@ -186,6 +193,96 @@ template <int p>
 __device__ __forceinline__ bool split2_quad(const Split2Node<p> &N, float m) {
   const float bw = m * N.Bw, bl = m * N.Bl;
   return bw * bw <= SPLIT_QUAD * N.rs * N.rs && bw * bl <= SPLIT_QUAD * N.rs * N.rh;
+}
+template <int p>
+__device__ __forceinline__ bool split2_cubic(const Split2Node<p> &N, float m) {
+  return split_cubic(m * N.Ba, m * N.Bw, m * N.Bl, N.rho.h, N.rs, N.rh);
+}
+// After the last order: whether the form of the remainders held.
+template <int p>
+__device__ __forceinline__ bool split2_form(const Split2Node<p> &N) {
+  if (N.form == 0) return split2_quad(N, 1.0f);
+  if (N.form == 2) return true;
+  const float dw = N.Bw - N.Pw, dl = N.Bl - N.Pl;
+  return split2_cubic(N, 1.0f) && dw * N.Bw <= SPLIT_MIX * N.rs * N.rs && dw * N.Bl <= SPLIT_MIX * N.rs * N.rh &&
+         dl * N.Bw <= SPLIT_MIX * N.rs * N.rh;
+}
+// The bounds after an order's U (float parts), and at k = 2 the terms of form 1.
+template <int p>
+__device__ __forceinline__ void split2_bounds(Split2Node<p> &N, const float2 *lv, float a, float w1, float w2, float l) {
+  const float pk = lv[Split2Node<p>::NL - 1].x;  // p^(k-1)
+  N.Ba = fmaf(pk, fabsf(a), N.Ba);
+  N.Bw = fmaf(pk, fmaxf(fabsf(w1), fabsf(w2)), N.Bw);
+  N.Bl = fmaf(pk, fabsf(l), N.Bl);
+}
+template <int p>
+__device__ __forceinline__ void split2_first(Split2Node<p> &N, const Split2Lin &o) {
+  N.w1 = o.W1;
+  N.w2 = o.W2;
+  N.l1 = o.L;
+  N.Pw = N.Bw;
+  N.Pl = N.Bl;
+  const float ri = recip(N.rho.h), v = __fmul_rn(o.W1.h, ri), w = __fmul_rn(o.W2.h, ri);
+  N.q1[0] = __fmul_rn(o.W1.h, v);
+  N.q1[1] = __fmul_rn(o.W1.h, w);
+  N.q1[2] = __fmul_rn(o.W2.h, w);
+  N.q1[3] = __fmul_rn(o.L.h, v);
+  N.q1[4] = __fmul_rn(o.L.h, w);
+}
+// The weighted sums of an order's remainders in forms 0 and 1 (without the leading
+// terms of form 1).
+template <int p>
+__device__ __forceinline__ void split2_levels(Split2Node<p> &N, float kap, int k, const float2 *lv, float a,
+                                              float w1, float w2, float l, float *q) {
+  constexpr int NL = Split2Node<p>::NL;
+#pragma unroll
+  for (int e = 0; e < 5; e++) q[e] = 0.0f;
+  if (N.form == 0) {
+#pragma unroll
+    for (int i = 0; i < NL; i++) {
+      const float c = lv[i].x, wt = lv[i].y;
+      N.A[i].h = fmaf(c, a, N.A[i].h);
+      N.W1[i].h = fmaf(c, w1, N.W1[i].h);
+      N.W2[i].h = fmaf(c, w2, N.W2[i].h);
+      N.L[i].h = fmaf(c, l, N.L[i].h);
+      float t[5];
+      split2_termsf(kap, N.A[i].h, N.W1[i].h, N.W2[i].h, N.L[i].h, t);
+#pragma unroll
+      for (int e = 0; e < 5; e++) q[e] = fmaf(wt, t[e], q[e]);
+    }
+  } else {
+    if (k == 2) {  // A without rho, the others without their first-order terms
+#pragma unroll
+      for (int i = 0; i < NL; i++) N.A[i].h = 0.0f;
+      w1 = w2 = l = 0.0f;
+    }
+#pragma unroll
+    for (int i = 0; i < NL; i++) {
+      const float r = (float)(i < p - 1 ? i - p + 1 : i - p + 2), c = lv[i].x, wt = lv[i].y;
+      N.A[i].h = fmaf(c, a, N.A[i].h);
+      N.W1[i].h = fmaf(c, w1, N.W1[i].h);
+      N.W2[i].h = fmaf(c, w2, N.W2[i].h);
+      N.L[i].h = fmaf(c, l, N.L[i].h);
+      const float R = recip(__fadd_rn(N.rho.h, N.A[i].h)), ra = __fmul_rn(-(r * r), N.A[i].h);
+      const float x1 = __fmul_rn(r, N.w1.h), x2 = __fmul_rn(r, N.w2.h);
+      const float y1 = __fadd_rn(x1, N.W1[i].h), y2 = __fadd_rn(x2, N.W2[i].h), yl = fmaf(r, N.l1.h, N.L[i].h);
+      // products of the sums less their leading part, r^2 q1 (1 + a / rho)
+      const float n0 = fmaf(ra, N.q1[0], __fmul_rn(N.W1[i].h, __fadd_rn(x1, y1)));
+      const float n1 = fmaf(ra, N.q1[1], fmaf(N.W1[i].h, y2, __fmul_rn(x1, N.W2[i].h)));
+      const float n2 = fmaf(ra, N.q1[2], __fmul_rn(N.W2[i].h, __fadd_rn(x2, y2)));
+      const float n3 = fmaf(ra, N.q1[3], fmaf(N.W1[i].h, yl, __fmul_rn(x1, N.L[i].h)));
+      const float n4 = fmaf(ra, N.q1[4], fmaf(N.W2[i].h, yl, __fmul_rn(x2, N.L[i].h)));
+      const float t0 = __fmul_rn(n0, R), t2 = __fmul_rn(n2, R);
+      const float kq = __fmul_rn(-kap, fmaf(r * r, __fadd_rn(N.q1[0], N.q1[2]), __fadd_rn(t0, t2)));
+      q[0] = fmaf(wt, t0, q[0]);
+      q[1] = fmaf(wt, __fmul_rn(n1, R), q[1]);
+      q[2] = fmaf(wt, t2, q[2]);
+      q[3] = fmaf(wt, __fmul_rn(R, fmaf(y1, kq, n3)), q[3]);
+      q[4] = fmaf(wt, __fmul_rn(R, fmaf(y2, kq, n4)), q[4]);
+    }
+  }
+#pragma unroll
+  for (int e = 0; e < 5; e++) q[e] = __fmul_rn(q[e], 1.0f / split_lq(p));
 }
 
 // U^(k-1)/(k-1)! of a node from the slots of its row (i0 + r) and its column
@@ -217,29 +314,27 @@ __device__ __forceinline__ void split2_sums(const Split2Slots &x, int i0, int j0
   for (int c = 0; c < 4; c++) u[c] = ff_add(ff_mul(ff_norm(a[c]), lx), ff_mul(ff_norm(b[c]), ly));
 }
 
-// An order of a node in pairs (lv: the order's level weights); flt: remainders in
-// float. u: from split2_sums.
+// Order k of a node in pairs, the remainders in the node's form. u: from
+// split2_sums, o: from split2_lin.
 template <int p>
-__device__ __forceinline__ void split2_order(const Split2Const &C, Split2Node<p> &N, const float2 *lv, bool flt,
+__device__ __forceinline__ void split2_order(const Split2Const &C, Split2Node<p> &N, int k, const float2 *lv,
                                              const FF *u, const Split2Lin &o, FF *F, FF *G) {
   constexpr int NL = 2 * p - 1;
-  if (flt) {
-    float q[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-#pragma unroll
-    for (int i = 0; i < NL; i++) {
-      const float c = lv[i].x, wt = lv[i].y;
-      N.A[i].h = fmaf(c, u[0].h, N.A[i].h);
-      N.W1[i].h = fmaf(c, o.W1.h, N.W1[i].h);
-      N.W2[i].h = fmaf(c, o.W2.h, N.W2[i].h);
-      N.L[i].h = fmaf(c, o.L.h, N.L[i].h);
-      float t[5];
-      split2_termsf(C.kap.h, N.A[i].h, N.W1[i].h, N.W2[i].h, N.L[i].h, t);
-#pragma unroll
-      for (int e = 0; e < 5; e++) q[e] = fmaf(wt, t[e], q[e]);
-    }
-#pragma unroll
-    for (int e = 0; e < 5; e++) q[e] = __fmul_rn(q[e], 1.0f / split_lq(p));
+  if (N.form < 2) {
+    float q[5];
+    split2_levels(N, C.kap.h, k, lv, u[0].h, o.W1.h, o.W2.h, o.L.h, q);
     split2_remf(C, N.v, N.w, u, o, q, F, G);
+    if (k == 3 && N.form == 1) {  // the leading terms
+      const float ri = recip(N.rho.h);
+      const FF dv = ff_quot(N.w1, N.rho, ri), dw = ff_quot(N.w2, N.rho, ri);
+      const FF q0 = ff_mul(N.w1, dv), q2 = ff_mul(N.w2, dw), kq = ff_mul(C.kap, ff_add(q0, q2));
+      F[1] = ff_add(F[1], ff_add(q0, ff_neg(kq)));
+      F[2] = ff_add(F[2], ff_mul(N.w1, dw));
+      F[3] = ff_add(F[3], ff_add(ff_mul(dv, N.l1), ff_neg(ff_mul(N.v, kq))));
+      G[1] = F[2];
+      G[2] = ff_add(G[2], ff_add(q2, ff_neg(kq)));
+      G[3] = ff_add(G[3], ff_add(ff_mul(dw, N.l1), ff_neg(ff_mul(N.w, kq))));
+    }
   } else {
     FF q[5];
 #pragma unroll
@@ -263,12 +358,12 @@ __device__ __forceinline__ void split2_order(const Split2Const &C, Split2Node<p>
   }
 }
 
-// An order of a node in float (F, G high parts only).
+// Order k of a node in float (F, G high parts only).
 template <int p>
-__device__ __forceinline__ void split2_tail(const Split2Const &C, Split2Node<p> &N, const float2 *lv, const Split2Slots &x,
+__device__ __forceinline__ void split2_tail(const Split2Const &C, Split2Node<p> &N, int k, const float2 *lv, const Split2Slots &x,
                                             int i0, int j0, int js, const float *gx, const float *gy, float lx,
                                             float ly, FF *F, FF *G) {
-  constexpr int n = 2 * p, NL = n - 1;
+  constexpr int n = 2 * p;
   float a[4] = {0.0f, 0.0f, 0.0f, 0.0f}, b[4] = {0.0f, 0.0f, 0.0f, 0.0f}, u[4];
 #pragma unroll
   for (int r = 0; r < n; r++) {
@@ -289,25 +384,13 @@ __device__ __forceinline__ void split2_tail(const Split2Const &C, Split2Node<p> 
   const float m1 = __fmul_rn(v, __fadd_rn(u[1], W1)), m2 = __fmul_rn(w, __fadd_rn(u[2], W2));
   const float dp = fmaf(gm1, u[3], __fmul_rn(-kap, __fadd_rn(m1, m2)));
   const float Lp = __fadd_rn(u[3], dp), L1 = fmaf(-h, u[0], Lp);
-  const float pk = lv[NL - 1].x;
-  N.Ba = fmaf(pk, fabsf(u[0]), N.Ba);
-  N.Bw = fmaf(pk, fmaxf(fabsf(W1), fabsf(W2)), N.Bw);
-  N.Bl = fmaf(pk, fabsf(L1), N.Bl);
-  float q[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+  split2_bounds(N, lv, u[0], W1, W2, L1);
+  float q[5];
+  split2_levels(N, kap, k, lv, u[0], W1, W2, L1, q);
+  if (k == 3) {  // the leading terms (0 in form 0)
 #pragma unroll
-  for (int i = 0; i < NL; i++) {
-    const float c = lv[i].x, wt = lv[i].y;
-    N.A[i].h = fmaf(c, u[0], N.A[i].h);
-    N.W1[i].h = fmaf(c, W1, N.W1[i].h);
-    N.W2[i].h = fmaf(c, W2, N.W2[i].h);
-    N.L[i].h = fmaf(c, L1, N.L[i].h);
-    float t[5];
-    split2_termsf(kap, N.A[i].h, N.W1[i].h, N.W2[i].h, N.L[i].h, t);
-#pragma unroll
-    for (int e = 0; e < 5; e++) q[e] = fmaf(wt, t[e], q[e]);
+    for (int e = 0; e < 5; e++) q[e] = __fadd_rn(q[e], N.q1[e]);
   }
-#pragma unroll
-  for (int e = 0; e < 5; e++) q[e] = __fmul_rn(q[e], 1.0f / split_lq(p));
   const float kq = __fmul_rn(kap, __fadd_rn(q[0], q[2]));
   F[0].h = u[1];
   F[1].h = __fadd_rn(__fadd_rn(m1, dp), __fsub_rn(q[0], kq));

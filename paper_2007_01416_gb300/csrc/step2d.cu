@@ -1075,7 +1075,7 @@ __device__ __forceinline__ bool cat2d_split(Smem2S &sm, const Step2DArgs &a, int
   }
   const int i0 = base + ib * n, j0 = base + ia;
   const int dir = (l >> 2) & 1, fc = l & 3, f0 = dir ? base + p - 1 : base + (p - 1) * n, fs = dir ? n : 1;
-  bool allow = true;
+  int form = 0;
 #pragma unroll 1
   for (;;) {
     Split2Node<p> N;
@@ -1087,23 +1087,27 @@ __device__ __forceinline__ bool cat2d_split(Smem2S &sm, const Step2DArgs &a, int
     __syncwarp(mask);
     S = FF{0.0f, 0.0f};
     if (l < 8) split2_flux<p>(xs, sm.tab, dir, fc, f0, fs, 840.0f, S);
-    bool flt = allow, tail = false;
+    N.form = form;
+    bool tail = false;
 #pragma unroll 1
     for (int k = 2; k <= n; k++) {
       const float2 lx = sm.lx.v[0][k - 2], ly = sm.ly.v[0][k - 2], *lv = sm.tab.lv[p - 2][k - 2];
-      if (!tail && flt) tail = __all_sync(mask, split2_small(N, F, G));
+      if (!tail && N.form < 2 && (k > 2 || N.form == 0)) tail = __all_sync(mask, split2_small(N, F, G));
       if (tail) {
-        split2_tail(C, N, lv, xs, i0, j0, n, gx, gy, lx.x, ly.x, F, G);
+        split2_tail(C, N, k, lv, xs, i0, j0, n, gx, gy, lx.x, ly.x, F, G);
       } else {
         FF u[4];
         split2_sums<p>(xs, i0, j0, n, gx, gy, ff_of(lx), ff_of(ly), u);
         const Split2Lin o = split2_lin(C, N.v, N.w, N.h, u);
-        const float pk = lv[n - 2].x;
-        N.Ba = fmaf(pk, fabsf(u[0].h), N.Ba);
-        N.Bw = fmaf(pk, fmaxf(fabsf(o.W1.h), fabsf(o.W2.h)), N.Bw);
-        N.Bl = fmaf(pk, fabsf(o.L.h), N.Bl);
-        if (k == 2 && flt) flt = __all_sync(mask, split2_quad(N, 2.0f));
-        split2_order(C, N, lv, flt, u, o, F, G);
+        split2_bounds(N, lv, u[0].h, o.W1.h, o.W2.h, o.L.h);
+        if (k == 2) {
+          if (N.form == 0 && !__all_sync(mask, split2_quad(N, 2.0f))) N.form = 1;
+          if (N.form == 1) {
+            if (!__all_sync(mask, split2_cubic(N, 1.6f))) N.form = 2;
+            split2_first(N, o);
+          }
+        }
+        split2_order(C, N, k, lv, u, o, F, G);
       }
       __syncwarp(mask);
       split2_put(xs, base + l, F, G);
@@ -1111,8 +1115,8 @@ __device__ __forceinline__ bool cat2d_split(Smem2S &sm, const Step2DArgs &a, int
       if (l < 8) split2_flux<p>(xs, sm.tab, dir, fc, f0, fs, sm.tab.k840[k - 1], S);
     }
     if (!__all_sync(mask, split2_held(N))) return false;
-    if (!flt || __all_sync(mask, split2_quad(N, 1.0f))) break;
-    allow = false;
+    if (__all_sync(mask, split2_form(N))) break;
+    form = N.form + 1;
   }
   return true;
 }
@@ -1652,7 +1656,7 @@ __device__ __forceinline__ void split_tasks(Smem2H<P, FLUX> &sm, const Step2DArg
     const unsigned tk = act ? sm.task[p][base + ti] : 0u;
     const int an = (int)(tk & 0xffu);
     const int ax = an % NAH - 1, ay = an / NAH - 1;
-    bool allow = true;
+    int form = 0;
     FF S;
 #pragma unroll 1
     for (;;) {
@@ -1670,26 +1674,31 @@ __device__ __forceinline__ void split_tasks(Smem2H<P, FLUX> &sm, const Step2DArg
       const bool off = !act || sm.bad[ti] != 0;  // no say in the round's votes
       S = FF{0.0f, 0.0f};
       if (act && node < 8) split2_flux<p>(xs, sm.tab, dir, fc, f0, fs, 840.0f, S);
-      bool flt = allow, tail = false;
+      N.form = form;
+      bool tail = false;
 #pragma unroll 1
       for (int k = 2; k <= n; k++) {
         const float2 lx = sm.slx.v[p - 2][k - 2], ly = sm.sly.v[p - 2][k - 2], *lv = sm.tab.lv[p - 2][k - 2];
-        if (!tail && flt) tail = __syncthreads_and(off || split2_small(N, F, G)) != 0;
+        if (!tail && N.form < 2 && (k > 2 || N.form == 0))
+          tail = __syncthreads_and(off || split2_small(N, F, G)) != 0;
         if (tail) {
-          if (act) split2_tail(C, N, lv, xs, i0, j0, n, gx, gy, lx.x, ly.x, F, G);
+          if (act) split2_tail(C, N, k, lv, xs, i0, j0, n, gx, gy, lx.x, ly.x, F, G);
         } else {
           FF u[4];
           Split2Lin o;
           if (act) {
             split2_sums<p>(xs, i0, j0, n, gx, gy, ff_of(lx), ff_of(ly), u);
             o = split2_lin(C, N.v, N.w, N.h, u);
-            const float pk = lv[n - 2].x;
-            N.Ba = fmaf(pk, fabsf(u[0].h), N.Ba);
-            N.Bw = fmaf(pk, fmaxf(fabsf(o.W1.h), fabsf(o.W2.h)), N.Bw);
-            N.Bl = fmaf(pk, fabsf(o.L.h), N.Bl);
+            split2_bounds(N, lv, u[0].h, o.W1.h, o.W2.h, o.L.h);
           }
-          if (k == 2 && flt) flt = __syncthreads_and(off || split2_quad(N, 2.0f)) != 0;
-          if (act) split2_order(C, N, lv, flt, u, o, F, G);
+          if (k == 2) {
+            if (N.form == 0 && !__syncthreads_and(off || split2_quad(N, 2.0f))) N.form = 1;
+            if (N.form == 1) {
+              if (!__syncthreads_and(off || split2_cubic(N, 1.6f))) N.form = 2;
+              if (act) split2_first(N, o);
+            }
+          }
+          if (act) split2_order(C, N, k, lv, u, o, F, G);
         }
         __syncthreads();
         if (act) split2_put(xs, tid, F, G);
@@ -1699,8 +1708,8 @@ __device__ __forceinline__ void split_tasks(Smem2H<P, FLUX> &sm, const Step2DArg
       if (!off && !split2_held(N)) sm.bad[ti] = 1;
       // (off is the state before this order's verdict: a block that fails here
       // has no say in whether the round repeats)
-      if (!flt || __syncthreads_and(off || !split2_held(N) || split2_quad(N, 1.0f))) break;
-      allow = false;
+      if (__syncthreads_and(off || !split2_held(N) || split2_form(N))) break;
+      form = N.form + 1;
     }
     __syncthreads();
     if (act) {
@@ -1726,7 +1735,7 @@ __device__ __forceinline__ void split_tasks(Smem2H<P, FLUX> &sm, const Step2DArg
 }
 
 template <int P, int FLUX>
-__global__ void __launch_bounds__(NT, 1) k_step2d_hi(const Step2DArgs a) {
+__global__ void __launch_bounds__(NT, P <= 3 ? 2 : 1) k_step2d_hi(const Step2DArgs a) {
   using PH = Phys2<FLUX>;
   constexpr int S = PH::S;
   constexpr int TW = Smem2H<P, FLUX>::TW;

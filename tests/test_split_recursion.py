@@ -1,7 +1,7 @@
 """The FP64 flux recursion in float-float pairs against the oracle over every
 range that selects one of its forms: increments of 2^-2 (FP64 evaluation), of
-2^-5..2^-10 (pairs), around 2^-12 (float remainders), 2^-20 and 2^-40 (float
-from a middle order on), states at rest and in units far from 1 (beyond the
+2^-5..2^-8 (pairs), to 2^-10 (leading terms in pairs), around 2^-12 (float
+remainders), 2^-20 and 2^-40 (float from a middle order on), states at rest and in units far from 1 (beyond the
 pairs' exponent range at 1e-18 and 1e18), grids whose tiles are ragged.
 
 Bar: an element is formed from u_i, lambda F_{i-1/2} and lambda F_{i+1/2}. Both
@@ -44,7 +44,7 @@ def _state(flux, nx, amp, unit, seed):
 @pytest.mark.parametrize("flux", [W.EULER1D, W.BURGERS])
 @pytest.mark.parametrize("P", [2, 3, 4])
 @pytest.mark.parametrize("nx,log2amp,unit", [(33, -2, 1.0), (97, -3, 1.0), (333, -2, 1.0), (1001, -1, 1.0),
-                                             (777, -6, 1e5), (1500, -12, 1.0), (401, -40, 1.0), (256, -5, 1e-12),
+                                             (777, -6, 1e5), (1500, -12, 1.0), (700, -4, 1.0), (2500, -5, 1.0), (401, -40, 1.0), (256, -5, 1e-12),
                                              (256, -5, 1e-18), (256, -5, 1e18), (12001, -2, 1.0), (40001, -3, 1.0)])
 def test_step_over_the_increment_ranges(env, flux, P, nx, log2amp, unit):
     torch, O, acat = env
