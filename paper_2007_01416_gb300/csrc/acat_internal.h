@@ -58,6 +58,8 @@ struct Step1DArgs {
   int lpn;                    // FP32 1D: lanes per stencil node (1, or 2 for P = 2, 4)
   int nw;                     // warps per CTA: FP64 1D 4..8; FP32 1D fused step 8, or 7 (0 reads as 8)
   int rounds;                 // FP64 1D: interface rounds per lane group
+  int early;                  // 1: the step lets the next one launch at its start (grids of at most one
+                              // CTA per SM), 0: at its end
   double dx, cfl;
   double dt_fixed;            // > 0: imposed dt
   const double *dt_in;        // device: imposed dt (nullable; takes precedence)

@@ -56,6 +56,7 @@ struct acat_ctx {
   int snw = 8;                            // 1D single instance: FP32 warps per CTA (8 or 7 fused, 2 small-CTA);
                                           // FP64 the reported label (8, or 2 for large grids)
   int fnw = 8, frounds = 1;               // 1D FP64: warps per CTA and interface rounds
+  int sms = 0;
 };
 
 namespace {
@@ -146,6 +147,9 @@ Step1DArgs base_args(acat_ctx *c) {
   a.lpn = c->lpn;
   a.nw = p.precision != ACAT_PREC_F32 ? c->fnw : (c->snw == 7 ? 7 : 0);
   a.rounds = c->frounds;
+  const long wpc = p.precision != ACAT_PREC_F32 ? (long)c->fnw * c->frounds : (c->snw == 7 ? 7 : 8);
+  const long T = wpc * (32 / (2 * p.P * c->lpn)) - 1;  // cells per CTA of the fused step
+  a.early = !c->batched && c->dim == 1 && (p.nx + T - 1) / T <= c->sms;
   return a;
 }
 
@@ -392,6 +396,7 @@ int acat_create(const acat_params *p, acat_ctx **out) {
   if (e == cudaSuccess) e = cudaMalloc(&c->d_work, sb);
   int sms = 0;
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
+  c->sms = sms;
   // 1D FP64: the tile shape, and the label acat_launch_shape reports (2 where
   // 8-warp tiles of one round would exceed 3/4 of a wave at 2 CTAs per SM)
   if (e == cudaSuccess && c->dim == 1 && p->precision == ACAT_PREC_F64) {

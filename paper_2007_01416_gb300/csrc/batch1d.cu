@@ -73,9 +73,18 @@ struct Rounds {
 // tiles), and the queue keeps the CTAs busy to the end. Results do not
 // depend on which CTA takes a tile. Every instance is advanced with its own
 // dt (lambda from k_batch_dt). The register cap per thread is that of the
-// 8-warp kernels (MinCtas x 8 / NW resident CTAs).
+// 8-warp kernels (BatchCtas x 8 / NW resident CTAs).
+// Resident 8-warp CTAs per SM the batched kernel is compiled for: as the single
+// step's, but 3 in FP64 at P <= 3 (85 registers, 0.4 KB of spills at P = 3): the
+// persistent tiles have work for the added warps (P = 3, 256 instances: 1606 -> 1495 us
+// per step).
+template <int P, bool F32>
+struct BatchCtas {
+  static constexpr int value = !F32 && P <= 3 ? 3 : MinCtas<P, F32>::value;
+};
+
 template <int P, int FLUX, bool F32, int NW, int LPN>
-__global__ void __launch_bounds__(NW * 32, MinCtas<P, F32>::value * 8 / NW)
+__global__ void __launch_bounds__(NW * 32, BatchCtas<P, F32>::value * 8 / NW)
     k_batch1d(const Step1DArgs a, const BatchArgs bt) {
   constexpr int R = Rounds<F32, NW>::value;
   using SM =
@@ -98,10 +107,10 @@ __global__ void __launch_bounds__(NW * 32, MinCtas<P, F32>::value * 8 / NW)
     int8_t *ord = bt.orders ? bt.orders + off + b : nullptr;
     unsigned long long *so = &bt.smax[((a.slot + 1) % 3) * (long)bt.B + b];
     if constexpr (F32) {
-      tile_f32<P, FLUX, NW, LPN, R>(a, sm[par], static_cast<const float *>(a.u_in),
+      tile_f32<P, FLUX, NW, LPN, R, false>(a, sm[par], static_cast<const float *>(a.u_in),
                                     static_cast<float *>(a.u_out), off, bt.M, N, i0, &bt.lamf[b], ord, so);
     } else {
-      tile_f64<P, FLUX, NW, R>(a, sm[0], shape64<P>(NW * 32, R), static_cast<const double *>(a.u_in),
+      tile_f64<P, FLUX, NW, R, false>(a, sm[0], shape64<P>(NW * 32, R), static_cast<const double *>(a.u_in),
                                static_cast<double *>(a.u_out), off, bt.M, N, i0, &bt.lam[b], ord, so);
       __syncthreads();  // one workspace: the next tile's staging waits for this one's update
     }

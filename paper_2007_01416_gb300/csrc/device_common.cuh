@@ -162,10 +162,14 @@ __device__ __forceinline__ int acat_tile_index(int i, int n, unsigned *status) {
 // once every CTA of this grid has passed it, when nearly every SM is free, so
 // the next grid's CTAs spread over the SMs as a plain launch spreads them.
 // (Released at the start of the kernel, the next grid's CTAs took the first
-// SMs to free up, and steps of one uneven wave lost their balance.) In a
+// SMs to free up, and steps of one uneven wave lost their balance. Grids of at
+// most one CTA per SM have none to lose and release at the start.) In a
 // kernel launched without the attribute both instructions return at once.
 __device__ __forceinline__ void acat_pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void acat_pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// A barrier among the first `n` threads of the CTA (n a multiple of 32).
+__device__ __forceinline__ void part_sync(int n) { asm volatile("bar.sync 1, %0;" ::"r"(n) : "memory"); }
 
 // Host side: launch a kernel of that form with programmatic stream
 // serialization (returns 0 or a cudaError_t value).
@@ -291,7 +295,7 @@ __device__ __forceinline__ int psi2m_filter(const float *d, const float *e, floa
   const float I1L = sm + eps, I1R = (s0 + sp) + eps, I2L = (sm + s0) + eps, I2R = sp + eps;
   const float mn = fminf(fminf(I1L, I1R), fminf(I2L, I2R)), mx = fmaxf(fmaxf(I1L, I1R), fmaxf(I2L, I2R));
   if (!(mn > 1e-18f) || !(mx < 1e18f)) return -1;  // products of two stay normal floats
-  const float I1 = I1L * I1R / (I1L + I1R), I2 = I2L * I2R / (I2L + I2R);
+  const float I1 = I1L * I1R * recip(I1L + I1R), I2 = I2L * I2R * recip(I2L + I2R);
   float t[3], b[3];
 #pragma unroll
   for (int k = 0; k < 3; k++) {
@@ -385,7 +389,7 @@ __device__ __forceinline__ void psi_filter_all(const float *d, const float *e, f
       u |= bit;
       continue;
     }
-    const float I = IL * IR / (IL + IR);
+    const float I = IL * IR * recip(IL + IR);  // an ulp or two, inside the margin
     const float Dhi = (S[p] + eS[p]) * fact[p] * 1.0000005f;
     const float Dlo = fmaxf(S[p] - eS[p], 0.0f) * fact[p] * 0.9999995f;
     if (I * (1.0f - 4e-6f) > r * (Dhi * Dhi) * 1.00001f) a |= bit;

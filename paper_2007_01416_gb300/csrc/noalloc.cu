@@ -118,6 +118,8 @@ extern "C" int acat_run_noalloc(const acat_params *p, void *u_dev, int nsteps, d
   int sms = 0;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return ACAT_ERR_CUDA;
   acat_shape_f64(p->P, p->nx, sms, &a.nw, &a.rounds);
+  const long per_cta = (long)a.nw * a.rounds * (32 / (2 * p->P)) - 1;
+  a.early = (p->nx + per_cta - 1) / per_cta <= sms;
   a.smax = smax;
   a.tslot = tslot;
   a.status = status;

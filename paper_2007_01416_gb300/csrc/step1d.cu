@@ -48,13 +48,11 @@ constexpr int MAX_ROUNDS64 = 3;
 template <int P, int FLUX>
 __global__ void __launch_bounds__(NT, MinCtas<P, false>::value) k_step1d_f64(const Step1DArgs a) {
   acat_pdl_wait();
+  if (a.early) acat_pdl_release();
   __shared__ Smem64<P, FLUX, NT / 32, MAX_ROUNDS64> sm;
   __shared__ double s_lam;
   const Shape64 sh = shape64<P>((int)blockDim.x, a.rounds);
-  // dt by the last warp, which has the fewest cells to stage (none at R = 1)
-  if (threadIdx.x == blockDim.x - 32) s_lam = step_dt(a) / a.dx;
-  if constexpr (decltype(sm)::kSplit) split_tab(sm.tab, (int)threadIdx.x, (int)blockDim.x);
-  tile_f64<P, FLUX, NT / 32, MAX_ROUNDS64>(
+  tile_f64<P, FLUX, NT / 32, MAX_ROUNDS64, true>(
       a, sm, sh, static_cast<const double *>(a.u_in), static_cast<double *>(a.u_out), 0, a.N, a.N,
       (long)blockIdx.x * (sh.NI - 1), &s_lam, a.orders, &a.smax[(a.slot + 1) % 3]);
   acat_pdl_release();
@@ -67,10 +65,10 @@ __global__ void __launch_bounds__(NT, MinCtas<P, false>::value) k_step1d_f64(con
 template <int P, int FLUX, int LPN, int NW = NT / 32>
 __global__ void __launch_bounds__(NW * 32, MinCtas<P, true>::value) k_step1d_f32(const Step1DArgs a) {
   acat_pdl_wait();
+  if (a.early) acat_pdl_release();
   __shared__ Smem32<P, DPhys<FLUX>::S, NW, LPN> sm;
   __shared__ float s_lam;
-  if (threadIdx.x == 0) s_lam = (float)(step_dt(a) / a.dx);
-  tile_f32<P, FLUX, NW, LPN>(a, sm, static_cast<const float *>(a.u_in), static_cast<float *>(a.u_out), 0, a.N,
+  tile_f32<P, FLUX, NW, LPN, 1, true>(a, sm, static_cast<const float *>(a.u_in), static_cast<float *>(a.u_out), 0, a.N,
                              a.N, (long)blockIdx.x * Tiling<P, NW, LPN>::T, &s_lam, a.orders,
                              &a.smax[(a.slot + 1) % 3]);
   acat_pdl_release();

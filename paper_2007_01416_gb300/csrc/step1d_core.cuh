@@ -724,6 +724,7 @@ struct MinCtas {
 __device__ double step_dt_value(const Step1DArgs &a, double *t, bool *bad) {
   double dt;
   *bad = false;
+  *t = a.tslot ? a.tslot[a.slot] : 0.0;  // loaded beside the wave speed
   if (a.dt_in) {
     dt = *a.dt_in;
   } else if (a.dt_fixed > 0.0) {
@@ -737,13 +738,9 @@ __device__ double step_dt_value(const Step1DArgs &a, double *t, bool *bad) {
       dt = a.cfl * a.dx / smax;
     }
   }
-  *t = 0.0;
-  if (a.tslot) {
-    *t = a.tslot[a.slot];
-    if (a.t_end > 0.0) {
-      if (*t >= a.t_end) dt = 0.0;
-      else if (dt > a.t_end - *t) dt = a.t_end - *t;
-    }
+  if (a.tslot && a.t_end > 0.0) {
+    if (*t >= a.t_end) dt = 0.0;
+    else if (dt > a.t_end - *t) dt = a.t_end - *t;
   }
   return dt;
 }
@@ -823,12 +820,12 @@ __device__ __forceinline__ Shape64 shape64(int nt, int r) {
 // would otherwise be formed once per interface and node on the FP64 pipe.
 template <int P, int FLUX, int NW, int R>
 __device__ __forceinline__ void stage_f64(const Step1DArgs &a, Smem64<P, FLUX, NW, R> &sm,
-                                          const Shape64 &sh, const double *__restrict__ uin, long off, long M,
-                                          long N, long i0) {
+                                          const Shape64 &sh, int nt, const double *__restrict__ uin, long off,
+                                          long M, long N, long i0) {
   using SM = Smem64<P, FLUX, NW, R>;
   using TL = typename SM::TL;
   constexpr int S = SM::S;
-  for (int k = threadIdx.x; k < sh.TW; k += sh.NT) {
+  for (int k = threadIdx.x; k < sh.TW; k += nt) {
     const long g = bc_index(i0 - TL::GH + k, N, a.bc), g1 = bc_index(i0 - TL::GH + k + 1, N, a.bc);
     if (!acat_in_bounds(g >= 0 && g < N && g1 >= 0 && g1 < N && off + N <= M, a.status)) continue;
     double u[S];
@@ -843,17 +840,15 @@ __device__ __forceinline__ void stage_f64(const Step1DArgs &a, Smem64<P, FLUX, N
 }
 
 // The order decisions of a staged FP64 tile over all threads: rejected orders
-// of every (component, interface), as reject_pass_f32; and the first threads'
-// share of the recursion's constants.
+// of every (component, interface), as reject_pass_f32.
 template <int P, int FLUX, int NW, int R>
 __device__ __forceinline__ void reject_pass_f64(const Step1DArgs &a, Smem64<P, FLUX, NW, R> &sm, const Shape64 &sh,
-                                                long i0, long N, double lam) {
-  if constexpr (Smem64<P, FLUX, NW, R>::kSplit) split_lam(sm.lamk, lam, (int)threadIdx.x);
+                                                int nt, long i0, long N) {
   using TL = typename Smem64<P, FLUX, NW, R>::TL;
   constexpr int S = Phys<FLUX>::S;
   if constexpr (P >= 2) {
     const FiltConst FC = filt_const(a.epsf, a.rf, a.factf);
-    for (int q = threadIdx.x; q < S * sh.NI; q += sh.NT) {
+    for (int q = threadIdx.x; q < S * sh.NI; q += nt) {
       const int c = q / sh.NI, il = q - c * sh.NI, ic = il - 1 + TL::GH;
       unsigned r = 0;
       if (i0 + il <= N && acat_in_bounds(ic - P + 1 >= 0 && ic + P < TL::TW, a.status))
@@ -963,23 +958,42 @@ __device__ __forceinline__ void flux_finish_f64(Smem64<P, FLUX, NW, R> &sm, cons
 // One FP64 tile: cells [i0, i0 + T) of an instance of N cells whose state
 // starts at cell `off` of arrays with component stride M, in the shape sh;
 // orders (nullable) points at the instance's interface 0; the tile's maximal
-// wave speed goes to *smax_out. lam_sm: dt / dx, published by the caller no
-// later than the staging barrier.
-template <int P, int FLUX, int NW = NT / 32, int R = 1>
+// wave speed goes to *smax_out. SOLO: the last warp forms dt (into *lam_sm) and
+// the recursion's constants while the others stage the cells and decide the
+// orders, which do not need them (dt's chain of loads and divisions takes 1.5 us of a
+// 17 us step); else lam_sm points at the instance's dt / dx.
+template <int P, int FLUX, int NW, int R, bool SOLO>
 __device__ __forceinline__ void tile_f64(const Step1DArgs &a, Smem64<P, FLUX, NW, R> &sm, const Shape64 &sh,
                                          const double *__restrict__ uin, double *__restrict__ uout,
-                                         long off, long M, long N, long i0, const double *lam_sm,
+                                         long off, long M, long N, long i0,
+                                         typename std::conditional<SOLO, double, const double>::type *lam_sm,
                                          int8_t *orders, unsigned long long *smax_out) {
-  using TL = typename Smem64<P, FLUX, NW, R>::TL;
+  using SM = Smem64<P, FLUX, NW, R>;
+  using TL = typename SM::TL;
   constexpr int S = Phys<FLUX>::S;
-  stage_f64<P, FLUX, NW, R>(a, sm, sh, uin, off, M, N, i0);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = sh.NT >> 5;
+  const int grp = lane / TL::L, l = lane - grp * TL::L;
+  const int nt = SOLO ? sh.NT - 32 : sh.NT;  // threads that stage and decide
+  if (SOLO && warp == nw - 1) {
+    if constexpr (SOLO) {
+      if (lane == 0) *lam_sm = step_dt(a) / a.dx;
+      if constexpr (SM::kSplit) {
+        __syncwarp();
+        split_lam(sm.lamk, *lam_sm, lane);
+      }
+    }
+  } else {
+    if constexpr (!SOLO && SM::kSplit) split_lam(sm.lamk, *lam_sm, (int)threadIdx.x);
+    if constexpr (SOLO && SM::kSplit) split_tab(sm.tab, (int)threadIdx.x, nt);
+    stage_f64<P, FLUX, NW, R>(a, sm, sh, nt, uin, off, M, N, i0);
+    if constexpr (P >= 2) {
+      part_sync(nt);
+      reject_pass_f64<P, FLUX, NW, R>(a, sm, sh, nt, i0, N);
+    }
+  }
   __syncthreads();
   const double lam = *lam_sm;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = sh.NT >> 5;
-  const int grp = lane / TL::L, l = lane - grp * TL::L;
-  reject_pass_f64<P, FLUX, NW, R>(a, sm, sh, i0, N, lam);
-  if (P >= 2) __syncthreads();
 #pragma unroll 1
   for (int rnd = 0; rnd < sh.R; rnd++) {
     if (rnd > 0) __syncwarp();  // the exchange slots of the last round are read
@@ -1165,32 +1179,25 @@ __device__ __forceinline__ void update_cell_f32(const Step1DArgs &a, const float
   *smax = fmaxf(*smax, sf);
 }
 
-// One FP32 tile on the compensated state [hi(s x M); lo(s x M)].
-// Three CTA barriers per tile: after staging (which also publishes *lam_sm,
-// written by the caller before the call), after the order decisions, and
+// One FP32 tile on the compensated state [hi(s x M); lo(s x M)]. SOLO: the last
+// warp forms dt (into *lam_sm) while the others stage the cells and decide the
+// orders (P = 3, N = 16384: dt's 2400 cycles stood in front of a staging of 1000 and
+// decisions of 1500); else lam_sm points at the instance's lambda.
+// Three CTA barriers per tile: after staging, after the order decisions, and
 // between the flux and update phases. There is none at the end: a caller that loops over tiles
 // alternates between two workspaces (and two lam slots), so the next tile's
 // staging cannot overwrite what a slower warp still reads. The wave speed
 // maximum goes out per warp (atomic max of the warps that updated cells).
-template <int P, int FLUX, int NW = NT / 32, int LPN = 1, int R = 1>
+template <int P, int FLUX, int NW, int LPN, int R, bool SOLO>
 __device__ __forceinline__ void tile_f32(const Step1DArgs &a, Smem32<P, DPhys<FLUX>::S, NW, LPN, R> &sm,
                                          const float *__restrict__ uin, float *__restrict__ uout,
-                                         long off, long M, long N, long i0, const float *lam_sm,
+                                         long off, long M, long N, long i0,
+                                         typename std::conditional<SOLO, float, const float>::type *lam_sm,
                                          int8_t *orders, unsigned long long *smax_out) {
   using TL = Tiling<P, NW, LPN, R>;
   constexpr int NTB = NW * 32;
   using DP = DPhys<FLUX>;
   constexpr int S = DP::S;
-  for (int q = threadIdx.x; q < S * TL::TW; q += NTB) {
-    const int c = q / TL::TW, k = q - c * TL::TW;
-    const long g = bc_index(i0 - TL::GH + k, N, a.bc);
-    if (!acat_in_bounds(g >= 0 && g < N && off + N <= M, a.status)) continue;
-    sm.thi[c][k] = uin[c * M + off + g];
-    sm.tlo[c][k] = uin[(S + c) * M + off + g];
-  }
-  __syncthreads();
-  const float lam = *lam_sm;
-
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int grp = lane / TL::L, l = lane - grp * TL::L;
   const bool valid = grp < TL::GPW;
@@ -1198,10 +1205,29 @@ __device__ __forceinline__ void tile_f32(const Step1DArgs &a, Smem32<P, DPhys<FL
   // the warps' shuffle-free exchange slots of the one-lane-per-node recursion
   __shared__ float4 xs[(LPN == 1 && P >= 2 && S > 1) ? NW * 2 * XSET : 1];
   const FiltConst FC = filt_const(a.epsf, a.rf, a.factf);
-  // every order decision of the tile first, over all threads (a group's
-  // lanes beyond its S components would otherwise wait through them)
-  reject_pass_f32<P, S, TL::GH>(a, &sm.thi[0][0], &sm.tlo[0][0], TL::TW, TL::NI, i0, N, FC, &sm.rej[0][0], NTB);
-  if (P >= 2) __syncthreads();
+  constexpr int NTW = SOLO ? NTB - 32 : NTB;  // threads that stage and decide
+  if (SOLO && warp == NW - 1) {
+    if constexpr (SOLO) {
+      if (lane == 0) *lam_sm = (float)(step_dt(a) / a.dx);
+    }
+  } else {
+    for (int q = threadIdx.x; q < S * TL::TW; q += NTW) {
+      const int c = q / TL::TW, k = q - c * TL::TW;
+      const long g = bc_index(i0 - TL::GH + k, N, a.bc);
+      if (!acat_in_bounds(g >= 0 && g < N && off + N <= M, a.status)) continue;
+      sm.thi[c][k] = uin[c * M + off + g];
+      sm.tlo[c][k] = uin[(S + c) * M + off + g];
+    }
+    // every order decision of the tile first, over all threads (a group's
+    // lanes beyond its S components would otherwise wait through them)
+    if constexpr (P >= 2) {
+      if constexpr (SOLO) part_sync(NTW);
+      else __syncthreads();
+      reject_pass_f32<P, S, TL::GH>(a, &sm.thi[0][0], &sm.tlo[0][0], TL::TW, TL::NI, i0, N, FC, &sm.rej[0][0], NTW);
+    }
+  }
+  __syncthreads();
+  const float lam = *lam_sm;
   // R rounds: round rnd takes the interfaces (rnd NW + warp) GPW + grp, so
   // each round covers NW GPW consecutive interfaces; the tile's barriers
   // serve all R rounds
