@@ -39,6 +39,7 @@ struct alignas(16) SplitTab {
   float g1[3][8][8];   // [p-2][j][r]
   float gh[3][8];
   float k840[8];       // 840 / k at k - 1
+  double ik[8];        // 1 / k at k - 1
 };
 static_assert(sizeof(SplitTab) % 16 == 0, "copied in 16-byte pieces");
 
@@ -167,7 +168,7 @@ struct Step2DArgs {
 int acat_launch_step2d(int P, int flux, int prec, const Step2DArgs &a, void *stream);
 int acat_launch_smax2d(int flux, int prec, const Step2DArgs &a, void *stream);
 int acat_upload_tables_1d(const AcatTables *T, const SplitTab *G);
-int acat_upload_tables_adj(const AcatTables *T);
+int acat_upload_tables_adj(const AcatTables *T, const SplitTab *G);
 int acat_upload_tables_batch(const AcatTables *T, const SplitTab *G);
 int acat_adjoint_slots(int P);
 // Adjoint of one 1D step (a.u_in = u^n, dt from a.dt_in or a.dt_fixed): ubar0 from ubar1.

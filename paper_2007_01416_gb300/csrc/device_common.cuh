@@ -107,6 +107,12 @@ __device__ __forceinline__ Bits64 bits_of(double x) {
 __device__ __forceinline__ float small_float(unsigned n) {
   return __fsub_rn(__uint_as_float(0x4b000000u + n), 8388608.0f);
 }
+// a float as a double, by its bits (0 below 2^-126; finite values)
+__device__ __forceinline__ double d_bits(float x) {
+  const unsigned u = __float_as_uint(x), e = (u >> 23) & 0xffu;
+  const unsigned hi = (u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u);
+  return e ? __hiloint2double((int)hi, (int)(u << 29)) : 0.0;
+}
 __device__ __forceinline__ float f_bits(double x) { return __uint_as_float(bits_of(x).hi); }
 
 // fused multiply-add in the arithmetic type of its arguments

@@ -133,6 +133,8 @@ constexpr float SPLIT_TAU = 0x1p-5f;    // increments, of the local scales
 constexpr float SPLIT_QUAD = 0x1p-23f;  // quadratic terms that float carries
 constexpr float SPLIT_CUB = 0x1p-27f;   // form 1: cubic terms that float carries,
 constexpr float SPLIT_MIX = 0x1p-25f;   // and products of the first-order and the further terms
+constexpr float SPLIT_ADJ = 0x1p-8f;    // increments at which the adjoint takes its Jacobians from pairs
+constexpr float SPLIT_ADJ_H = 0x1p40f;  // and the largest h whose products with a cotangent they carry
 constexpr float SPLIT_TAIL = 0x1p-28f;  // F^(k-2) from which on float suffices
 
 // Whether the cubic terms W W max(a, W) and W L max(a, W) are below SPLIT_CUB of
@@ -165,7 +167,8 @@ struct SplitRec<ACAT_FLUX_EULER1D, TW> {
 };
 
 template <int FLUX, int TW>
-__device__ __forceinline__ void split_record(SplitRec<FLUX, TW> &r, int k, const double *u, double gm1) {
+__device__ __forceinline__ void split_record(SplitRec<FLUX, TW> &r, int k, const double *u, double gm1,
+                                             double *v_out = nullptr, double *h_out = nullptr) {
   if constexpr (FLUX == ACAT_FLUX_BURGERS) {
     const FF w = ff_bits(u[0]);
     const F3 f = f3_from(__dmul_rn(__dmul_rn(0.5, u[0]), u[0]));
@@ -177,6 +180,8 @@ __device__ __forceinline__ void split_record(SplitRec<FLUX, TW> &r, int k, const
     const double p = __dmul_rn(gm1, fma(__dmul_rn(-0.5, u[1]), v, u[2]));
     const double H = __dadd_rn(u[2], p), h = __dmul_rn(H, ri);
     const double f1 = fma(u[1], v, p), f2 = __dmul_rn(v, H);
+    if (v_out) *v_out = v;
+    if (h_out) *h_out = h;
     r.fd[0][k] = u[1];
     r.fd[1][k] = f1;
     r.fd[2][k] = f2;
@@ -226,11 +231,13 @@ __device__ __forceinline__ FF split_sum(unsigned mask, int base, int l, FF t) {
 // G x (840 LH) of one Euler interface by a group of 2p lanes (lane l <-> node
 // l - p + 1); ic: tile index of cell i. xa, xb: the group's exchange slots (two
 // sets XSET apart). Returns whether the float-float recursion holds (uniform in
-// the group); G is in lane `base`.
-template <int p, int TW>
+// the group); G is in lane `base`. ADJ: keeps the node's U^(k-1)/(k-1)! as
+// (a, W, L) in xst, pair e of order k at xst[((k - 2) 6 + e) 32], and takes the
+// tighter bound SPLIT_ADJ; no flux.
+template <int p, int TW, bool ADJ = false>
 __device__ __forceinline__ bool cat_split_euler(const SplitRec<ACAT_FLUX_EULER1D, TW> &rec, const Step1DArgs &a,
                                                 const SplitTab &tab, const float2 *lamk, int ic, int l, int base,
-                                                float4 *xa, float2 *xb, FF *G) {
+                                                float4 *xa, float2 *xb, FF *G, float *xst = nullptr) {
   constexpr int n = 2 * p, NL = n - 1;
   const unsigned mask = ((1u << n) - 1u) << base;
   const FF gam = ff_of(a.sgam), kap = ff_of(a.skap), omk = ff_of(a.somk), gm = ff_of(a.sgm1);
@@ -299,6 +306,13 @@ __device__ __forceinline__ bool cat_split_euler(const SplitRec<ACAT_FLUX_EULER1D
         Ba = fmaf(pk, fabsf(u0), Ba);
         Bw = fmaf(pk, fabsf(w), Bw);
         Bl = fmaf(pk, fabsf(L1), Bl);
+        if constexpr (ADJ) {
+          float *q = xst + (k - 2) * 6 * 32;
+          q[0] = u0;
+          q[64] = w;
+          q[128] = L1;
+          q[32] = q[96] = q[160] = 0.0f;
+        }
         float sq = 0.0f, st = 0.0f;
 #pragma unroll
         for (int q = 0; q < NL; q++) {
@@ -341,6 +355,15 @@ __device__ __forceinline__ bool cat_split_euler(const SplitRec<ACAT_FLUX_EULER1D
       Ba = fmaf(pk, fabsf(u[0].h), Ba);
       Bw = fmaf(pk, fabsf(w.h), Bw);
       Bl = fmaf(pk, fabsf(L1.h), Bl);
+      if constexpr (ADJ) {
+        float *q = xst + (k - 2) * 6 * 32;
+        q[0] = u[0].h;
+        q[32] = u[0].l;
+        q[64] = w.h;
+        q[96] = w.l;
+        q[128] = L1.h;
+        q[160] = L1.l;
+      }
       if (k == 2 && flt) {  // float remainders, by the first-order increments with a margin of 4
         const float bw = 2.0f * Bw, bl = 2.0f * Bl;
         flt = __all_sync(mask, bw * bw <= SPLIT_QUAD * rs * rs && bw * bl <= SPLIT_QUAD * rs * rh);
@@ -388,11 +411,13 @@ __device__ __forceinline__ bool cat_split_euler(const SplitRec<ACAT_FLUX_EULER1D
 #pragma unroll
       for (int c = 0; c < 3; c++) ff_acc(S[c], Y[c], ck);
     }
-    const bool small = Ba <= SPLIT_TAU * rho.h && Bw <= SPLIT_TAU * rs && Bl <= SPLIT_TAU * rh;
-    if (!__all_sync(mask, small)) return false;
+    constexpr float tau = ADJ ? SPLIT_ADJ : SPLIT_TAU;
+    const bool small = Ba <= tau * rho.h && Bw <= tau * rs && Bl <= tau * rh;
+    if (!__all_sync(mask, small && (!ADJ || h.h < SPLIT_ADJ_H))) return false;
     if (!flt || __all_sync(mask, Bw * Bw <= SPLIT_QUAD * rs * rs && Bw * Bl <= SPLIT_QUAD * rs * rh)) break;
     allow = false;  // the remainders grew past float: once more with pairs
   }
+  if constexpr (ADJ) return true;
   const float gw = tab.gh[p - 2][l];
 #pragma unroll
   for (int c = 0; c < 3; c++) G[c] = split_sum<n>(mask, base, l, ff_mulf(ff_norm(S[c]), gw));

@@ -374,7 +374,7 @@ int acat_upload_tables_current_device() {
   acat_build_split(&G);
   int e = acat_upload_tables_1d(&T, &G);
   if (e == 0) e = acat_upload_tables_2d(&T, &G);
-  if (e == 0) e = acat_upload_tables_adj(&T);
+  if (e == 0) e = acat_upload_tables_adj(&T, &G);
   if (e == 0) e = acat_upload_tables_batch(&T, &G);
   return e;
 }

@@ -191,5 +191,8 @@ void acat_build_split(SplitTab *T) {
       T->gh[p - 2][m] = times(s, kLH[p]);
     }
   }
-  for (int k = 1; k <= ACAT_MAXN; k++) T->k840[k - 1] = (float)(840 / k);
+  for (int k = 1; k <= ACAT_MAXN; k++) {
+    T->k840[k - 1] = (float)(840 / k);
+    T->ik[k - 1] = 1.0 / (double)k;
+  }
 }
