@@ -177,6 +177,11 @@ __device__ __forceinline__ void acat_pdl_release() { asm volatile("griddepcontro
 // A barrier among the first `n` threads of the CTA (n a multiple of 32).
 __device__ __forceinline__ void part_sync(int n) { asm volatile("bar.sync 1, %0;" ::"r"(n) : "memory"); }
 
+// The same on barrier `id` (1..15) among n threads in whole warps.
+__device__ __forceinline__ void part_sync_id(int id, int n) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
+}
+
 // Host side: launch a kernel of that form with programmatic stream
 // serialization (returns 0 or a cudaError_t value).
 template <typename... Params, typename... Args>

@@ -1915,7 +1915,7 @@ int launch2(const Step2DArgs &a, cudaStream_t st) {
 // 2D step for P = 3, 4 in FP32, and the rectangular stencils in FP32 at
 // P = 2..4: the structure of k_step2d_hi on the compensated state. Every
 // block task (square or rectangular) runs one thread per node on a
-// (2P)^2-thread slot with runtime extents 2 p1 x 2 p2, in the delta
+// (2P)^2-thread slot with extents 2 p1 x 2 p2, in the delta
 // formulation of the P <= 2 FP32 kernel: node j carries increments about the
 // anchor state u_a, f(u_j) - f(u_a) from a cancellation-free difference, and
 // every time level's flux increment f(u_j + del) - f(u_j) likewise; the
@@ -1925,10 +1925,9 @@ int launch2(const Step2DArgs &a, cudaStream_t st) {
 // The float weight tables in shared memory: the FP32 block tasks index them
 // with per-task orders and a per-thread node, which constant memory serves
 // one address at a time.
-struct TabSF {
-  float g1[ACAT_MAXP + 1][ACAT_MAXN][ACAT_MAXN];
-  float gk[ACAT_MAXP + 1][ACAT_MAXN][ACAT_MAXN];
-  float taylor[ACAT_MAXP + 1][ACAT_MAXN][ACAT_MAXN];
+struct alignas(16) TabSF {
+  float g1[ACAT_MAXP + 1][ACAT_MAXN][ACAT_MAXN];   // [p][j][r], 0 from r = 2p on
+  float2 lv[ACAT_MAXP + 1][ACAT_MAXN][ACAT_MAXN];  // [p][k-1][level r + p - 1]: r^(k-1) / (k-1)! and gamma^{k-1,0}_r
   float gh[ACAT_MAXP + 1][ACAT_MAXN];
   float invfact[ACAT_MAXN + 1];
 };
@@ -1964,7 +1963,10 @@ struct Smem2HF {
   static constexpr int RW = PAD ? 2 * P + 1 : 2 * P, TS = 2 * P * RW;
   static constexpr int YC = PAD ? RW : 1, YS = PAD ? 1 : 2 * P;
   static constexpr int XS = (NT / (4 * P * P) + 1) * TS;
-  float X[XS][S], Y[XS][S];
+  // order k reads set (k & 1) and writes the other from P = 3 on: one barrier per
+  // order. At P = 2 the barrier is half a warp's and one set is kept.
+  static constexpr bool DB = P >= 3;
+  alignas(16) float X[DB ? 2 : 1][XS][S], Y[DB ? 2 : 1][XS][S];
   unsigned rej[NAF<P> * NAF<P>];    // rejected orders: bit dir * (P - 1) + (p - 2)
   unsigned task[2 * NAF<P> * NAF<P>];  // anchor | wants | p1 << 12 | p2 << 15
   int ntask;
@@ -1972,33 +1974,117 @@ struct Smem2HF {
   TabSF tab;
 };
 
+template <int q>
+struct OrderTag {
+  static constexpr int value = q;
+};
+
+// The threads of a task's slot wait for one another: two whole warps at P = 4,
+// half a warp at P = 2, 36 threads across warps at P = 3 (the CTA).
+template <int P>
+__device__ __forceinline__ void slot_sync(int ti) {
+  if constexpr (P == 4) part_sync_id(ti + 1, 64);
+  else if constexpr (P == 2) __syncwarp(0xffffu << (threadIdx.x & 16u));
+  else __syncthreads();
+}
+
+// U of one node from a row of X and a column of Y (node r at X + r, Y + r ys) with
+// weights wx, wy over n nodes (0 beyond the task's extents).
+template <int n, int S>
+__device__ __forceinline__ void hi_slope(const float (*X)[S], const float (*Y)[S], int ys, const float *wx,
+                                         const float *wy, float *Ux, float *Uy) {
+  if constexpr (S == 4) {
+    float2 a0 = f2dup(0.0f), a1 = a0, b0 = a0, b1 = a0;
+#pragma unroll
+    for (int r = 0; r < n; r++) {
+      const float4 x = *reinterpret_cast<const float4 *>(X[r]), y = *reinterpret_cast<const float4 *>(Y[r * ys]);
+      const float2 u = f2dup(wx[r]), v = f2dup(wy[r]);
+      a0 = f2fma(u, make_float2(x.x, x.y), a0);
+      a1 = f2fma(u, make_float2(x.z, x.w), a1);
+      b0 = f2fma(v, make_float2(y.x, y.y), b0);
+      b1 = f2fma(v, make_float2(y.z, y.w), b1);
+    }
+    Ux[0] = a0.x, Ux[1] = a0.y, Ux[2] = a1.x, Ux[3] = a1.y;
+    Uy[0] = b0.x, Uy[1] = b0.y, Uy[2] = b1.x, Uy[3] = b1.y;
+  } else {
+#pragma unroll
+    for (int c = 0; c < S; c++) Ux[c] = Uy[c] = 0.0f;
+#pragma unroll
+    for (int r = 0; r < n; r++)
+#pragma unroll
+      for (int c = 0; c < S; c++) {
+        Ux[c] = fmaf(wx[r], X[r][c], Ux[c]);
+        Uy[c] = fmaf(wy[r], Y[r * ys][c], Uy[c]);
+      }
+  }
+}
+
+// The remainder sums of order k over the 2p levels, two levels in float2 lanes
+// (the level r = 0 keeps X = 0 and so its remainder).
+template <int p, typename RP>
+__device__ __forceinline__ void hi_levels(const TabSF &TB, int k, const typename RP::Base &bj, const float *X,
+                                          float2 (*xs)[RP::NX > 0 ? RP::NX : 1], float *A) {
+  constexpr int NX = RP::NX, NR = RP::NR, NRA = NR > 0 ? NR : 1;
+  if constexpr (NX > 0) {
+    const float4 *lv = reinterpret_cast<const float4 *>(TB.lv[p][k - 1]);
+    float2 A2[NRA];
+#pragma unroll
+    for (int c = 0; c < NR; c++) A2[c] = f2dup(0.0f);
+#pragma unroll
+    for (int q = 0; q < p; q++) {
+      const float4 w = lv[q];
+      float2 R[NRA];
+#pragma unroll
+      for (int c = 0; c < NX; c++) xs[q][c] = f2fma(make_float2(w.x, w.z), f2dup(X[c]), xs[q][c]);
+      RP::rem2(bj, xs[q], R);
+#pragma unroll
+      for (int c = 0; c < NR; c++) A2[c] = f2fma(make_float2(w.y, w.w), R[c], A2[c]);
+    }
+#pragma unroll
+    for (int c = 0; c < NR; c++) A[c] = A2[c].x + A2[c].y;
+  }
+}
+
+// What bounds it: latency of shared memory, the reciprocals and the barriers, at
+// the 16 warps per SM that its registers allow. Hence the orders unrolled for the
+// task's pm (with runtime extents every node and level was a branch, and each
+// load waited for by itself), slots that wait for their own threads only, one
+// barrier per order where there are two sets, and FMAs in float2 lanes. Issue
+// slots used at P = 4: 53 % before, 60 % now, of 15 % fewer instructions. ms a step,
+// rectangular: 512 x 512 P = 4 2.90 -> 2.19, P = 3 1.09 -> 0.99, 1024 x 1024 P = 2
+// 1.10 -> 0.83; square P = 3 1024 x 1024 4.02 -> 3.70, P = 4 512 x 512 3.05 -> 2.29.
 template <int P, int FLUX>
 __device__ __forceinline__ void block_tasks_f32(Smem2HF<P, FLUX> &sm, const Step2DArgs &a, float lx, float ly) {
   const TabSF &TB = sm.tab;
   using PH = Phys2<FLUX>;
   using RP = RPhys2<FLUX>;
+  using SM = Smem2HF<P, FLUX>;
   constexpr int S = PH::S, NX = RP::NX, NR = RP::NR, NXA = NX > 0 ? NX : 1, NRA = NR > 0 ? NR : 1;
   constexpr int NM = 2 * P, NN = NM * NM, per = NT / NN;
+  static_assert(P != 4 || NN == 64, "two warps per slot");
   const float gm1 = a.gm1f, axv = a.advf[0], ayv = a.advf[1];
   const int nt = sm.ntask;
   const int tid = threadIdx.x, ti = tid / NN, node = tid - ti * NN;
   const int ia = node % NM, ib = node / NM;
-  using SM = Smem2HF<P, FLUX>;
   const int xrow = ti * SM::TS + ib * SM::RW, ycol = ti * SM::TS + ia * SM::YC;  // row / column
   const int xw = xrow + ia, yw = ycol + ib * SM::YS;                             // own slots
-  for (int base = 0; base < nt; base += per) {
+  // P = 3: every thread takes every barrier
+  constexpr bool ALL = P == 3;
+#pragma unroll 1
+  for (int base = 0; ALL ? base < nt : base + ti < nt; base += per) {
     const bool slot_ok = ti < per && base + ti < nt;
     const unsigned tk = slot_ok ? sm.task[base + ti] : 0u;
     const int an = (int)(tk & 0x3ffu);
     const int p1 = slot_ok ? (int)((tk >> 12) & 7u) : 1, p2 = slot_ok ? (int)((tk >> 15) & 7u) : 1;
-    const int n1 = 2 * p1, n2 = 2 * p2, pm = p1 > p2 ? p1 : p2, n = 2 * pm, zt = pm - 1;
+    const int n1 = 2 * p1, n2 = 2 * p2, pm = p1 > p2 ? p1 : p2, n = 2 * pm;
     const bool act = slot_ok && ia < n1 && ib < n2;
     const int ax = an % NAF<P> - 1, ay = an / NAF<P> - 1;
-    float Ff[S], Fg[S], xs[NM][NXA];
+    float Ff[S], Fg[S];
+    float2 xs[P][NXA];
     typename RP::Base bj;
     if (act) {
-      const int tx = acat_tile_index(ax + P - p1 + 1 + ia, Smem2HF<P, FLUX>::TW, a.status);
-      const int ty = acat_tile_index(ay + P - p2 + 1 + ib, Smem2HF<P, FLUX>::TW, a.status);
+      const int tx = acat_tile_index(ax + P - p1 + 1 + ia, SM::TW, a.status);
+      const int ty = acat_tile_index(ay + P - p2 + 1 + ib, SM::TW, a.status);
       float ua[S], ual[S], uj[S], ujl[S], dh[S], dl[S];
 #pragma unroll
       for (int c = 0; c < S; c++) {
@@ -2019,13 +2105,13 @@ __device__ __forceinline__ void block_tasks_f32(Smem2HF<P, FLUX> &sm, const Step
     }
 #pragma unroll
     for (int c = 0; c < S; c++) {
-      sm.X[xw][c] = Ff[c];
-      sm.Y[yw][c] = Fg[c];
+      sm.X[0][xw][c] = Ff[c];
+      sm.Y[0][yw][c] = Fg[c];
     }
 #pragma unroll
-    for (int rr = 0; rr < NM; rr++)
+    for (int q = 0; q < P; q++)
 #pragma unroll
-      for (int c = 0; c < NX; c++) xs[rr][c] = RP::init(bj, c);
+      for (int c = 0; c < NX; c++) xs[q][c] = f2dup(RP::init(bj, c));
     // the derivative weights of the node's row and column, read once per task
     // at P <= 3 (at P = 4 they would cost the registers of the second CTA per
     // SM, and the loop reads them from the shared table)
@@ -2038,101 +2124,90 @@ __device__ __forceinline__ void block_tasks_f32(Smem2HF<P, FLUX> &sm, const Step
         wy[r] = act && r < n2 ? __fmul_rn(TB.g1[p2][ib][r], -ly) : 0.0f;
       }
     }
+    const int kn = ALL ? NM : n;
 #pragma unroll 1
-    for (int k = 2; k <= NM; k++) {
-      __syncthreads();
+    for (int k = 2; k <= kn; k++) {
+      slot_sync<P>(ti);
       const bool go = act && k <= n;
+      const int rd = SM::DB ? k & 1 : 0, wr = SM::DB ? rd ^ 1 : 0;
+      if (SM::DB && !act && k == 2) {  // nodes outside the task's extents: read with weight 0
+#pragma unroll
+        for (int c = 0; c < S; c++) sm.X[wr][xw][c] = sm.Y[wr][yw][c] = 0.0f;
+      }
       float U[S];
-      if (go) {
-        if constexpr (HW) {  // the scaled weights: one accumulation over row and column
+      const auto slope = [&](auto pc) {
+        constexpr int q = decltype(pc)::value;
+        float Ux[S], Uy[S];
+        if constexpr (HW) {
+          hi_slope<2 * q, S>(&sm.X[rd][xrow], &sm.Y[rd][ycol], SM::YS, wx, wy, Ux, Uy);
 #pragma unroll
-          for (int c = 0; c < S; c++) U[c] = 0.0f;
-#pragma unroll
-          for (int r = 0; r < NM; r++) {
-            if (r < n1) {
-#pragma unroll
-              for (int c = 0; c < S; c++) U[c] = fmaf(wx[r], sm.X[xrow + r][c], U[c]);
-            }
-            if (r < n2) {
-#pragma unroll
-              for (int c = 0; c < S; c++) U[c] = fmaf(wy[r], sm.Y[ycol + r * SM::YS][c], U[c]);
-            }
-          }
+          for (int c = 0; c < S; c++) U[c] = Ux[c] + Uy[c];
         } else {
-          float Ux[S], Uy[S];
+          float gx[NM], gy[NM];
 #pragma unroll
-          for (int c = 0; c < S; c++) Ux[c] = Uy[c] = 0.0f;
-#pragma unroll
-          for (int r = 0; r < NM; r++) {
-            if (r < n1) {
-              const float w = TB.g1[p1][ia][r];
-#pragma unroll
-              for (int c = 0; c < S; c++) Ux[c] = fmaf(w, sm.X[xrow + r][c], Ux[c]);
-            }
-            if (r < n2) {
-              const float w = TB.g1[p2][ib][r];
-#pragma unroll
-              for (int c = 0; c < S; c++) Uy[c] = fmaf(w, sm.Y[ycol + r * SM::YS][c], Uy[c]);
-            }
+          for (int r = 0; r < 2 * q; r += 4) {
+            *reinterpret_cast<float4 *>(&gx[r]) = *reinterpret_cast<const float4 *>(&TB.g1[p1][ia][r]);
+            *reinterpret_cast<float4 *>(&gy[r]) = *reinterpret_cast<const float4 *>(&TB.g1[p2][ib][r]);
           }
+          hi_slope<2 * q, S>(&sm.X[rd][xrow], &sm.Y[rd][ycol], SM::YS, gx, gy, Ux, Uy);
 #pragma unroll
           for (int c = 0; c < S; c++) U[c] = -(lx * Ux[c]) - ly * Uy[c];
         }
-      }
-      __syncthreads();
-      if (go) {
-        float X[NXA], A[NRA], af[S], ag[S];
+      };
+      float X[NXA], A[NRA], af[S], ag[S];
+      const auto levels = [&](auto pc) {
+        constexpr int q = decltype(pc)::value;
         RP::lin(bj, U, X, af, ag);
-#pragma unroll
-        for (int c = 0; c < NR; c++) A[c] = 0.0f;
-#pragma unroll
-        for (int rr = 0; rr < (NX > 0 ? NM : 0); rr++) {
-          if (rr >= n || rr == zt) continue;
-          const float cr = TB.taylor[pm][rr][k - 1], wk = TB.gk[pm][k - 1][rr];
-          float R[NRA];
-#pragma unroll
-          for (int c = 0; c < NX; c++) xs[rr][c] = fmaf(cr, X[c], xs[rr][c]);
-          RP::rem(bj, xs[rr], R);
-#pragma unroll
-          for (int c = 0; c < NR; c++) A[c] = fmaf(wk, R[c], A[c]);
-        }
+        hi_levels<q, RP>(TB, k, bj, X, xs, A);
         RP::add(bj, U, A, af, ag);
+      };
+      if (go) {
+        if (P == 4 && pm == 4) slope(OrderTag<(P >= 4 ? 4 : P)>{});
+        else if (P >= 3 && pm == 3) slope(OrderTag<(P >= 3 ? 3 : P)>{});
+        else slope(OrderTag<2>{});
+      }
+      if constexpr (!SM::DB) slot_sync<P>(ti);
+      if (go) {
+        if (P == 4 && pm == 4) levels(OrderTag<(P >= 4 ? 4 : P)>{});
+        else if (P >= 3 && pm == 3) levels(OrderTag<(P >= 3 ? 3 : P)>{});
+        else levels(OrderTag<2>{});
 #pragma unroll
         for (int c = 0; c < S; c++) {
-          sm.X[xw][c] = af[c];
-          sm.Y[yw][c] = ag[c];
+          if (k < n) {
+            sm.X[wr][xw][c] = af[c];
+            sm.Y[wr][yw][c] = ag[c];
+          }
           if (k <= n1) Ff[c] = fmaf(TB.invfact[k], af[c], Ff[c]);
           if (k <= n2) Fg[c] = fmaf(TB.invfact[k], ag[c], Fg[c]);
         }
       }
     }
-    __syncthreads();
+    // the weighted fluxes, into the set that the last order did not read
+    constexpr int fs = SM::DB ? 1 : 0;
     if (act) {
 #pragma unroll
       for (int c = 0; c < S; c++) {
-        if (ib == p2 - 1) sm.X[xw][c] = TB.gh[p1][ia] * Ff[c];
-        if (ia == p1 - 1) sm.Y[yw][c] = TB.gh[p2][ib] * Fg[c];
+        if (ib == p2 - 1) sm.X[fs][xw][c] = TB.gh[p1][ia] * Ff[c];
+        if (ia == p1 - 1) sm.Y[fs][yw][c] = TB.gh[p2][ib] * Fg[c];
       }
     }
-    __syncthreads();
-    if (slot_ok && node == 0) {
-      if (tk & WF32)
-#pragma unroll
-        for (int c = 0; c < S; c++) {
-          float t = 0.0f;
-          for (int r = 0; r < n1; r++) t += sm.X[ti * SM::TS + (p2 - 1) * SM::RW + r][c];
+    slot_sync<P>(ti);
+    if (slot_ok && node < 2 * S) {
+      const int c = node % S;
+      float t = 0.0f;
+      if (node < S) {
+        if (tk & WF32) {
+          for (int r = 0; r < n1; r++) t += sm.X[fs][ti * SM::TS + (p2 - 1) * SM::RW + r][c];
           sm.Fx[ay][ax + 1][c] = t;
         }
-      if (tk & WG32)
-#pragma unroll
-        for (int c = 0; c < S; c++) {
-          float t = 0.0f;
-          for (int r = 0; r < n2; r++) t += sm.Y[ti * SM::TS + (p1 - 1) * SM::YC + r * SM::YS][c];
-          sm.Gy[ay + 1][ax][c] = t;
-        }
+      } else if (tk & WG32) {
+        for (int r = 0; r < n2; r++) t += sm.Y[fs][ti * SM::TS + (p1 - 1) * SM::YC + r * SM::YS][c];
+        sm.Gy[ay + 1][ax][c] = t;
+      }
     }
-    __syncthreads();
+    if constexpr (!SM::DB) slot_sync<P>(ti);
   }
+  __syncthreads();
 }
 
 template <int P, int FLUX>
@@ -2141,7 +2216,8 @@ __global__ void __launch_bounds__(NT, 2) k_step2d_hi_f32(const Step2DArgs a) {
   constexpr int S = PH::S;
   constexpr int TW = Smem2HF<P, FLUX>::TW;
   constexpr int CELLS = TW * TW;
-  __shared__ Smem2HF<P, FLUX> sm;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  Smem2HF<P, FLUX> &sm = *reinterpret_cast<Smem2HF<P, FLUX> *>(smem_raw);
   __shared__ double s_red[2][NT / 32];
   const int tid = threadIdx.x;
   const long NXl = a.NX, NYl = a.NY;
@@ -2157,8 +2233,8 @@ __global__ void __launch_bounds__(NT, 2) k_step2d_hi_f32(const Step2DArgs a) {
     constexpr int NW3 = (ACAT_MAXP + 1) * ACAT_MAXN * ACAT_MAXN;
     for (int q = tid; q < NW3; q += NT) {
       (&sm.tab.g1[0][0][0])[q] = (&c_tab.g1f[0][0][0])[q];
-      (&sm.tab.gk[0][0][0])[q] = (&c_tab.gkf[0][0][0])[q];
-      (&sm.tab.taylor[0][0][0])[q] = (&c_tab.taylorf[0][0][0])[q];
+      const int tp = q / (ACAT_MAXN * ACAT_MAXN), tk = q / ACAT_MAXN % ACAT_MAXN, tr = q % ACAT_MAXN;
+      sm.tab.lv[tp][tk][tr] = make_float2(c_tab.taylorf[tp][tr][tk], c_tab.gkf[tp][tk][tr]);
     }
     for (int q = tid; q < (ACAT_MAXP + 1) * ACAT_MAXN; q += NT) (&sm.tab.gh[0][0])[q] = (&c_tab.ghf[0][0])[q];
     for (int q = tid; q <= ACAT_MAXN; q += NT) sm.tab.invfact[q] = c_tab.invfactf[q];
@@ -2307,8 +2383,7 @@ __global__ void __launch_bounds__(NT, 2) k_step2d_hi_f32(const Step2DArgs a) {
 template <int P, int FLUX>
 int launch2_hi_f32(const Step2DArgs &a, cudaStream_t st) {
   dim3 grid((unsigned)((a.NX + TXF<P> - 1) / TXF<P>), (unsigned)((a.NY + TXF<P> - 1) / TXF<P>));
-  k_step2d_hi_f32<P, FLUX><<<grid, NT, 0, st>>>(a);
-  return (int)cudaGetLastError();
+  return launch_big(k_step2d_hi_f32<P, FLUX>, grid, sizeof(Smem2HF<P, FLUX>), a, st);
 }
 
 template <int P, int FLUX>
