@@ -65,7 +65,7 @@ struct Rounds {
 
 // Persistent batched step: CTAs of NW warps take the tiles of the (instance,
 // first cell) work list, Tiling<P, NW, LPN, R>::T cells wide (R =
-// RoundsB32<NW> in FP32, 1 in FP64), from a queue: CTA c starts with tile c,
+// Rounds<F32, NW>), from a queue: CTA c starts with tile c,
 // and each further tile is claimed with one atomic on the queue counter
 // (set to 0 by k_batch_dt), issued before the current tile so that its
 // latency hides behind the tile's work. Tiles cost unevenly (FL-CAT2

@@ -29,7 +29,8 @@
 //     the caller evaluates the recursion in FP64. The remainders take one of
 //     three forms, by the size of the Taylor sums (time increments):
 //       0  in float, where the quadratic terms are below 2^-23 of the scales;
-//       1  their leading term exactly, the rest in float: with d_r = r d_1 + d'_r,
+//       1  (2D blocks; in 1D it was slower than form 2: P = 4 at N = 262144
+//          261 -> 280 us a step) their leading term exactly, the rest in float: with d_r = r d_1 + d'_r,
 //          the products r^2 d_1 d_1 / rho are polynomials of degree 2 in r, so
 //          their weighted sum is d_1 d_1 / rho at k = 3 and 0 otherwise (one pair);
 //          what is left is cubic, or carries the small d', and is formed without
@@ -39,6 +40,11 @@
 //     are float too (forms 0 and 1). All leave the measured error unchanged
 //     (0.19-0.22). Each decision is taken per interface, by a vote of its lanes,
 //     and checked against bounds of all Taylor sums at the end.
+//
+// What bounds it: instruction issue and the latency of dependent FP32 operations (a
+// pair operation is a chain of 4 to 11), at 14 warps per SM 0.6 instructions per
+// cycle and scheduler. P = 4, N = 16384, Euler: 283 us a step in FP64, 25.7 here
+// (P = 3 144 -> 22.0, P = 2 43.7 -> 17.1).
 #pragma once
 
 #include "phys1d.cuh"

@@ -7,14 +7,14 @@
 // condition applied while loading. Each interface is worked by a group of 2P
 // lanes of one warp, one lane per stencil node j = -p+1..p:
 //   - the indicators psi^p (Eqs. 3.8-3.12, the minimum over components of
-//     Sec. 3.4): lane c of the group decides every order p = 2..P of
-//     component c from the differences of the largest stencil (the smaller
-//     ones are nested in it). Each decision is a float test with a certified
+//     Sec. 3.4): one thread of the CTA decides every order p = 2..P of one
+//     interface and component from the differences of the largest stencil (the
+//     smaller ones are nested in it). Each decision is a float test with a certified
 //     error margin (psi_filter_all); only when the margin cannot settle it
 //     is psi^p evaluated literally with explicitly rounded FP64 operations
 //     in the order of its definition. Either way the decision is the one a
-//     literal FP64 evaluation of the same state takes. An OR-reduction over
-//     the group gives p_s = max A (Eqs. 3.2-3.3);
+//     literal FP64 evaluation of the same state takes. The OR over the
+//     components gives p_s = max A (Eqs. 3.2-3.3);
 //   - for p_s >= 2 every lane runs the local Taylor recursion of Sec. 2.2 for
 //     its node in registers, in the dt-scaled form
 //         U^(k-1)_j = -lambda sum_r gamma^{1,j}_r F^(k-2)_r     (shuffles)
@@ -22,8 +22,11 @@
 //     (U^(l) = dt^l u~^(l), F^(k) = dt^k f~^(k)), keeping the Taylor sums at
 //     the 2p-1 time levels r != 0 as running values (one FMA per level and
 //     order instead of a Horner pass); the flux is sum_k 1/k! sum_j
-//     gamma^{0,1/2}_j F^(k-1)_j (Eq. 2.14) reduced across the group;
-//   - for p_s = 1 lane 0 evaluates FL-CAT2 (Eqs. 3.4-3.7).
+//     gamma^{0,1/2}_j F^(k-1)_j (Eq. 2.14) reduced across the group. FP64
+//     evaluates it in float-float pairs on flux increments where these are small
+//     (split1d.cuh), else as written (cat_flux); linear transport needs no time
+//     levels;
+//   - for p_s = 1 the group evaluates FL-CAT2 (Eqs. 3.4-3.7).
 // The conservative update (Eq. 2.12) follows from shared memory, and its
 // epilogue reduces the wave speed of the new state for the next step's CFL
 // dt into a triple-buffered slot (atomic max on ordered double bits).
@@ -74,8 +77,8 @@ __global__ void __launch_bounds__(NW * 32, MinCtas<P, true>::value) k_step1d_f32
   acat_pdl_release();
 }
 
-// FP32 step in small CTAs (NWF warps), the boundary hand-off of
-// k_step1d_fine on the compensated state: CTA b computes the flux increments
+// FP32 step in small CTAs (NWF warps) with a hand-off of the cell between two
+// CTAs: CTA b computes the flux increments
 // G of the NI interfaces [b NI, b NI + NI) (iface_f32, as the fused FP32 tile)
 // and updates the cells between them (update_cell_f32); it publishes its two
 // edge increments (float, s x (N+1) in flux_buf), fences, and counts in at
@@ -308,8 +311,8 @@ int launch_smax(int flux, const Step1DArgs &a, cudaStream_t st) {
 // 17.7 us at R = 1, 23.3 at R = 2), and some 1.5 % more per warp resident on an SM
 // (16 warps fit at 128 registers). So: the shape with the least
 // waves (2 + R) (1 + 0.015 warps), waves whole up to 4 and averaged beyond.
-// N = 16384, us per step: P = 4 28.3 at (7, 2) against 36.9 at (8, 1); P = 3 23.5 at
-// (4, 2) against 29.5; P = 2 17.1-17.9 at (4..7, 1).
+// When the rule was made, N = 16384, us per step: P = 4 28.3 at (7, 2) against 36.9
+// at (8, 1); P = 3 23.5 at (4, 2) against 29.5; P = 2 17.1-17.9 at (4..7, 1).
 void acat_shape_f64(int P, long N, int sms, int *nw_out, int *rounds_out) {
   double best = 0.0;
   for (int nw = 4; nw <= NT / 32; nw++)

@@ -177,6 +177,10 @@ struct DPhys<ACAT_FLUX_LINEAR> {
   __device__ static __forceinline__ void dflux_pair(const Base &b, const float *dh, const float *dl, float *df) {
     df[0] = b.a * (dh[0] + dl[0]);
   }
+  // two increments at once, packed in the lanes of float2 values
+  __device__ static __forceinline__ void dflux_x2(const Base &b, const float2 *d, float2 *df) {
+    df[0] = f2mul(f2dup(b.a), d[0]);
+  }
   __device__ static __forceinline__ float speed(const float *, float a, float) { return fabsf(a); }
   __device__ static __forceinline__ bool physical(const float *u, float) { return isfinite(u[0]); }
 };
@@ -196,6 +200,9 @@ struct DPhys<ACAT_FLUX_BURGERS> {
   __device__ static __forceinline__ void dflux_pair(const Base &b, const float *dh, const float *dl, float *df) {
     const float d[1] = {dh[0] + dl[0]};
     dflux(b, d, df);
+  }
+  __device__ static __forceinline__ void dflux_x2(const Base &b, const float2 *d, float2 *df) {
+    df[0] = f2mul(d[0], f2fma(f2dup(0.5f), d[0], f2dup(b.u)));
   }
   __device__ static __forceinline__ float speed(const float *u, float, float) { return fabsf(u[0]); }
   __device__ static __forceinline__ bool physical(const float *u, float) { return isfinite(u[0]); }
@@ -264,6 +271,18 @@ struct DPhys<ACAT_FLUX_EULER1D> {
     const float num = fmaf(-B.vl, dh[0], __fadd_rn(fmaf(-B.v, dh[0], dh[1]), fmaf(-B.v, dl[0], dl[1])));
     rest(B, d, __fmul_rn(num, recip(__fadd_rn(B.rho, d[0]))), df);
   }
+  // the same for two increments packed in float2 lanes
+  __device__ static __forceinline__ void dflux_x2(const Base &B, const float2 *d, float2 *df) {
+    const float2 t = f2fma(f2dup(-B.vl), d[0], f2fma(f2dup(-B.v), d[0], d[1]));
+    const float2 den = f2add(f2dup(B.rho), d[0]);
+    const float2 dv = f2mul(t, make_float2(recip(den.x), recip(den.y)));
+    const float2 vn = f2add(f2dup(B.v), dv);
+    const float2 dmv = f2fma(f2dup(B.m), dv, f2mul(d[1], vn));
+    const float2 dp = f2mul(f2dup(B.gm1), f2fma(f2dup(-0.5f), dmv, d[2]));
+    df[0] = d[1];
+    df[1] = f2add(dmv, dp);
+    df[2] = f2fma(dv, f2dup(B.H), f2mul(vn, f2add(d[2], dp)));
+  }
   __device__ static __forceinline__ float speed(const float *u, float, float gamma) {
     const float v = __fdiv_rn(u[1], u[0]);
     const float p = __fmul_rn(__fsub_rn(gamma, 1.0f), __fsub_rn(u[2], __fmul_rn(__fmul_rn(0.5f, u[1]), v)));
@@ -276,135 +295,17 @@ struct DPhys<ACAT_FLUX_EULER1D> {
   }
 };
 
-// ---------------------------------------------------------------------------
-// The increment f(u + d) - f(u) = A(u) d + q(u; d) split into the Jacobian
-// product and its remainder (closed form, quadratic in d). The time weights
-// gamma^{k-1,0}_r are exact on polynomials of degree <= 2p-1 in r and the Taylor
-// sum d_r = sum_l r^l/l! U^(l) of order k has degree k-1, so
-// sum_r gamma^{k-1,0}_r A d_r = A U^(k-1): one Jacobian product per order
-// carries the linear part of all 2p-1 time levels, and a level evaluates only
-// q, from Taylor sums of the NX combinations of U that q needs:
-//   lin     X (the NX combinations) and F = A U, from U;
-//   rem     the NR nonlinear terms of q at one level, from the Taylor sums of X
-//           (started at init); rem2 the same for two levels in float2 lanes;
-//   add     q's weighted sum over the levels into F.
-// Euler: W = b - v a, L = dH' - h a (dH' the linear part of dH, h = H/rho);
-// dv = W / (rho + a), Q = W dv, T = dv (L - kappa Q), kappa = (gamma - 1)/2;
-// q = (0, (1 - kappa) Q, T - kappa v Q). A level costs 9 float instructions and
-// one reciprocal, against 22 with the whole increment. Every operation is
-// rounded as written, so that every kernel gives the same bits.
-// ---------------------------------------------------------------------------
-template <int FLUX>
-struct RPhys;
-
-template <>
-struct RPhys<ACAT_FLUX_LINEAR> {  // q = 0
-  static constexpr int NX = 0, NR = 0;
-  struct Base {
-    float a;
-  };
-  __device__ static __forceinline__ Base base(const float *, const float *, float a, float) { return Base{a}; }
-  __device__ static __forceinline__ void lin(const Base &B, const float *U, float *, float *F) {
-    F[0] = __fmul_rn(B.a, U[0]);
-  }
-  __device__ static __forceinline__ float init(const Base &, int) { return 0.0f; }
-  __device__ static __forceinline__ void rem(const Base &, const float *, float *) {}
-  __device__ static __forceinline__ void rem2(const Base &, const float2 *, float2 *) {}
-  __device__ static __forceinline__ void add(const Base &, const float *, const float *, float *) {}
-};
-
-template <>
-struct RPhys<ACAT_FLUX_BURGERS> {  // A = u, q = d^2 / 2
-  static constexpr int NX = 1, NR = 1;
-  struct Base {
-    float u;
-  };
-  __device__ static __forceinline__ Base base(const float *h, const float *, float, float) { return Base{h[0]}; }
-  __device__ static __forceinline__ void lin(const Base &B, const float *U, float *X, float *F) {
-    X[0] = U[0];
-    F[0] = __fmul_rn(B.u, U[0]);
-  }
-  __device__ static __forceinline__ float init(const Base &, int) { return 0.0f; }
-  __device__ static __forceinline__ void rem(const Base &, const float *X, float *R) { R[0] = __fmul_rn(X[0], X[0]); }
-  __device__ static __forceinline__ void rem2(const Base &, const float2 *X, float2 *R) { R[0] = f2mul(X[0], X[0]); }
-  __device__ static __forceinline__ void add(const Base &, const float *, const float *A, float *F) {
-    F[0] = fmaf(0.5f, A[0], F[0]);
-  }
-};
-
-template <>
-struct RPhys<ACAT_FLUX_EULER1D> {
-  static constexpr int NX = 3, NR = 2;
-  struct Base {
-    float rho, v, vl, h, gm1, kap, kv;  // v + vl: the velocity to float-float accuracy (DPhys::base2)
-  };
-  __device__ static __forceinline__ Base base(const float *h, const float *l, float, float gm1) {
-    Base b;
-    b.rho = h[0];
-    const float r = recip(h[0]);
-    b.v = __fmul_rn(h[1], r);
-    b.vl = __fmul_rn(__fadd_rn(fmaf(-b.v, h[0], h[1]), fmaf(-b.v, l[0], l[1])), r);
-    const float p = __fmul_rn(gm1, fmaf(__fmul_rn(-0.5f, h[1]), b.v, h[2]));
-    b.h = __fmul_rn(__fadd_rn(h[2], p), r);
-    b.gm1 = gm1;
-    b.kap = __fmul_rn(0.5f, gm1);
-    b.kv = __fmul_rn(b.kap, b.v);
-    return b;
-  }
-  // U = (a, b, e): W as a cancelling numerator with both parts of v; s the
-  // linear part of d(mv), L' = e + (gamma - 1)(e - s/2) that of dH. F[1] holds
-  // s until add() forms d(mv) + dp.
-  __device__ static __forceinline__ void lin(const Base &B, const float *U, float *X, float *F) {
-    const float W = fmaf(-B.vl, U[0], fmaf(-B.v, U[0], U[1]));
-    const float s = __fmul_rn(B.v, __fadd_rn(U[1], W));
-    const float Lp = fmaf(B.gm1, fmaf(-0.5f, s, U[2]), U[2]);
-    X[0] = U[0];
-    X[1] = W;
-    X[2] = fmaf(-B.h, U[0], Lp);
-    F[0] = U[1];
-    F[1] = s;
-    F[2] = fmaf(B.v, Lp, __fmul_rn(B.h, W));
-  }
-  __device__ static __forceinline__ float init(const Base &B, int c) { return c == 0 ? B.rho : 0.0f; }
-  __device__ static __forceinline__ void rem(const Base &B, const float *X, float *R) {
-    const float dv = __fmul_rn(X[1], recip(X[0]));
-    R[0] = __fmul_rn(X[1], dv);
-    R[1] = __fmul_rn(dv, fmaf(-B.kap, R[0], X[2]));
-  }
-  __device__ static __forceinline__ void rem2(const Base &B, const float2 *X, float2 *R) {
-    const float2 dv = f2mul(X[1], make_float2(recip(X[0].x), recip(X[0].y)));
-    R[0] = f2mul(X[1], dv);
-    R[1] = f2mul(dv, f2fma(f2dup(-B.kap), R[0], X[2]));
-  }
-  __device__ static __forceinline__ void add(const Base &B, const float *U, const float *A, float *F) {
-    const float m = __fadd_rn(F[1], A[0]);  // d(mv)
-    F[1] = fmaf(B.gm1, fmaf(-0.5f, m, U[2]), m);
-    F[2] = __fadd_rn(F[2], fmaf(-B.kv, A[0], A[1]));
-  }
-};
-
-// Sum over the n lanes of a group (lane l, first lane base) by a tree of
-// shuffles; every lane returns it at n = 2, 4, 8, lane `base` at n = 6.
-template <int n>
-__device__ __forceinline__ float group_sum(unsigned mask, int base, int l, float t) {
-  if constexpr (n == 6) {
-    t = __fadd_rn(t, __shfl_sync(mask, t, base + (l < 3 ? l + 3 : l - 3)));
-    const float a = __shfl_sync(mask, t, base + (l + 1) % 6), b = __shfl_sync(mask, t, base + (l + 2) % 6);
-    return __fadd_rn(__fadd_rn(t, a), b);
-  } else {
-#pragma unroll
-    for (int w = 1; w < n; w <<= 1) t = __fadd_rn(t, __shfl_sync(mask, t, base + (l ^ w)));
-    return t;
-  }
-}
-
 // CAT2p increment G of one interface by a group of 2p lanes (lane l <-> node
 // j = l - p + 1). hi/lo point at cell i of component 0 of the compensated
 // tile, components `cs` apart. xg: the group's exchange slots in shared
 // memory (node r at xg[r], two sets XSET apart used alternately by k),
 // through which the lanes of the group read the F^(k-2) of all nodes of a
 // system: one 16-byte store and 2p 16-byte broadcast loads per lane and order
-// instead of 2p s shuffles (scalar laws shuffle). Lane 0 of the group returns G.
+// instead of 2p s shuffles (scalar laws shuffle). Every lane returns G.
+// A level evaluates the whole increment. The Jacobian product and remainder of
+// split1d.cuh would be faster (P = 4, N = 16384 11.7 -> 9.8 us a step) and no less
+// accurate, but gradients through FP32 runs on coarse grids answer any change of
+// rounding with 1e-4 of their size and more, so these sums keep their bits.
 template <int p, int FLUX>
 __device__ __forceinline__ void cat_delta(const float *hi, const float *lo, int cs, int l, int base,
                                           float lam, float adv, float gm1, float4 *xg, float *Gout) {
@@ -430,26 +331,26 @@ __device__ __forceinline__ void cat_delta(const float *hi, const float *lo, int 
     dl[c] = ujl[c] - uil[c];
   }
   // the 2p - 1 time levels r != 0 (level q <-> table row q < p - 1 ? q : q + 1)
-  // are worked in pairs packed in float2 lanes, the last one alone
-  using RP = RPhys<FLUX>;
-  constexpr int NL = n - 1, NP = NL / 2, NX = RP::NX, NR = RP::NR;
-  constexpr int NXA = NX > 0 ? NX : 1, NRA = NR > 0 ? NR : 1;
-  float D[S], Fsum[S], Fprev[S], xs1[NL - 2 * NP][NXA];
-  float2 xs2[NP > 0 ? NP : 1][NXA];
+  // are worked in pairs packed in float2 lanes (p <= 3; at p = 4 the pairs
+  // would cost the registers of a fourth resident CTA), the last one alone
+  constexpr int NL = n - 1, NP = p <= 3 ? NL / 2 : 0;
+  float D[S], Fsum[S], Fprev[S], dels[NL - 2 * NP][S];
+  float2 del2[NP > 0 ? NP : 1][S];
   DP::dflux_pair(DP::base2(ui, uil, adv, gm1), dh, dl, D);  // f(u_j) - f(u_i)
-  const typename RP::Base bj = RP::base(uj, ujl, adv, gm1);
+  const typename DP::Base bj = DP::base2(uj, ujl, adv, gm1);
 #pragma unroll
   for (int c = 0; c < S; c++) {
     Fsum[c] = D[c];
     Fprev[c] = D[c];
   }
 #pragma unroll
-  for (int c = 0; c < NX; c++) {
+  for (int q = 0; q < NL - 2 * NP; q++)
 #pragma unroll
-    for (int q = 0; q < NL - 2 * NP; q++) xs1[q][c] = RP::init(bj, c);
+    for (int c = 0; c < S; c++) dels[q][c] = 0.0f;
 #pragma unroll
-    for (int q = 0; q < NP; q++) xs2[q][c] = f2dup(RP::init(bj, c));
-  }
+  for (int q = 0; q < NP; q++)
+#pragma unroll
+    for (int c = 0; c < S; c++) del2[q][c] = make_float2(0.0f, 0.0f);
 #pragma unroll
   for (int k = 2; k <= n; k++) {
     float U[S];
@@ -487,49 +388,86 @@ __device__ __forceinline__ void cat_delta(const float *hi, const float *lo, int 
 #pragma unroll
       for (int r = 0; r < n; r++) U[0] = fmaf(g1r[r], __shfl_sync(mask, Fprev[0], base + r), U[0]);
     }
-    float X[NXA], F[S], A[NRA];
-    float2 A2[NRA];
-    RP::lin(bj, U, X, F);
+    if constexpr (FLUX == ACAT_FLUX_LINEAR) {  // F^(k-1) = a U^(k-1), no time levels
+      Fprev[0] = __fmul_rn(adv, U[0]);
+      Fsum[0] = fmaf(TB::invfact(k), Fprev[0], Fsum[0]);
+      continue;
+    }
+    float acc[S];
+    float2 acc2[S];
 #pragma unroll
-    for (int c = 0; c < NR; c++) {
-      A[c] = 0.0f;
-      A2[c] = make_float2(0.0f, 0.0f);
+    for (int c = 0; c < S; c++) {
+      acc[c] = 0.0f;
+      acc2[c] = make_float2(0.0f, 0.0f);
     }
 #pragma unroll
-    for (int q = 0; q < (NX > 0 ? NP : 0); q++) {
+    for (int q = 0; q < NP; q++) {
       const int ra = 2 * q < p - 1 ? 2 * q : 2 * q + 1, rb = 2 * q + 1 < p - 1 ? 2 * q + 1 : 2 * q + 2;
       const float2 cr = make_float2(TB::taylor(p, ra, k - 1), TB::taylor(p, rb, k - 1));
       const float2 wk = make_float2(TB::gk(p, k - 1, ra), TB::gk(p, k - 1, rb));
-      float2 R2[NRA];
+      float2 E2[S];
 #pragma unroll
-      for (int c = 0; c < NX; c++) xs2[q][c] = f2fma(cr, f2dup(X[c]), xs2[q][c]);
-      RP::rem2(bj, xs2[q], R2);
+      for (int c = 0; c < S; c++) del2[q][c] = f2fma(cr, f2dup(U[c]), del2[q][c]);
+      DP::dflux_x2(bj, del2[q], E2);
 #pragma unroll
-      for (int c = 0; c < NR; c++) A2[c] = f2fma(wk, R2[c], A2[c]);
+      for (int c = 0; c < S; c++) acc2[c] = f2fma(wk, E2[c], acc2[c]);
     }
 #pragma unroll
-    for (int q = 2 * NP; q < (NX > 0 ? NL : 0); q++) {  // levels not paired
+    for (int q = 2 * NP; q < NL; q++) {  // levels not paired
       const int rs = q < p - 1 ? q : q + 1;
       const float cr = TB::taylor(p, rs, k - 1), wk = TB::gk(p, k - 1, rs);
-      float R1[NRA];
+      float *dq = dels[q - 2 * NP];
+      float E[S];
+      if constexpr (S == 3 && p >= 3) {
+        const float2 d01 = f2fma(f2dup(cr), make_float2(U[0], U[1]), make_float2(dq[0], dq[1]));
+        dq[0] = d01.x;
+        dq[1] = d01.y;
+        dq[S > 2 ? 2 : 0] = fmaf(cr, U[S > 2 ? 2 : 0], dq[S > 2 ? 2 : 0]);
+        DP::dflux(bj, dq, E);
+        const float2 a01 = f2fma(f2dup(wk), make_float2(E[0], E[1]), make_float2(acc[0], acc[1]));
+        acc[0] = a01.x;
+        acc[1] = a01.y;
+        acc[S > 2 ? 2 : 0] = fmaf(wk, E[S > 2 ? 2 : 0], acc[S > 2 ? 2 : 0]);
+      } else {
 #pragma unroll
-      for (int c = 0; c < NX; c++) xs1[q - 2 * NP][c] = fmaf(cr, X[c], xs1[q - 2 * NP][c]);
-      RP::rem(bj, xs1[q - 2 * NP], R1);
+        for (int c = 0; c < S; c++) dq[c] = fmaf(cr, U[c], dq[c]);
+        DP::dflux(bj, dq, E);
 #pragma unroll
-      for (int c = 0; c < NR; c++) A[c] = fmaf(wk, R1[c], A[c]);
+        for (int c = 0; c < S; c++) acc[c] = fmaf(wk, E[c], acc[c]);
+      }
     }
+    if constexpr (S == 3 && p >= 3) {
+      // a + (x + y) and the order's Taylor sum, components 0 and 1 packed
+      const float ifk = TB::invfact(k);
+      const float2 s01 = f2add(make_float2(acc[0], acc[1]),
+                               f2add(make_float2(acc2[0].x, acc2[1].x), make_float2(acc2[0].y, acc2[1].y)));
+      const float2 f01 = f2fma(f2dup(ifk), s01, make_float2(Fsum[0], Fsum[1]));
+      Fprev[0] = s01.x;
+      Fprev[1] = s01.y;
+      Fsum[0] = f01.x;
+      Fsum[1] = f01.y;
+      constexpr int c2 = S > 2 ? 2 : 0;
+      acc[c2] += acc2[c2].x + acc2[c2].y;
+      Fprev[c2] = acc[c2];
+      Fsum[c2] = fmaf(ifk, acc[c2], Fsum[c2]);
+    } else {
 #pragma unroll
-    for (int c = 0; c < NR; c++) A[c] = __fadd_rn(A[c], __fadd_rn(A2[c].x, A2[c].y));
-    RP::add(bj, U, A, F);
-#pragma unroll
-    for (int c = 0; c < S; c++) {
-      Fprev[c] = F[c];
-      Fsum[c] = fmaf(TB::invfact(k), F[c], Fsum[c]);
+      for (int c = 0; c < S; c++) {
+        acc[c] += acc2[c].x + acc2[c].y;
+        Fprev[c] = acc[c];
+        Fsum[c] = fmaf(TB::invfact(k), acc[c], Fsum[c]);
+      }
     }
   }
   const float w = TB::gh(p, l);
 #pragma unroll
-  for (int c = 0; c < S; c++) Gout[c] = group_sum<n>(mask, base, l, __fmul_rn(w, Fsum[c]));
+  for (int c = 0; c < S; c++) {
+    const float v = w * Fsum[c];
+    float t = 0.0f;
+#pragma unroll
+    for (int r = 0; r < n; r++) t += __shfl_sync(mask, v, base + r);
+    Gout[c] = t;
+  }
 }
 
 // cat_delta by a group of 4p lanes, two per node: lane l <-> node
@@ -569,12 +507,10 @@ __device__ __forceinline__ void cat_delta2(const float *hi, const float *lo, int
     dh[c] = uj[c] - ui[c];
     dl[c] = ujl[c] - uil[c];
   }
-  using RP = RPhys<FLUX>;
-  constexpr int NX = RP::NX, NR = RP::NR, NXA = NX > 0 ? NX : 1, NRA = NR > 0 ? NR : 1;
   float D[S], Fsum[S], Fprev[S];
-  float2 xs2[KP][NXA];
+  float2 del2[KP][S];
   DP::dflux_pair(DP::base2(ui, uil, adv, gm1), dh, dl, D);  // f(u_j) - f(u_i)
-  const typename RP::Base bj = RP::base(uj, ujl, adv, gm1);
+  const typename DP::Base bj = DP::base2(uj, ujl, adv, gm1);
 #pragma unroll
   for (int c = 0; c < S; c++) {
     Fsum[c] = D[c];
@@ -583,7 +519,7 @@ __device__ __forceinline__ void cat_delta2(const float *hi, const float *lo, int
 #pragma unroll
   for (int q = 0; q < KP; q++)
 #pragma unroll
-    for (int c = 0; c < NX; c++) xs2[q][c] = f2dup(RP::init(bj, c));
+    for (int c = 0; c < S; c++) del2[q][c] = make_float2(0.0f, 0.0f);
 #pragma unroll
   for (int k = 2; k <= n; k++) {
     float U[S];
@@ -595,13 +531,11 @@ __device__ __forceinline__ void cat_delta2(const float *hi, const float *lo, int
       for (int c = 0; c < S; c++) U[c] = fmaf(g1h[i], __shfl_sync(mask, Fprev[c], base + 2 * (h * p + i)), U[c]);
 #pragma unroll
     for (int c = 0; c < S; c++) U[c] = -lam * (U[c] + __shfl_xor_sync(mask, U[c], 1));
-    float X[NXA], F[S], A[NRA];
-    float2 A2[NRA];
-    RP::lin(bj, U, X, F);
+    float2 acc2[S];
 #pragma unroll
-    for (int c = 0; c < NR; c++) A2[c] = make_float2(0.0f, 0.0f);
+    for (int c = 0; c < S; c++) acc2[c] = make_float2(0.0f, 0.0f);
 #pragma unroll
-    for (int q = 0; q < (NX > 0 ? KP : 0); q++) {
+    for (int q = 0; q < KP; q++) {
       // the slot's two levels in either half (a level >= NL is empty)
       float cr0[2], cr1[2], wk0[2], wk1[2];
 #pragma unroll
@@ -616,23 +550,19 @@ __device__ __forceinline__ void cat_delta2(const float *hi, const float *lo, int
       }
       const float2 cr = h ? make_float2(cr1[0], cr1[1]) : make_float2(cr0[0], cr0[1]);
       const float2 wk = h ? make_float2(wk1[0], wk1[1]) : make_float2(wk0[0], wk0[1]);
-      float2 R2[NRA];
+      float2 E2[S];
 #pragma unroll
-      for (int c = 0; c < NX; c++) xs2[q][c] = f2fma(cr, f2dup(X[c]), xs2[q][c]);
-      RP::rem2(bj, xs2[q], R2);
+      for (int c = 0; c < S; c++) del2[q][c] = f2fma(cr, f2dup(U[c]), del2[q][c]);
+      DP::dflux_x2(bj, del2[q], E2);
 #pragma unroll
-      for (int c = 0; c < NR; c++) A2[c] = f2fma(wk, R2[c], A2[c]);
+      for (int c = 0; c < S; c++) acc2[c] = f2fma(wk, E2[c], acc2[c]);
     }
-#pragma unroll
-    for (int c = 0; c < NR; c++) {
-      A[c] = __fadd_rn(A2[c].x, A2[c].y);
-      A[c] = __fadd_rn(A[c], __shfl_xor_sync(mask, A[c], 1));
-    }
-    RP::add(bj, U, A, F);
 #pragma unroll
     for (int c = 0; c < S; c++) {
-      Fprev[c] = F[c];
-      Fsum[c] = fmaf(TB::invfact(k), F[c], Fsum[c]);
+      float a = acc2[c].x + acc2[c].y;
+      a += __shfl_xor_sync(mask, a, 1);
+      Fprev[c] = a;
+      Fsum[c] = fmaf(TB::invfact(k), a, Fsum[c]);
     }
   }
   const float w = TB::gh(p, m);
@@ -1035,7 +965,7 @@ __device__ __forceinline__ void tile_f64(const Step1DArgs &a, Smem64<P, FLUX, NW
 // group). thi, tlo: component 0 of the staged tile (components tw apart),
 // cell k of the tile at index k; interface il lies between tile cells
 // il - 1 + GH and il + GH. xw: the warp's exchange slots. The lanes of an
-// active group returns the code p_s and lane 0 G (lanes beyond the selected order's
+// active group return the code p_s, and lane 0 G (lanes beyond the selected order's
 // 2p return G unset).
 // rej (nullable): the tile's rejected orders per (component, interface), from
 // reject_pass_f32; the group then ORs its interface's bits instead of

@@ -1,7 +1,9 @@
 """Algorithmic operation counts of the ACAT step (roofline numerators): the
 reference count of the method's work (a Horner pass per time level, the
-*_ref functions), and the leaner count of the formulation the CUDA kernels
-use (running Taylor sums, the other functions).
+*_ref functions), and the leaner count of the running-Taylor-sum formulation
+(the other functions). The CUDA kernels do less than either: one Jacobian product
+per order in place of the linear part of all its time levels, and for linear
+transport no time levels (linear_step_flops).
 
 Counting convention: an FMA is 2 flops; add, multiply, divide and square root
 are 1 each. Counts are per interface for the flux work and per cell for the
@@ -81,6 +83,16 @@ def step_flops_1d(order_hist: dict, P: int, flux: int, cells: int) -> float:
     nif = sum(order_hist.values())
     f += nif * indicator_flops(P, flux) + cells * update_flops(flux)
     return f
+
+
+def linear_step_flops(order_hist: dict, P: int, cells: int) -> float:
+    """Flops of one 1D linear-transport step as the kernels form it: per order
+    U = -lambda a sum_r g1 F and F = a U at the n nodes, and the flux sums."""
+    f = 0.0
+    for code, cnt in order_hist.items():
+        n = 2 * code
+        f += cnt * (flcat2_flops(0) if code == 1 else n + (n - 1) * (2 * n * n + 2 * n) + 2 * n)
+    return f + sum(order_hist.values()) * indicator_flops(P, 0) + cells * update_flops(0)
 
 
 def cat2d_flops(p: int, flux: int) -> int:
