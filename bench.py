@@ -8,7 +8,8 @@ Riemann data with an entropy wave. One benchmark step is one full run of the
 the CFL dt reduced on the device) from the resident initial state.
 
 Metric: cell-updates/s (cells x ACAT steps / time), FP64. The JSON line also
-carries the roofline of the step kernel (FP64 FMA pipe, measured live), the
+carries the roofline of the step kernel (FP32 FMA pipes, measured live: the
+FP64 flux recursion runs on them in float-float pairs), the
 end-to-end number through the host-buffer entry point, the CPU oracle as a
 baseline, and variants (P = 2; FP32 when built).
 
@@ -216,7 +217,7 @@ def run_reference(args):
 
 
 KERNEL_SOURCES = [os.path.join(ROOT, "paper_2007_01416_gb300", "csrc", f)
-                  for f in ("step1d.cu", "step1d_core.cuh", "phys1d.cuh", "device_common.cuh")]
+                  for f in ("step1d.cu", "step1d_core.cuh", "split1d.cuh", "phys1d.cuh", "device_common.cuh")]
 
 
 def sources_sha(paths) -> str:
@@ -431,7 +432,7 @@ def measure_2d_hi(torch, acat, W, flops, n, P, steps, K, flush, peak, prec=0):
     t = min(ms)
     ctx.close()
     return {"value": n * n * steps / (t * 1e-3), "unit": UNIT, "ms_per_run": t, "steps": steps, "n": n,
-            "P": P, "roofline_frac": fl / (t / steps * 1e-3) / peak, "roofline_peak": "fp64",
+            "P": P, "roofline_frac": fl / (t / steps * 1e-3) / peak, "roofline_peak": "fp32",
             "blocks_per_anchor": {str(p): round(blocks[p] / (n * n), 4) for p in blocks},
             "flcat2_directions": round(flc / (2 * n * n), 4)}
 
@@ -480,7 +481,7 @@ def measure_2d_rect(torch, acat, W, flops, n, P, steps, K, flush, peak, prec=0):
     t = min(ms)
     ctx.close()
     return {"value": n * n * steps / (t * 1e-3), "unit": UNIT, "ms_per_run": t, "steps": steps, "n": n,
-            "P": P, "roofline_frac": fl / (t / steps * 1e-3) / peak, "roofline_peak": "fp64",
+            "P": P, "roofline_frac": fl / (t / steps * 1e-3) / peak, "roofline_peak": "fp32",
             "rect_blocks_per_anchor": round(rect / (n * n), 4),
             "square_blocks_per_anchor": round(int((blk & (pF == pG)).sum()) / (n * n), 4),
             "flcat2_directions": round(flc / (2 * n * n), 4)}
@@ -715,13 +716,13 @@ def measure_linear(torch, acat, W, flops, prec, P, nx, steps, K, flush, peak):
     ctx.acat_step(u, tmp, -1.0, None, None, orders)
     torch.cuda.synchronize()
     h = np.bincount(orders.cpu().numpy().astype(np.int64), minlength=5)
-    fl = flops.step_flops_1d({k: int(h[k]) for k in range(1, 5)}, P, W.LINEAR, nx)
+    fl = flops.linear_step_flops({k: int(h[k]) for k in range(1, 5)}, P, nx)
     fl_ref = flops.step_flops_1d_ref({k: int(h[k]) for k in range(1, 5)}, P, W.LINEAR, nx)
     t = min(ms)
     ctx.close()
-    # the reference count's Horner pass per time level dominates when the flux
-    # costs one flop, and the kernel's running sums do not do that work: the
-    # formulation count is the roofline numerator here, the other one is shown
+    # the reference count's time levels dominate when the flux costs one flop, and
+    # the kernel has none for a linear flux: its own count is the roofline
+    # numerator here, the other one is shown
     return {"value": nx * steps / (t * 1e-3), "unit": UNIT, "steps": steps, "nx": nx, "P": P,
             "roofline_frac": fl / (t / steps * 1e-3) / peak,
             "roofline_frac_reference_count": fl_ref / (t / steps * 1e-3) / peak,
@@ -782,18 +783,18 @@ def run_ours(args):
         vms = sum(v["ms"]) / 2
         variants["P2_f64"] = {
             "value": cells_steps / (vms * 1e-3), "unit": UNIT, "ms_per_step": vms,
-            "roofline_frac": v["flops_per_step_ref"] / (vms / args.acat_steps * 1e-3) / peak64,
-            "roofline_frac_formulation_count": v["flops_per_step"] / (vms / args.acat_steps * 1e-3) / peak64,
-            "order_mix": v["order_mix"]}
+            "roofline_frac": v["flops_per_step_ref"] / (vms / args.acat_steps * 1e-3) / peak32,
+            "roofline_frac_formulation_count": v["flops_per_step"] / (vms / args.acat_steps * 1e-3) / peak32,
+            "roofline_peak": "fp32", "order_mix": v["order_mix"]}
         # the switchable variants of FL-CAT2 and the p = 2 indicator: psi~^2 and HLL
         v = measure(torch, acat, W, flops, NX, P_MAIN, acat.PREC_F64, args.acat_steps, 2, 1, flush,
                     False, dev_index, extra={"psi2_mod": 1, "lo_flux": acat.LO_HLL})
         vms = sum(v["ms"]) / 2
         variants["P4_f64_psi2mod_hll"] = {
             "value": cells_steps / (vms * 1e-3), "unit": UNIT, "ms_per_step": vms,
-            "roofline_frac": v["flops_per_step_ref"] / (vms / args.acat_steps * 1e-3) / peak64,
-            "roofline_frac_formulation_count": v["flops_per_step"] / (vms / args.acat_steps * 1e-3) / peak64,
-            "order_mix": v["order_mix"]}
+            "roofline_frac": v["flops_per_step_ref"] / (vms / args.acat_steps * 1e-3) / peak32,
+            "roofline_frac_formulation_count": v["flops_per_step"] / (vms / args.acat_steps * 1e-3) / peak32,
+            "roofline_peak": "fp32", "order_mix": v["order_mix"]}
         for P in (4, 2):
             v = measure(torch, acat, W, flops, NX, P, acat.PREC_F32, args.acat_steps, 3, 1, flush,
                         False, dev_index, shape="auto")
@@ -823,9 +824,8 @@ def run_ours(args):
         # 2D Euler, P = 2: 4096^2 x 500 steps in FP32 (the 2D configuration), and the
         # plain FP64 step at 1024^2 x 20 steps for the FP32 / FP64 ratio
         v32 = measure_2d(torch, acat, W, flops, 4096, acat.PREC_F32, 500, 2, flush, peak32)
-        v64 = measure_2d(torch, acat, W, flops, 1024, acat.PREC_F64, 20, 2, flush, peak64)
-        v32["roofline_peak"] = "fp32"
-        v64["roofline_peak"] = "fp64"
+        v64 = measure_2d(torch, acat, W, flops, 1024, acat.PREC_F64, 20, 2, flush, peak32)
+        v32["roofline_peak"] = v64["roofline_peak"] = "fp32"
         v32["speedup_vs_f64_per_cell_update"] = v32["value"] / v64["value"]
         c2 = W.euler2d_quadrants(n=4096, seed=SEED, P=2, steps=500, cfl=CFL)
         v32["accuracy"] = f32_error(torch, acat, c2.problem_kwargs(), c2.u0, 10)
@@ -834,14 +834,13 @@ def run_ours(args):
         variants["2d_euler_P2_1024_f64"] = v64
         # the high-order 2D step (square blocks, P = 3)
         variants["2d_euler_P3_smooth_1024_f64"] = measure_2d_hi(torch, acat, W, flops, 1024, 3, 10, 2, flush,
-                                                                peak64)
+                                                                peak32)
         # rectangular stencils S_{p1,p2} on four-quadrant data at P = 4
         variants["2d_euler_P4_quadrants_rect_512_f64"] = measure_2d_rect(torch, acat, W, flops, 512, 4, 4, 2,
-                                                                         flush, peak64)
+                                                                         flush, peak32)
         # the same two high-order 2D workloads in FP32 (compensated state)
         h32 = measure_2d_hi(torch, acat, W, flops, 1024, 3, 10, 2, flush, peak32, prec=acat.PREC_F32)
         r32 = measure_2d_rect(torch, acat, W, flops, 512, 4, 4, 2, flush, peak32, prec=acat.PREC_F32)
-        h32["roofline_peak"] = r32["roofline_peak"] = "fp32"
         ch = W.euler2d_smooth(n=1024, seed=SEED, P=3, steps=10)
         h32["accuracy"] = f32_error(torch, acat, ch.problem_kwargs(), ch.u0, 10)
         cr = W.euler2d_quadrants(n=512, seed=SEED, P=4, steps=4)
@@ -853,8 +852,8 @@ def run_ours(args):
         # batched: 4096 ragged instances (P = 3), 1000 steps in FP32, and 10 steps of
         # the plain FP64 step for the ratio
         b32 = measure_batch(torch, acat, W, flops, acat.PREC_F32, 1000, 1, flush, peak32)
-        b64 = measure_batch(torch, acat, W, flops, acat.PREC_F64, 10, 1, flush, peak64)
-        b32["roofline_peak"], b64["roofline_peak"] = "fp32", "fp64"
+        b64 = measure_batch(torch, acat, W, flops, acat.PREC_F64, 10, 1, flush, peak32)
+        b32["roofline_peak"] = b64["roofline_peak"] = "fp32"
         b32["speedup_vs_f64_per_cell_update"] = b32["value"] / b64["value"]
         import numpy as np
         sizes, states = W.euler1d_batched(n_inst=4096, seed=SEED)
@@ -896,21 +895,22 @@ def run_ours(args):
         "config": {"workload": WORKLOAD, "nx": NX, "P": P_MAIN, "acat_steps": args.acat_steps,
                    "precision": "f64", "cfl": CFL, "seed": SEED,
                    "l2": "256 MiB buffer written between timed runs; the 0.4 MB state is "
-                         "L2-resident within a run (the step is FP64-pipe bound)"},
-        "roofline": {"bound": "alu", "achieved": achieved / 1e12, "peak": peak64 / 1e12,
-                     "unit": "TFLOP/s", "frac": achieved / peak64,
+                         "L2-resident within a run (the step is bound by instruction issue)"},
+        "roofline": {"bound": "alu", "achieved": achieved / 1e12, "peak": peak32 / 1e12,
+                     "unit": "TFLOP/s", "frac": achieved / peak32,
                      "traffic": profile_traffic(KERNEL_SOURCES),
-                     "kernel": f"k_step1d_fine<{P_MAIN}, EULER1D> (2-warp CTAs, one launch per step)",
-                     "peak_source": "measured live: FP64 FMA-chain kernel on all SMs (best of 3); "
-                                    "the measured HBM and bf16 peaks do not bound this FP64-pipe kernel",
+                     "kernel": f"k_step1d_f64<{P_MAIN}, EULER1D> (one launch per step)",
+                     "peak_source": "measured live: FP32 FMA-chain kernel on all SMs (best of 3): the flux "
+                                    "recursion reaches FP64 accuracy in float-float pairs, some 10 FP32 "
+                                    "instructions per counted operation; the FP64 peak is in fma_peaks_tflops",
                      "flop_count": "reference count of the method (a Horner pass per time level; "
                                    "18304 flops per interface at p = 4)",
                      "flops_per_launch": m["flops_per_step_ref"], "kernel_ms": kernel_ms,
                      "formulation_count": {
-                         "what": "the kernel's own formulation (running Taylor sums; 12112 flops per "
-                                 "interface at p = 4)",
+                         "what": "running Taylor sums (12112 flops per interface at p = 4); the "
+                                 "kernel does one Jacobian product per order and the remainders",
                          "flops_per_launch": m["flops_per_step"], "achieved": achieved_form / 1e12,
-                         "frac": achieved_form / peak64},
+                         "frac": achieved_form / peak32},
                      "order_mix": m["order_mix"]},
         "e2e": {"value": e2e_val, "unit": UNIT, "h2d_bytes_per_step": sb, "d2h_bytes_per_step": sb,
                 "ms_per_step": e2e_best},
