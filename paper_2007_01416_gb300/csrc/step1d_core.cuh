@@ -806,8 +806,7 @@ __device__ __forceinline__ void cat_iface_f64(const Step1DArgs &a, Smem64<P, FLU
       const int xo = warp * 2 * XSET + (P >= 3 ? xslot(base) : base);
       ok = cat_split_euler<p, TW>(sm.rec, a, sm.tab, sm.lamk.v[p - 2], ic, l, base, &sm.xa[xo], &sm.xb[xo], G);
     } else {
-      ok = cat_split_burgers<p, TW>(sm.rec, (float)a.cfl * __frcp_rn((float)lam), sm.tab, sm.lamk.v[p - 2], ic, l,
-                                    base, G);
+      ok = cat_split_burgers<p, TW>(sm.rec, sm.tab, sm.lamk.v[p - 2], ic, l, base, G);
     }
     if (ok) {
       if (l == 0) {
