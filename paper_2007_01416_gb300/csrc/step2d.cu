@@ -1361,7 +1361,10 @@ struct Smem2H {
   SplitLam slx, sly;
   SplitTab tab;
   unsigned char cF[TXH][TXH + 1], cG[TXH + 1][TXH];  // p where the flux is a pair, else 0
-  int bad[NT / 16], nfail;
+  struct {
+    int bad, big[2], quad, cub, redo;  // stamps of a slot's last objections
+  } vote[NT / 16];
+  int nfail;
   unsigned rej[NAH * NAH];    // rejected orders: bit dir * (P - 1) + (p - 2)
   unsigned short task[P + 1][2 * NAH * NAH];
   int ntask[P + 1];
@@ -1630,10 +1633,13 @@ __device__ __forceinline__ void rect_tasks(Smem2H<P, FLUX> &sm, const Step2DArgs
 }
 
 // The block tasks of order p in float-float pairs (split2d.cuh), one thread per
-// node, NT / (2p)^2 tasks per round. The choices of precision are those of the
-// round (one vote of the CTA with the barriers that the exchange needs anyway);
-// the tasks whose increments are too large for the pairs are left in
-// sm.task[p][0 .. ntask) for block_tasks, the FP64 recursion.
+// node, NT / (2p)^2 tasks per round. Every choice of precision is the block's own:
+// which blocks share a round depends on the order in which the warps filled the list, and
+// the fluxes on a tile's edge are formed by two CTAs. A node that objects writes the
+// vote's stamp to its slot's word before a barrier that the exchange needs anyway, and
+// the slot's threads compare after it (stamps only grow, so no word is reset). Blocks
+// whose increments are too large for the pairs drop out and are left in sm.task[p][0 .. ntask)
+// for block_tasks, the FP64 recursion.
 template <int p, int P, int FLUX>
 __device__ __forceinline__ void split_tasks(Smem2H<P, FLUX> &sm, const Step2DArgs &a) {
   constexpr int n = 2 * p, nn = n * n, per = NT / nn, z = p - 1, TW = Smem2H<P, FLUX>::TW;
@@ -1650,85 +1656,100 @@ __device__ __forceinline__ void split_tasks(Smem2H<P, FLUX> &sm, const Step2DArg
   }
   const int i0 = ti * nn + ib * n, j0 = ti * nn + ia;
   const int dir = (node >> 2) & 1, fc = node & 3, f0 = ti * nn + (dir ? z : z * n), fs = dir ? n : 1;
+  auto &V = sm.vote[ti];  // idle threads past the last slot have one of their own
+  if (tid < NT / 16) sm.vote[tid] = {};
   if (tid == 0) sm.nfail = 0;
+  __syncthreads();
+  int stamp = 0;
 #pragma unroll 1
   for (int base = 0; base < nt; base += per) {
     const bool act = ti < per && base + ti < nt;
     const unsigned tk = act ? sm.task[p][base + ti] : 0u;
     const int an = (int)(tk & 0xffu);
     const int ax = an % NAH - 1, ay = an / NAH - 1;
+    bool live = act;  // not yet delivered
     int form = 0;
-    FF S;
 #pragma unroll 1
     for (;;) {
-      if (tid < per) sm.bad[tid] = 0;
-      __syncthreads();
       Split2Node<p> N;
-      FF F[4], G[4];
-      if (act) {
+      FF F[4], G[4], S{0.0f, 0.0f};
+      stamp++;
+      if (live) {
         const int tx = acat_tile_index(ax + P - p + 1 + ia, TW, a.status);
         const int ty = acat_tile_index(ay + P - p + 1 + ib, TW, a.status);
-        if (!split2_start(C, sm.rec[ty * TW + tx], sm.rec[(ay + P) * TW + ax + P], N, F, G)) sm.bad[ti] = 1;
+        if (!split2_start(C, sm.rec[ty * TW + tx], sm.rec[(ay + P) * TW + ax + P], N, F, G)) V.bad = stamp;
+        if (!split2_small(N, F, G)) V.big[0] = stamp;
         split2_put(xs, tid, F, G);
       }
       __syncthreads();
-      const bool off = !act || sm.bad[ti] != 0;  // no say in the round's votes
-      S = FF{0.0f, 0.0f};
-      if (act && node < 8) split2_flux<p>(xs, sm.tab, dir, fc, f0, fs, 840.0f, S);
+      bool on = live && V.bad != stamp, tail = form == 0 && V.big[0] != stamp;
+      if (on && node < 8) split2_flux<p>(xs, sm.tab, dir, fc, f0, fs, 840.0f, S);
       N.form = form;
-      bool tail = false;
 #pragma unroll 1
       for (int k = 2; k <= n; k++) {
         const float2 lx = sm.slx.v[p - 2][k - 2], ly = sm.sly.v[p - 2][k - 2], *lv = sm.tab.lv[p - 2][k - 2];
-        if (!tail && N.form < 2 && (k > 2 || N.form == 0))
-          tail = __syncthreads_and(off || split2_small(N, F, G)) != 0;
-        if (tail) {
-          if (act) split2_tail(C, N, k, lv, xs, i0, j0, n, gx, gy, lx.x, ly.x, F, G);
-        } else {
-          FF u[4];
-          Split2Lin o;
-          if (act) {
-            split2_sums<p>(xs, i0, j0, n, gx, gy, ff_of(lx), ff_of(ly), u);
-            o = split2_lin(C, N.v, N.w, N.h, u);
-            split2_bounds(N, lv, u[0].h, o.W1.h, o.W2.h, o.L.h);
+        FF u[4];
+        Split2Lin o;
+        if (on && !tail) {
+          split2_sums<p>(xs, i0, j0, n, gx, gy, ff_of(lx), ff_of(ly), u);
+          o = split2_lin(C, N.v, N.w, N.h, u);
+          split2_bounds(N, lv, u[0].h, o.W1.h, o.W2.h, o.L.h);
+        }
+        if (k == 2) {
+          stamp++;
+          if (on && !tail) {
+            if (!split2_held(N)) V.bad = stamp;  // the bounds only grow
+            if (N.form == 0 && !split2_quad(N, 2.0f)) V.quad = stamp;
+            if (N.form <= 1 && !split2_cubic(N, 1.6f)) V.cub = stamp;
           }
-          if (k == 2) {
-            if (N.form == 0 && !__syncthreads_and(off || split2_quad(N, 2.0f))) N.form = 1;
+          __syncthreads();
+          on = on && V.bad != stamp;
+          if (on && !tail) {
+            if (N.form == 0 && V.quad == stamp) N.form = 1;
             if (N.form == 1) {
-              if (!__syncthreads_and(off || split2_cubic(N, 1.6f))) N.form = 2;
-              if (act) split2_first(N, o);
+              if (V.cub == stamp) N.form = 2;
+              split2_first(N, o);
             }
           }
-          if (act) split2_order(C, N, k, lv, u, o, F, G);
         }
+        if (on) {
+          if (tail) split2_tail(C, N, k, lv, xs, i0, j0, n, gx, gy, lx.x, ly.x, F, G);
+          else split2_order(C, N, k, lv, u, o, F, G);
+        }
+        stamp++;
+        if (on && !split2_small(N, F, G)) V.big[(k & 1) ^ 1] = stamp;  // the other word may still be read
         __syncthreads();
-        if (act) split2_put(xs, tid, F, G);
+        if (on) split2_put(xs, tid, F, G);
         __syncthreads();
-        if (act && node < 8) split2_flux<p>(xs, sm.tab, dir, fc, f0, fs, sm.tab.k840[k - 1], S);
+        tail |= N.form < 2 && V.big[(k & 1) ^ 1] != stamp;
+        if (on && node < 8) split2_flux<p>(xs, sm.tab, dir, fc, f0, fs, sm.tab.k840[k - 1], S);
       }
-      if (!off && !split2_held(N)) sm.bad[ti] = 1;
-      // (off is the state before this order's verdict: a block that fails here
-      // has no say in whether the round repeats)
-      if (__syncthreads_and(off || !split2_held(N) || split2_form(N))) break;
+      stamp++;
+      if (on) {
+        if (!split2_held(N)) V.bad = stamp;
+        else if (!split2_form(N)) V.redo = stamp;
+      }
+      __syncthreads();
+      const bool fail = live && (!on || V.bad == stamp), again = live && !fail && V.redo == stamp;
+      if (live && !again) {
+        if (fail) {
+          if (node == 0) sm.task[p][atomicAdd(&sm.nfail, 1)] = (unsigned short)tk;  // below base + per: read already
+        } else if (node < 8) {
+          const float2 v = make_float2(S.h, S.l);
+          if (dir == 0 && (tk & WANT_F)) {
+            *reinterpret_cast<float2 *>(&sm.Fx[ay][ax + 1][fc]) = v;
+            if (fc == 0) sm.cF[ay][ax + 1] = (unsigned char)p;
+          }
+          if (dir == 1 && (tk & WANT_G)) {
+            *reinterpret_cast<float2 *>(&sm.Gy[ay + 1][ax][fc]) = v;
+            if (fc == 0) sm.cG[ay + 1][ax] = (unsigned char)p;
+          }
+        }
+      }
       form = N.form + 1;
+      live = again;
+      if (!__syncthreads_or(again)) break;
     }
-    __syncthreads();
-    if (act) {
-      if (sm.bad[ti]) {
-        if (node == 0) sm.task[p][atomicAdd(&sm.nfail, 1)] = (unsigned short)tk;  // below base + per: read already
-      } else if (node < 8) {
-        const float2 v = make_float2(S.h, S.l);
-        if (dir == 0 && (tk & WANT_F)) {
-          *reinterpret_cast<float2 *>(&sm.Fx[ay][ax + 1][fc]) = v;
-          if (fc == 0) sm.cF[ay][ax + 1] = (unsigned char)p;
-        }
-        if (dir == 1 && (tk & WANT_G)) {
-          *reinterpret_cast<float2 *>(&sm.Gy[ay + 1][ax][fc]) = v;
-          if (fc == 0) sm.cG[ay + 1][ax] = (unsigned char)p;
-        }
-      }
-    }
-    __syncthreads();
   }
   __syncthreads();
   if (tid == 0) sm.ntask[p] = sm.nfail;
