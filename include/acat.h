@@ -172,10 +172,11 @@ int acat_create_batched(const acat_params *p, int n_inst, const int32_t *n_per_i
  *     nw and cps only move work between CTAs: every interface flux, wave
  *     speed and update is computed from the same values, so the states are
  *     bit-identical.
- *   - Single-instance contexts: cps is 0. FP64: nw is fixed, 8 or, for large
- *     grids, 2: a label of the grid size, so that shapes a caller has stored
- *     still apply; the step picks its tiles by a rule on P and N. FP32: nw = 8 (the fused step, lpn 1
- *     or 2), nw = 7 (the fused step in tiles of 7 floor(32 / 2P) - 1
+ *   - Single-instance contexts: cps is 0. FP64: nw is fixed, 4 to 8 by a rule
+ *     on P, N and the SM count (which also sets the interface rounds of a tile);
+ *     acat_set_launch_shape changes nothing there and accepts that nw, and the 8 or,
+ *     for large grids, 2 that earlier versions reported. FP32: nw = 8 (the fused step,
+ *     lpn 1 or 2), nw = 7 (the fused step in tiles of 7 floor(32 / 2P) - 1
  *     cells, lpn = 1: a grid of a few waves then fills every SM with the
  *     same number of CTAs) or nw = 2 (the small-CTA step with the boundary
  *     hand-off, lpn = 1); all compute every interface and cell from the

@@ -54,7 +54,7 @@ struct acat_ctx {
   float *d_flux = nullptr;                // 1D FP32: CTA-edge increments of the small-CTA step
   int *d_cnt = nullptr;                   // 1D: its boundary hand-off counters
   int snw = 8;                            // 1D single instance: FP32 warps per CTA (8 or 7 fused, 2 small-CTA);
-                                          // FP64 the reported label (8, or 2 for large grids)
+                                          // FP64 a value that shapes stored by callers may hold (8 or 2)
   int fnw = 8, frounds = 1;               // 1D FP64: warps per CTA and interface rounds
   int sms = 0;
 };
@@ -397,8 +397,9 @@ int acat_create(const acat_params *p, acat_ctx **out) {
   int sms = 0;
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
   c->sms = sms;
-  // 1D FP64: the tile shape, and the label acat_launch_shape reports (2 where
-  // 8-warp tiles of one round would exceed 3/4 of a wave at 2 CTAs per SM)
+  // 1D FP64: the tile shape. snw: what acat_launch_shape reported when the step had
+  // CTAs of 8 warps, or of 2 where 8-warp tiles of one round would exceed 3/4 of a wave
+  // at 2 CTAs per SM; acat_set_launch_shape still takes it from callers that stored it
   if (e == cudaSuccess && c->dim == 1 && p->precision == ACAT_PREC_F64) {
     acat_shape_f64(p->P, p->nx, sms, &c->fnw, &c->frounds);
     const long T = acat_cells_per_cta_1d(p->P, ACAT_PREC_F64), ctas = (p->nx + T - 1) / T;
@@ -501,7 +502,7 @@ int acat_launch_shape(const acat_ctx *c, int *nw, int *lpn, int *cps) {
     w = c->bnw;
     k = c->bcps > 0 ? c->bcps : acat_batch_occupancy(c->p.P, c->p.flux, c->p.precision, c->bnw, c->lpn);
   } else {
-    w = c->snw;
+    w = c->p.precision != ACAT_PREC_F32 ? c->fnw : c->snw;
   }
   if (nw) *nw = w;
   if (lpn) *lpn = c->lpn;
@@ -513,11 +514,9 @@ int acat_set_launch_shape(acat_ctx *c, int nw, int lpn, int cps) {
   if (!c || cps < 0) return ACAT_ERR_INVALID_ARG;
   if (c->dim != 1) return ACAT_ERR_UNSUPPORTED;
   if (!c->batched) {
-    int w0 = 0, l0 = 0, k0 = 0;
-    acat_launch_shape(c, &w0, &l0, &k0);
     if (cps != 0) return ACAT_ERR_UNSUPPORTED;
     if (c->p.precision != ACAT_PREC_F32) {  // fixed for a single FP64 instance
-      if (nw != w0) return ACAT_ERR_UNSUPPORTED;
+      if (nw != c->fnw && nw != c->snw) return ACAT_ERR_UNSUPPORTED;
       return lpn == c->lpn ? ACAT_OK : ACAT_ERR_UNSUPPORTED;
     }
     // FP32: the fused step of 8 warps (one or two lanes per node) or 7 warps (one
