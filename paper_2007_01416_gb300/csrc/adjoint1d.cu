@@ -808,35 +808,46 @@ __global__ void __launch_bounds__(NWA * 32) k_adj1d_split(const Step1DArgs a, co
   __syncwarp();
   const int grp = lane / TL::L, l = lane - grp * TL::L, il = warp * TL::GPW + grp, base = grp * TL::L;
   const long m = i0 + il;
-  if (grp < TL::GPW && m <= N) {
-    const int ic = il - 1 + TL::GH, ps = order(il);
-    if (ps > 1 && acat_in_bounds(ic - P + 1 >= 0 && ic + P < TL::TW, a.status)) {
-      double Fb[S], ub[S], *out = contrib + m * NS * S;
-      cotangent(m, Fb);
-      const double *q0 = &sm.tile[0][ic];
-      if (ps == 4) {
-        if constexpr (P >= 4)
-          if (!cat_adj_split<4, P>(a, sm, ic, l, base, warp, lane, Fb, ub))
-            cat_flux_adj<4, ACAT_FLUX_EULER1D>(q0, TL::TW, l, base, lam, a.adv, gm1, Fb, ub);
-      } else if (ps == 3) {
-        if constexpr (P >= 3)
-          if (l < 6 && !cat_adj_split<3, P>(a, sm, ic, l, base, warp, lane, Fb, ub))
-            cat_flux_adj<3, ACAT_FLUX_EULER1D>(q0, TL::TW, l, base, lam, a.adv, gm1, Fb, ub);
-      } else if (l < 4) {
-        if (!cat_adj_split<2, P>(a, sm, ic, l, base, warp, lane, Fb, ub))
-          cat_flux_adj<2, ACAT_FLUX_EULER1D>(q0, TL::TW, l, base, lam, a.adv, gm1, Fb, ub);
-      }
-      if (l < 2 * ps) {
-        const int s = (l - ps + 1) + NS / 2 - 1;
+  const int ic = il - 1 + TL::GH;
+  const bool mine = grp < TL::GPW && m <= N;
+  int ps = mine ? order(il) : 1;
+  if (ps > 1 && !acat_in_bounds(ic - P + 1 >= 0 && ic + P < TL::TW, a.status)) ps = 1;
+  double Fb[S], ub[S];
+  const double *q0 = &sm.tile[0][ic];
+  bool done = true;  // the lanes of a stencil that the pairs carry
+  if (ps > 1) {
+    cotangent(m, Fb);
+    if (ps == 4) {
+      if constexpr (P >= 4) done = cat_adj_split<4, P>(a, sm, ic, l, base, warp, lane, Fb, ub);
+    } else if (ps == 3) {
+      if constexpr (P >= 3)
+        if (l < 6) done = cat_adj_split<3, P>(a, sm, ic, l, base, warp, lane, Fb, ub);
+    } else if (l < 4) {
+      done = cat_adj_split<2, P>(a, sm, ic, l, base, warp, lane, Fb, ub);
+    }
+  }
+  __syncwarp();  // the warp's other stencils take the FP64 sweep together, wherever they left the pairs
+  if (!done) {
+    if (ps == 4) {
+      if constexpr (P >= 4) cat_flux_adj<4, ACAT_FLUX_EULER1D>(q0, TL::TW, l, base, lam, a.adv, gm1, Fb, ub);
+    } else if (ps == 3) {
+      if constexpr (P >= 3) cat_flux_adj<3, ACAT_FLUX_EULER1D>(q0, TL::TW, l, base, lam, a.adv, gm1, Fb, ub);
+    } else {
+      cat_flux_adj<2, ACAT_FLUX_EULER1D>(q0, TL::TW, l, base, lam, a.adv, gm1, Fb, ub);
+    }
+  }
+  if (ps > 1) {
+    double *out = contrib + m * NS * S;
+    if (l < 2 * ps) {
+      const int s = (l - ps + 1) + NS / 2 - 1;
 #pragma unroll
-        for (int c = 0; c < S; c++) out[s * S + c] = ub[c];
-      } else if (l < NS) {
-        // slots of nodes outside S_ps: zero (lanes 2ps..2P-1 cover them)
-        const int k = l - 2 * ps, s = k < NS / 2 - ps ? k : k + 2 * ps;
-        if (s >= 0 && s < NS)
+      for (int c = 0; c < S; c++) out[s * S + c] = ub[c];
+    } else if (l < NS) {
+      // slots of nodes outside S_ps: zero (lanes 2ps..2P-1 cover them)
+      const int k = l - 2 * ps, s = k < NS / 2 - ps ? k : k + 2 * ps;
+      if (s >= 0 && s < NS)
 #pragma unroll
-          for (int c = 0; c < S; c++) out[s * S + c] = 0.0;
-      }
+        for (int c = 0; c < S; c++) out[s * S + c] = 0.0;
     }
   }
   acat_pdl_release();
