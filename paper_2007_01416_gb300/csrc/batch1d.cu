@@ -54,18 +54,20 @@ __global__ void __launch_bounds__(NT) k_batch_dt(const Step1DArgs a, const Batch
   }
 }
 
-// Interface rounds per lane group in a tile of the FP32 batched step: eight
-// rounds (two at 16 warps, within 48 KB of static shared memory) make tiles
+// Interface rounds per lane group in a tile of the batched step: R rounds make tiles
 // of R NW GPW interfaces, so the tile's CTA barriers, order-decision pass and
-// update phase are shared by R times the flux work.
-template <bool F32, int NW>
+// update phase are shared by R times the flux work. FP32: eight (two at 16 warps, for
+// the shared memory). FP64: 32 / NW where a round is a recursion; at P = 1 a round is
+// one FL-CAT2 chain on the FP64 pipe, which only more and smaller tiles spread over the
+// SMs (60 instances of 40 to 4000 cells, Euler: 167 us a step with two rounds).
+template <int P, bool F32, int NW>
 struct Rounds {
-  static constexpr int value = F32 ? (NW >= 16 ? 2 : 8) : (NW >= 16 ? 1 : NW == 8 ? 2 : 4);
+  static constexpr int value = F32 ? (NW >= 16 ? 2 : 8) : (P == 1 || NW >= 16 ? 1 : NW == 8 ? 2 : 4);
 };
 
 // Persistent batched step: CTAs of NW warps take the tiles of the (instance,
 // first cell) work list, Tiling<P, NW, LPN, R>::T cells wide (R =
-// Rounds<F32, NW>), from a queue: CTA c starts with tile c,
+// Rounds<P, F32, NW>), from a queue: CTA c starts with tile c,
 // and each further tile is claimed with one atomic on the queue counter
 // (set to 0 by k_batch_dt), issued before the current tile so that its
 // latency hides behind the tile's work. Tiles cost unevenly (FL-CAT2
@@ -86,7 +88,7 @@ struct BatchCtas {
 template <int P, int FLUX, bool F32, int NW, int LPN>
 __global__ void __launch_bounds__(NW * 32, BatchCtas<P, F32>::value * 8 / NW)
     k_batch1d(const Step1DArgs a, const BatchArgs bt) {
-  constexpr int R = Rounds<F32, NW>::value;
+  constexpr int R = Rounds<P, F32, NW>::value;
   using SM =
       typename std::conditional<F32, Smem32<P, Phys<FLUX>::S, NW, LPN, R>, Smem64<P, FLUX, NW, R>>::type;
   // FP32: two workspaces used alternately (tile_f32 ends without a barrier)
@@ -254,12 +256,11 @@ int acat_batch_occupancy(int P, int flux, int prec, int nw, int lpn) {
 namespace {
 template <int NW, int LPN, bool F32>
 int cells_per_tile(int P) {
-  constexpr int R = Rounds<F32, NW>::value;
   switch (P) {
-  case 1: return Tiling<1, NW, LPN, R>::T;
-  case 2: return Tiling<2, NW, LPN, R>::T;
-  case 3: return Tiling<3, NW, LPN, R>::T;
-  case 4: return Tiling<4, NW, LPN, R>::T;
+  case 1: return Tiling<1, NW, LPN, Rounds<1, F32, NW>::value>::T;
+  case 2: return Tiling<2, NW, LPN, Rounds<2, F32, NW>::value>::T;
+  case 3: return Tiling<3, NW, LPN, Rounds<3, F32, NW>::value>::T;
+  case 4: return Tiling<4, NW, LPN, Rounds<4, F32, NW>::value>::T;
   }
   return 0;
 }
