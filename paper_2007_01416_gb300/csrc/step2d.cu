@@ -1364,7 +1364,8 @@ struct Smem2H {
   struct {
     int bad, big[2], quad, cub, redo;  // stamps of a slot's last objections
   } vote[NT / 16];
-  int nfail;
+  int nfail, nredo;
+  unsigned short redo[2 * NAH * NAH];  // blocks to repeat: a task word, its form in bits 10-11
   unsigned rej[NAH * NAH];    // rejected orders: bit dir * (P - 1) + (p - 2)
   unsigned short task[P + 1][2 * NAH * NAH];
   int ntask[P + 1];
@@ -1637,13 +1638,13 @@ __device__ __forceinline__ void rect_tasks(Smem2H<P, FLUX> &sm, const Step2DArgs
 // which blocks share a round depends on the order in which the warps filled the list, and
 // the fluxes on a tile's edge are formed by two CTAs. A node that objects writes the
 // vote's stamp to its slot's word before a barrier that the exchange needs anyway, and
-// the slot's threads compare after it (stamps only grow, so no word is reset). Blocks
-// whose increments are too large for the pairs drop out and are left in sm.task[p][0 .. ntask)
-// for block_tasks, the FP64 recursion.
+// the slot's threads compare after it (stamps only grow, so no word is reset). A block
+// whose remainders outgrew their form is repeated in later rounds, with others of its kind;
+// blocks whose increments are too large for the pairs drop out and are left in
+// sm.task[p][0 .. ntask) for block_tasks, the FP64 recursion.
 template <int p, int P, int FLUX>
 __device__ __forceinline__ void split_tasks(Smem2H<P, FLUX> &sm, const Step2DArgs &a) {
   constexpr int n = 2 * p, nn = n * n, per = NT / nn, z = p - 1, TW = Smem2H<P, FLUX>::TW;
-  const int nt = sm.ntask[p];
   const int tid = threadIdx.x, ti = tid / nn, node = tid - ti * nn;
   const int ia = node % n, ib = node / n;
   const Split2Const C = split2_const(a);
@@ -1658,23 +1659,22 @@ __device__ __forceinline__ void split_tasks(Smem2H<P, FLUX> &sm, const Step2DArg
   const int dir = (node >> 2) & 1, fc = node & 3, f0 = ti * nn + (dir ? z : z * n), fs = dir ? n : 1;
   auto &V = sm.vote[ti];  // idle threads past the last slot have one of their own
   if (tid < NT / 16) sm.vote[tid] = {};
-  if (tid == 0) sm.nfail = 0;
+  if (tid == 0) sm.nfail = sm.nredo = 0;
   __syncthreads();
-  int stamp = 0;
+  int stamp = 0, nt = sm.ntask[p];
+  const unsigned short *list = sm.task[p];
 #pragma unroll 1
-  for (int base = 0; base < nt; base += per) {
-    const bool act = ti < per && base + ti < nt;
-    const unsigned tk = act ? sm.task[p][base + ti] : 0u;
-    const int an = (int)(tk & 0xffu);
-    const int ax = an % NAH - 1, ay = an / NAH - 1;
-    bool live = act;  // not yet delivered
-    int form = 0;
+  while (nt > 0) {
 #pragma unroll 1
-    for (;;) {
+    for (int base = 0; base < nt; base += per) {
+      const bool act = ti < per && base + ti < nt;
+      const unsigned tk = act ? list[base + ti] : 0u;
+      const int an = (int)(tk & 0xffu), form = (int)(tk >> 10);
+      const int ax = an % NAH - 1, ay = an / NAH - 1;
       Split2Node<p> N;
       FF F[4], G[4], S{0.0f, 0.0f};
       stamp++;
-      if (live) {
+      if (act) {
         const int tx = acat_tile_index(ax + P - p + 1 + ia, TW, a.status);
         const int ty = acat_tile_index(ay + P - p + 1 + ib, TW, a.status);
         if (!split2_start(C, sm.rec[ty * TW + tx], sm.rec[(ay + P) * TW + ax + P], N, F, G)) V.bad = stamp;
@@ -1682,7 +1682,7 @@ __device__ __forceinline__ void split_tasks(Smem2H<P, FLUX> &sm, const Step2DArg
         split2_put(xs, tid, F, G);
       }
       __syncthreads();
-      bool on = live && V.bad != stamp, tail = form == 0 && V.big[0] != stamp;
+      bool on = act && V.bad != stamp, tail = form == 0 && V.big[0] != stamp;
       if (on && node < 8) split2_flux<p>(xs, sm.tab, dir, fc, f0, fs, 840.0f, S);
       N.form = form;
 #pragma unroll 1
@@ -1702,7 +1702,7 @@ __device__ __forceinline__ void split_tasks(Smem2H<P, FLUX> &sm, const Step2DArg
             if (N.form == 0 && !split2_quad(N, 2.0f)) V.quad = stamp;
             if (N.form <= 1 && !split2_cubic(N, 1.6f)) V.cub = stamp;
           }
-          __syncthreads();
+          if (!__syncthreads_or(on)) break;  // no block of the round is in pairs (any more)
           on = on && V.bad != stamp;
           if (on && !tail) {
             if (N.form == 0 && V.quad == stamp) N.form = 1;
@@ -1718,7 +1718,7 @@ __device__ __forceinline__ void split_tasks(Smem2H<P, FLUX> &sm, const Step2DArg
         }
         stamp++;
         if (on && !split2_small(N, F, G)) V.big[(k & 1) ^ 1] = stamp;  // the other word may still be read
-        __syncthreads();
+        if (!__syncthreads_or(on)) break;
         if (on) split2_put(xs, tid, F, G);
         __syncthreads();
         tail |= N.form < 2 && V.big[(k & 1) ^ 1] != stamp;
@@ -1730,10 +1730,13 @@ __device__ __forceinline__ void split_tasks(Smem2H<P, FLUX> &sm, const Step2DArg
         else if (!split2_form(N)) V.redo = stamp;
       }
       __syncthreads();
-      const bool fail = live && (!on || V.bad == stamp), again = live && !fail && V.redo == stamp;
-      if (live && !again) {
-        if (fail) {
-          if (node == 0) sm.task[p][atomicAdd(&sm.nfail, 1)] = (unsigned short)tk;  // below base + per: read already
+      if (act) {
+        const unsigned who = tk & 0x3ffu;
+        // both lists keep below base + per, which the round has read
+        if (!on || V.bad == stamp) {
+          if (node == 0) sm.task[p][atomicAdd(&sm.nfail, 1)] = (unsigned short)who;
+        } else if (V.redo == stamp) {
+          if (node == 0) sm.redo[atomicAdd(&sm.nredo, 1)] = (unsigned short)(who | (unsigned)(N.form + 1) << 10);
         } else if (node < 8) {
           const float2 v = make_float2(S.h, S.l);
           if (dir == 0 && (tk & WANT_F)) {
@@ -1746,10 +1749,12 @@ __device__ __forceinline__ void split_tasks(Smem2H<P, FLUX> &sm, const Step2DArg
           }
         }
       }
-      form = N.form + 1;
-      live = again;
-      if (!__syncthreads_or(again)) break;
+      __syncthreads();
     }
+    nt = sm.nredo;
+    list = sm.redo;
+    __syncthreads();
+    if (tid == 0) sm.nredo = 0;
   }
   __syncthreads();
   if (tid == 0) sm.ntask[p] = sm.nfail;
