@@ -83,7 +83,12 @@ enum {
  *   x0..y1        domain; cell centres x_i = x0 + (i + 1/2) dx.
  *   bc            ACAT_BC_PERIODIC or ACAT_BC_TRANSMISSIVE (zero-gradient
  *                 ghost cells, the "outflow"/"free" conditions of Sec. 5).
- *   precision     ACAT_PREC_F64, or ACAT_PREC_F32 (float arithmetic on a
+ *   precision     ACAT_PREC_F64 (FP64 state, decisions and update; the CAT2p
+ *                 fluxes of the nonlinear laws and the Jacobians of the Euler
+ *                 adjoint from pairs of floats where their increments are
+ *                 below fixed fractions of the stencil's own scales, with an
+ *                 error below that of the FP64 recursion, and in FP64
+ *                 elsewhere), or ACAT_PREC_F32 (float arithmetic on a
  *                 compensated float-pair state; the order decisions are
  *                 those of FP64 on the state value hi + lo).
  *   cfl           CFL number of the dt rule above.

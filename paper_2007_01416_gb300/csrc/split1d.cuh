@@ -28,18 +28,20 @@
 //     recursion at p = 4, 0.19 against 0.32 at p = 2; equal at 2^-3.5). Above TAU
 //     the caller evaluates the recursion in FP64. The remainders take one of
 //     three forms, by the size of the Taylor sums (time increments):
-//       0  in float, where the quadratic terms are below 2^-23 of the scales;
+//       0  in float, where the quadratic terms are below 2^-23 of the scales (Burgers:
+//          2^-25 of u^2);
 //       1  (2D blocks; in 1D it was slower than form 2: P = 4 at N = 262144
 //          261 -> 280 us a step) their leading term exactly, the rest in float: with d_r = r d_1 + d'_r,
 //          the products r^2 d_1 d_1 / rho are polynomials of degree 2 in r, so
 //          their weighted sum is d_1 d_1 / rho at k = 3 and 0 otherwise (one pair);
 //          what is left is cubic, or carries the small d', and is formed without
-//          cancellation. For cubic terms below 2^-25 and d' d_1 below 2^-23;
+//          cancellation. For cubic terms below 2^-27 and d' d_1 below 2^-25;
 //       2  in pairs.
 //     From the order on at which F^(k-2) is below 2^-28 of the scales the sums
 //     are float too (forms 0 and 1). All leave the measured error unchanged
-//     (0.19-0.22). Each decision is taken per interface, by a vote of its lanes,
-//     and checked against bounds of all Taylor sums at the end.
+//     (0.19-0.22). Each decision is taken per interface (2D: per block), by a vote of
+//     its lanes, against scales of its own nodes, and checked against bounds of all
+//     Taylor sums at the end.
 //
 // What bounds it: instruction issue and the latency of dependent FP32 operations (a
 // pair operation is a chain of 4 to 11), at 14 warps per SM 0.6 instructions per

@@ -712,7 +712,6 @@ struct Smem32 {
   float thi[S][Tiling<P, NW, LPN, R>::TW], tlo[S][Tiling<P, NW, LPN, R>::TW];
   float Gs[Tiling<P, NW, LPN, R>::NI][S];
   unsigned char rej[S][Tiling<P, NW, LPN, R>::NI];  // rejected orders per (component, interface)
-  float redf[NW];
 };
 
 // Block-wide maximum of `v` >= 0 over NW warps (thread 0 returns it).

@@ -1335,7 +1335,8 @@ __global__ void __launch_bounds__(NT) k_smax2d(const Step2DArgs a) {
 //      p_1 = p_2 (serving F and G), else one task per direction with p >= 2
 //      (square blocks S_{p_1}, S_{p_2}); FL-CAT2 directions done in place;
 //   4. for p = 2..P, the tasks of that p in rounds that pack NT / (2p)^2
-//      blocks densely onto the threads, every round in lockstep;
+//      blocks densely onto the threads, every round in lockstep (Euler: first in
+//      float-float pairs, split_tasks; what exceeds them in FP64, block_tasks);
 //   5. the conservative update (Eq. 4.9) and the wave speeds for the next dt.
 // ---------------------------------------------------------------------------
 constexpr int TXH = 12;        // cells per CTA side
