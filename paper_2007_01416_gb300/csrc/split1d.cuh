@@ -373,7 +373,8 @@ __device__ __forceinline__ bool cat_split_euler(const SplitRec<ACAT_FLUX_EULER1D
         q[128] = L1.h;
         q[160] = L1.l;
         // the bounds only grow: a coarse grid leaves for the FP64 sweep before the recursion
-        if (k == 2 && !__all_sync(mask, Ba <= SPLIT_ADJ * rho.h && Bw <= SPLIT_ADJ * rs && Bl <= SPLIT_ADJ * rh))
+        // (at p = 2 the vote cost what it saved)
+        if (p >= 3 && k == 2 && !__all_sync(mask, Ba <= SPLIT_ADJ * rho.h && Bw <= SPLIT_ADJ * rs && Bl <= SPLIT_ADJ * rh))
           return false;
       }
       if (k == 2 && flt) {  // float remainders, by the first-order increments with a margin of 4
