@@ -1675,15 +1675,17 @@ __device__ __forceinline__ void split_tasks(Smem2H<P, FLUX> &sm, const Step2DArg
       Split2Node<p> N;
       FF F[4], G[4], S{0.0f, 0.0f};
       stamp++;
+      bool big = false;
       if (act) {
         const int tx = acat_tile_index(ax + P - p + 1 + ia, TW, a.status);
         const int ty = acat_tile_index(ay + P - p + 1 + ib, TW, a.status);
         if (!split2_start(C, sm.rec[ty * TW + tx], sm.rec[(ay + P) * TW + ax + P], N, F, G)) V.bad = stamp;
-        if (!split2_small(N, F, G)) V.big[0] = stamp;
+        big = form > 0 || !split2_small(N, F, G);
+        if (big) V.big[0] = stamp;
         split2_put(xs, tid, F, G);
       }
-      __syncthreads();
-      bool on = act && V.bad != stamp, tail = form == 0 && V.big[0] != stamp;
+      const bool pairs = __syncthreads_or(big) != 0;  // else every block of the round is in float from k = 2
+      bool on = act && V.bad != stamp, tail = V.big[0] != stamp;
       if (on && node < 8) split2_flux<p>(xs, sm.tab, dir, fc, f0, fs, 840.0f, S);
       N.form = form;
 #pragma unroll 1
@@ -1696,7 +1698,7 @@ __device__ __forceinline__ void split_tasks(Smem2H<P, FLUX> &sm, const Step2DArg
           o = split2_lin(C, N.v, N.w, N.h, u);
           split2_bounds(N, lv, u[0].h, o.W1.h, o.W2.h, o.L.h);
         }
-        if (k == 2) {
+        if (k == 2 && pairs) {
           stamp++;
           if (on && !tail) {
             if (!split2_held(N)) V.bad = stamp;  // the bounds only grow
@@ -1718,8 +1720,13 @@ __device__ __forceinline__ void split_tasks(Smem2H<P, FLUX> &sm, const Step2DArg
           else split2_order(C, N, k, lv, u, o, F, G);
         }
         stamp++;
-        if (on && !split2_small(N, F, G)) V.big[(k & 1) ^ 1] = stamp;  // the other word may still be read
-        if (!__syncthreads_or(on)) break;
+        if (on && !tail && N.form < 2 && !split2_small(N, F, G))
+          V.big[(k & 1) ^ 1] = stamp;  // the other word may still be read
+        if (k == 2) {
+          if (!__syncthreads_or(on)) break;
+        } else {
+          __syncthreads();
+        }
         if (on) split2_put(xs, tid, F, G);
         __syncthreads();
         tail |= N.form < 2 && V.big[(k & 1) ^ 1] != stamp;
